@@ -46,6 +46,7 @@ struct QfConfig {
   int cpt = 1;      // columns per team thread (compile-time variant)
   int grid = 1;     // CTAs
   int rows_per_cta = 1;
+  int rgrid = 0;     // CTAs of the several-rows-a-step kernels (quadform_rows.cu); 0: not used
   int streamed = 0;  // 1: FP32 TMA-streamed kernel (quadform_f32.cu)
   int coop = 0;      // 1: the streamed gradient (pair, FP32) reduces its partials in one cooperative launch
 };
@@ -111,6 +112,35 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s);
 kg_status qf_eval(kg_problem* p, const void* x, void* f, cudaStream_t s);
 kg_status qf_grad(kg_problem* p, const void* x, void* f, void* gx, void* gA, const void* seed,
                   int accumulate, cudaStream_t s);
+
+// Native dense kernels for rows of up to 2048 entries (quadform_rows.cu).
+template <typename T>
+struct QfRowsCall {
+  const T* A;
+  const T* x;
+  int64_t m, n;
+  int grid, team;     // qf_rows_grid's CTAs; the caller's team width (0: by n)
+  const T* seed;
+  T* partials;        // [grid][n]
+  double* fpart;      // [grid]
+  unsigned* counter;  // nullable for the gradient: always a second launch then
+  T* y;               // eval, nullable: row values
+  T* f;
+  T* gx;
+  T* gA;
+  int accumulate;
+};
+bool qf_rows_supported(int64_t n);
+int qf_rows_grid(int dtype, int64_t m, int64_t n, int team);
+template <typename T>
+kg_status qf_rows_eval(const QfRowsCall<T>& c, cudaStream_t s);
+template <typename T>
+kg_status qf_rows_grad(const QfRowsCall<T>& c, cudaStream_t s);
+// Fixed-order sum of `nparts` partial rows of n into gx, and of nf f partials into f
+// (nullable), as a dependent launch (quadform.cu).
+template <typename T>
+kg_status qf_reduce_partials(const T* partials, int nparts, int n, const double* fpart, int nf, T* gx,
+                             T* f, int accumulate, cudaStream_t s);
 
 kg_status qf_native_fused_on_scratch(const double* A, int64_t m, int64_t n, const double* x,
                                      double* f, double* gx, double* scratch,

@@ -217,32 +217,40 @@ __global__ void __launch_bounds__(256) qf_transpose_kernel(const T* __restrict__
   if (j < n) partials[(int64_t)blockIdx.y * n + j] = s;
 }
 
-// Sum of the private partials in a fixed order: thread (cx, py) sums partials
-// py, py+PY, ... of column cx; the PY sums are then added in py order.
-// Block 0 also sums the per-CTA f partials into *f.
+// Sum of the private partials in a fixed order, a dependent launch: a block of 512
+// threads takes 64 bytes of columns, thread (cx, py) sums partials py, py + PY, ... of
+// column cx (eight loads in flight); the lanes of a warp that hold the same column add by
+// a butterfly, then the 16 warps' sums are added in warp order.  Block 0 also sums the
+// per-CTA f partials into *f.  Narrow blocks spread the loads of a short row of partials
+// over the chip: 304 partials of 255 doubles took 7.0 us in 8 blocks of 32 columns.
 template <typename T>
 __global__ void __launch_bounds__(512) qf_reduce_kernel(const T* __restrict__ partials, int nparts,
                                                         int n, const double* __restrict__ fpart,
                                                         int nf, T* gx, T* f, int accumulate) {
-  constexpr int CX = 32, PY = 16;
-  __shared__ T red[PY][CX + 1];
+  constexpr int CX = 64 / (int)sizeof(T), PY = 512 / CX;
+  __shared__ T red[16][CX];
   __shared__ double fred[32];
-  const int cx = threadIdx.x % CX, py = threadIdx.x / CX;
+  grid_dependency_wait();  // the partials are written and visible
+  const int cx = threadIdx.x % CX, py = threadIdx.x / CX, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * CX + cx;
   T s = T(0);
-  if (j < n)
-    for (int c = py; c < nparts; c += PY) s += partials[(int64_t)c * n + j];
-  red[py][cx] = s;
+  if (j < n) {
+#pragma unroll 8
+    for (int c = py; c < nparts; c += PY) s += __ldcg(partials + (int64_t)c * n + j);
+  }
+#pragma unroll
+  for (int o = CX; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) < CX) red[warp][cx] = s;
   __syncthreads();
-  if (py == 0 && j < n) {
+  if (threadIdx.x < CX && j < n) {
     T t = red[0][cx];
 #pragma unroll
-    for (int i = 1; i < PY; ++i) t += red[i][cx];
+    for (int i = 1; i < 16; ++i) t += red[i][cx];
     gx[j] = accumulate ? gx[j] + t : t;
   }
   if (blockIdx.x == 0 && f) {
     double fs = 0.0;
-    for (int i = threadIdx.x; i < nf; i += blockDim.x) fs += fpart[i];
+    for (int i = threadIdx.x; i < nf; i += blockDim.x) fs += __ldcg(fpart + i);
     fs = block_sum(fs, fred);
     if (threadIdx.x == 0) *f = (T)fs;
   }
@@ -250,6 +258,8 @@ __global__ void __launch_bounds__(512) qf_reduce_kernel(const T* __restrict__ pa
 
 // ---------------------------------------------------------------- host ----
 // Variants: (TEAM, CPT_MAX, block).  Team thread count x CPT_MAX bounds n.
+// Rows of up to 2048 entries go to the kernels of quadform_rows.cu; their variants here
+// size the atomic adjoint and say which teams hold a row.
 struct QfVariant {
   int team, cpt_max, block;
 };
@@ -283,7 +293,7 @@ static cudaError_t launch_team(int var, dim3 grid, cudaStream_t s, const QfArgs<
   const size_t smem = qf_smem_bytes<T>(v);
   cudaError_t e = cudaSuccess;
   auto go = [&](auto kern) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = set_smem_once(kern, smem);
     if (e == cudaSuccess) {
       prof_begin(s, MODE == QF_FUSED ? "qf_team_kernel<fused>" : "qf_team_kernel<eval>");
       kern<<<grid, v.block, smem, s>>>(a);
@@ -292,9 +302,6 @@ static cudaError_t launch_team(int var, dim3 grid, cudaStream_t s, const QfArgs<
     }
   };
   switch (var) {
-    case 0: go(qf_team_kernel<T, 32, 4, MODE>); break;
-    case 1: go(qf_team_kernel<T, 128, 8, MODE>); break;
-    case 2: go(qf_team_kernel<T, 256, 8, MODE>); break;
     case 3: go(qf_team_kernel<T, 512, 20, MODE>); break;
     case 4: go(qf_team_kernel<T, 512, 24, MODE>); break;
     default: e = cudaErrorInvalidValue;
@@ -395,11 +402,13 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
   if (p->opt.tile > 0) rows = p->opt.tile;
   c.rows_per_cta = (int)rows;
   c.grid = (int)((p->m + rows - 1) / rows);
-  int fp = std::max(c.grid, transpose_chunks(p));
+  if (qf_rows_supported(p->n))
+    c.rgrid = p->opt.tile > 0 ? c.grid : qf_rows_grid(p->dtype, p->m, p->n, p->opt.team);
+  int fp = std::max({c.grid, c.rgrid, transpose_chunks(p)});
   kg_status rc = ws_common(p, fp, s);
   if (rc != KG_OK) return rc;
   if (p->strategy == KG_STRATEGY_FUSED || p->strategy == KG_STRATEGY_TRANSPOSE) {
-    int parts = p->strategy == KG_STRATEGY_FUSED ? c.grid : transpose_chunks(p);
+    int parts = p->strategy != KG_STRATEGY_FUSED ? transpose_chunks(p) : c.rgrid ? c.rgrid : c.grid;
     rc = ws_alloc(p, &p->partials, p->esize * (size_t)parts * p->n, "xbar partials");
     if (rc != KG_OK) return rc;
   }
@@ -427,7 +436,51 @@ static QfArgs<T> make_args(kg_problem* p, const void* x, const void* seed) {
 }
 
 template <typename T>
+static QfRowsCall<T> rows_call(kg_problem* p, const void* x, void* f) {
+  QfRowsCall<T> r{};
+  r.A = static_cast<const T*>(p->data0);
+  r.x = static_cast<const T*>(x);
+  r.m = p->m;
+  r.n = p->n;
+  r.grid = p->qf.rgrid;
+  r.team = p->opt.team;
+  r.partials = static_cast<T*>(p->partials);
+  r.fpart = p->fpart;
+  r.counter = p->counter;
+  r.f = static_cast<T*>(f);
+  return r;
+}
+
+template <typename T>
+kg_status qf_reduce_partials(const T* partials, int nparts, int n, const double* fpart, int nf, T* gx,
+                             T* f, int accumulate, cudaStream_t s) {
+  constexpr int CX = 64 / (int)sizeof(T);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((n + CX - 1) / CX);
+  cfg.blockDim = dim3(512);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, qf_reduce_kernel<T>, partials, nparts, n, fpart, nf, gx, f,
+                                     accumulate);
+  count_launch();
+  return e == cudaSuccess ? KG_OK : cuda_fail(e, "qf reduce kernel");
+}
+template kg_status qf_reduce_partials<double>(const double*, int, int, const double*, int, double*, double*,
+                                              int, cudaStream_t);
+template kg_status qf_reduce_partials<float>(const float*, int, int, const double*, int, float*, float*, int,
+                                             cudaStream_t);
+
+template <typename T>
 static kg_status qf_eval_t(kg_problem* p, const void* x, void* f, T* y, cudaStream_t s) {
+  if (p->qf.rgrid) {
+    QfRowsCall<T> r = rows_call<T>(p, x, f);
+    r.y = y;
+    return qf_rows_eval(r, s);
+  }
   QfArgs<T> a = make_args<T>(p, x, nullptr);
   a.f = static_cast<T*>(f);
   a.y = y;
@@ -451,17 +504,21 @@ static kg_status qf_grad_t(kg_problem* p, const void* x, void* f, void* gx, void
   const int n = (int)p->n;
   cudaError_t e;
   if (p->strategy == KG_STRATEGY_FUSED) {
+    if (p->qf.rgrid) {
+      QfRowsCall<T> r = rows_call<T>(p, x, f);
+      r.seed = static_cast<const T*>(seed);
+      r.gx = static_cast<T*>(gx);
+      r.gA = static_cast<T*>(gA);
+      r.accumulate = accumulate;
+      return qf_rows_grad(r, s);
+    }
     QfArgs<T> a = make_args<T>(p, x, seed);
     a.gA = static_cast<T*>(gA);
     a.accumulate = accumulate;
     e = launch_team<T, QF_FUSED>(var, dim3(p->qf.grid), s, a);
     if (e != cudaSuccess) return cuda_fail(e, "qf fused kernel");
-    qf_reduce_kernel<T><<<(n + 31) / 32, 512, 0, s>>>(static_cast<const T*>(p->partials), p->qf.grid,
-                                                      n, p->fpart, p->qf.grid, static_cast<T*>(gx),
-                                                      static_cast<T*>(f), accumulate);
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "qf reduce kernel");
-    return KG_OK;
+    return qf_reduce_partials<T>(static_cast<const T*>(p->partials), p->qf.grid, n, p->fpart, p->qf.grid,
+                                 static_cast<T*>(gx), static_cast<T*>(f), accumulate, s);
   }
   if (gA) return fail(KG_ERR_UNSUPPORTED, "QUADFORM: gradient w.r.t. A needs the FUSED strategy");
   // forward with y stored (f written by the last CTA)
@@ -490,12 +547,8 @@ static kg_status qf_grad_t(kg_problem* p, const void* x, void* f, void* gx, void
   prof_end(s);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "qf transpose kernel");
-  qf_reduce_kernel<T><<<(n + 31) / 32, 512, 0, s>>>(static_cast<const T*>(p->partials), used, n,
-                                                    p->fpart, 0, static_cast<T*>(gx), nullptr,
-                                                    accumulate);
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "qf reduce kernel");
-  return KG_OK;
+  return qf_reduce_partials<T>(static_cast<const T*>(p->partials), used, n, p->fpart, 0,
+                               static_cast<T*>(gx), nullptr, accumulate, s);
 }
 
 // Native FP64 fused value-and-gradient with every workspace taken from
@@ -509,14 +562,27 @@ kg_status qf_native_fused_on_scratch(const double* A, int64_t m, int64_t n, cons
                                      size_t scratch_doubles, cudaStream_t s) {
   const int var = pick_variant(n, 0);
   if (var < 0) return fail(KG_ERR_INVALID_ARG, "n must be <= 12288");
-  const QfVariant& v = kVariants[var];
-  const int nteams = v.block / v.team;
-  const int resident = v.block >= 512 ? 1 : 2;
-  const int64_t target = (int64_t)num_sms() * resident;
   const int64_t max_grid = (int64_t)(scratch_doubles / ((size_t)n + 1));
   if (max_grid < 1)
     return fail(KG_ERR_INVALID_ARG, "scratch of " + std::to_string(scratch_doubles) +
                                         " doubles is too small for n = " + std::to_string(n));
+  if (qf_rows_supported(n)) {
+    QfRowsCall<double> r{};  // no arrival counter: more than one CTA's partials in a second launch
+    r.A = A;
+    r.x = x;
+    r.m = m;
+    r.n = n;
+    r.grid = (int)std::min<int64_t>(qf_rows_grid(KG_F64, m, n, 0), max_grid);
+    r.partials = scratch;
+    r.fpart = scratch + (size_t)r.grid * n;
+    r.f = f;
+    r.gx = gx;
+    return qf_rows_grad(r, s);
+  }
+  const QfVariant& v = kVariants[var];
+  const int nteams = v.block / v.team;
+  const int resident = v.block >= 512 ? 1 : 2;
+  const int64_t target = (int64_t)num_sms() * resident;
   const int64_t rows = std::max<int64_t>({(int64_t)nteams, (m + target - 1) / target,
                                           (m + max_grid - 1) / max_grid});
   const int grid = (int)((m + rows - 1) / rows);
@@ -536,11 +602,7 @@ kg_status qf_native_fused_on_scratch(const double* A, int64_t m, int64_t n, cons
   a.fpart = scratch + (size_t)grid * n;
   cudaError_t e = launch_team<double, QF_FUSED>(var, dim3(grid), s, a);
   if (e != cudaSuccess) return cuda_fail(e, "qf fused kernel");
-  qf_reduce_kernel<double><<<(int)((n + 31) / 32), 512, 0, s>>>(scratch, grid, (int)n, a.fpart, grid,
-                                                               gx, f, 0);
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "qf reduce kernel");
-  return KG_OK;
+  return qf_reduce_partials<double>(scratch, grid, (int)n, a.fpart, grid, gx, f, 0, s);
 }
 
 kg_status qf_grad(kg_problem* p, const void* x, void* f, void* gx, void* gA, const void* seed,
