@@ -13,13 +13,15 @@
 //                partial of the tile written to the instance's partial buffer;
 //                on float-pair copies (pair batches) the rows arrive by bulk
 //                copies into a shared-memory ring, otherwise by plain loads;
+//                pair arithmetic runs on packed column pairs (kg_pair2.cuh);
 //   tet tile:    elements [e0, e0 + T): f_e and the scatter of c_e into gu (zeroed
 //                by a small kernel earlier in the graph): one global reduction per
 //                contribution, or warp-combined first with the WARP strategy.
-// The CTA that finishes an instance's last tile (a per-instance arrival
-// counter; nobody waits) sums the instance's partials in tile order into gx
-// and f, and resets the counter.  The last CTA to leave resets the queue head,
-// so the graph can be replayed as is.
+// A dense instance of few tiles is summed into gx and f by the CTA that finishes
+// its last tile (a per-instance arrival counter); one of more than B_SUM_TILES
+// tiles by sum items of 256 columns at the end of the table, which wait for that
+// counter.  The last CTA to leave resets the queue head, so the graph can be
+// replayed as is.
 //
 // Tile sizes R and T are chosen per (kind, size bucket) by an autotuner that
 // times candidates on the instances of the batch at kg_batch_create and keeps
@@ -37,6 +39,7 @@
 #include <new>
 #include <sstream>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include <sys/stat.h>
@@ -44,6 +47,7 @@
 #include "kg_device.cuh"
 #include "kg_internal.h"
 #include "kg_pair.cuh"
+#include "kg_pair2.cuh"
 #include "kg_tet_elem.cuh"
 
 namespace kg {
@@ -59,18 +63,22 @@ struct BInst {
   int n;      // dense: columns; tet: vertices
   int64_t m;  // dense: rows; tet: elements
   int ntiles;
-  int team;   // dense: 32 or 256
+  int team;   // dense: threads of a row team
+  int pitch;  // dense, pair batches: n rounded up to even: entries of a copy's or a partial's row
   int prep;   // pair batches: d0 (dense A) or d1 (tet G) is the prepared float-pair copy
   const void* d0;
   const void* d1;
   const void* x;
   void* f;
   void* gx;
-  void* partials;  // dense: [ntiles][n]  (pair: Acc; native: T)
+  void* partials;  // dense: [ntiles][n] of T, or (pair) [ntiles][pitch] of Acc
   double* fpart;   // [ntiles]
-  unsigned* done;
+  unsigned* done;  // [0] tiles done, [1] sum items done
+  int nsum;        // dense: items that sum the partials (0: the last tile's CTA does)
 };
 
+// Rows (dense) or elements (tet) [start, start + count) of tile `tile`; or, tile < 0, a sum
+// item: columns [start, start + count) of a dense instance's gradient.
 struct BItem {
   int inst, tile;
   int64_t start;
@@ -100,19 +108,6 @@ __device__ __forceinline__ void prefetch_range_l2(const void* p, size_t bytes) {
   }
 }
 
-// The float pair (h, l) of v for pair arithmetic (zeros otherwise).
-template <bool PAIR, typename T>
-__device__ __forceinline__ void b_split(T v, float& h, float& l) {
-  if constexpr (PAIR) {
-    const Pair p = split_f64((double)v);
-    h = p.h;
-    l = p.l;
-  } else {
-    h = 0.f;
-    l = 0.f;
-  }
-}
-
 // Barrier over the TEAM threads of one row team: the whole CTA for TEAM = BT,
 // otherwise hardware barrier 1 + team (TEAM = 64 or 128).
 template <int TEAM>
@@ -133,11 +128,10 @@ __device__ __forceinline__ Acc team_warps_sum(const Acc* ra, int lane, bool uppe
   return k;
 }
 
-// Rows [w.start, w.start + w.count) of a dense instance on its FP64 or FP32
-// data (pair batches: split on every load); returns the tile's f.
-template <typename T, bool PAIR, int TEAM>
-__device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp, double* red,
-                             bool& bad) {
+// Rows [w.start, w.start + w.count) of a dense instance in native arithmetic;
+// returns the tile's f.
+template <typename T, int TEAM>
+__device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp, double* red) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = I.n;
   const T* __restrict__ A = static_cast<const T*>(I.d0);
@@ -145,387 +139,200 @@ __device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp,
   constexpr int NT = BT / TEAM;
   const int lt = tid % TEAM, team = tid / TEAM;
   const int cpt = (n + TEAM - 1) / TEAM;  // <= B_CPT, uniform over the item
-  float xh[B_CPT], xl[B_CPT];
-  T xv[B_CPT];
-  Acc xbp[B_CPT];
-  T xbn[B_CPT];
+  T xv[B_CPT], xbn[B_CPT];
 #pragma unroll
   for (int k = 0; k < B_CPT; ++k) {
     const int j = lt + k * TEAM;
     xv[k] = (k < cpt && j < n) ? x[j] : T(0);
-    if constexpr (PAIR) {
-      bad |= !pair_in_range((double)xv[k]);
-      b_split<PAIR>(xv[k], xh[k], xl[k]);
-    }
-    xbp[k] = acc_zero();
     xbn[k] = T(0);
   }
-  Acc fp = acc_zero();
   FSum<T> fn;
   const int64_t r1 = w.start + w.count;
-  if constexpr (PAIR) {
-    // Two rows per team and iteration, rows r and r + NT: their loads are issued
-    // together, and one transposed butterfly reduces both dot products (the
-    // first exchange hands each half of the team one row), so the reduction
-    // and, for teams wider than a warp, the barrier are paid once per two rows.
-    constexpr int W = TEAM < 32 ? TEAM : 32;  // lanes of the team inside one warp
-    const bool upper = (lane & (W / 2)) != 0;  // keeps the second row
-    const int iters2 = (w.count + 2 * NT - 1) / (2 * NT);
-    for (int itr = 0; itr < iters2; ++itr) {
-      const int64_t rr[2] = {w.start + (int64_t)itr * 2 * NT + team,
-                             w.start + (int64_t)itr * 2 * NT + NT + team};
-      const bool vr[2] = {rr[0] < r1, rr[1] < r1};
-      float ah[2][B_CPT], al[2][B_CPT];
+  const int iters = (w.count + NT - 1) / NT;
+  // software pipeline: the next row's loads are in flight while this row computes
+  T an[B_CPT];
+  auto load_row = [&](int itr_, T* dst) {
+    const int64_t r = w.start + (int64_t)itr_ * NT + team;
+    const bool v = itr_ < iters && r < r1;
+    const T* Ar = A + (v ? r : w.start) * (int64_t)n;
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const T* Ar = A + (vr[q] ? rr[q] : w.start) * (int64_t)n;
-#pragma unroll
-        for (int k = 0; k < B_CPT; ++k) {
-          const int j = lt + k * TEAM;
-          const T v = (k < cpt && vr[q] && j < n) ? __ldcs(Ar + j) : T(0);
-          b_split<PAIR, T>(v, ah[q][k], al[q][k]);
-        }
-      }
-      Acc y[2] = {acc_zero(), acc_zero()};
-#pragma unroll
-      for (int k = 0; k < B_CPT; ++k) {
-        if (k < cpt) {
-          acc_fma(y[0], ah[0][k], al[0][k], xh[k], xl[k]);
-          acc_fma(y[1], ah[1][k], al[1][k], xh[k], xl[k]);
-        }
-      }
-      Acc keep = upper ? y[1] : y[0];
-      keep = acc_add(keep, shfl_xor_acc2(upper ? y[0] : y[1], W / 2));
-#pragma unroll
-      for (int o = W / 4; o > 0; o >>= 1) keep = acc_add(keep, shfl_xor_acc2(keep, o));
-      if constexpr (TEAM > 32) {  // warps of the team exchange through shared memory
-        constexpr int TW = TEAM / 32;
-        Acc* ra = reinterpret_cast<Acc*>(red) + (itr & 1) * 2 * BW + team * 2 * TW;  // [TW][2]
-        if ((lane & (W / 2 - 1)) == 0) ra[(warp % TW) * 2 + (upper ? 1 : 0)] = keep;
-        team_barrier<TEAM>(team);
-        keep = team_warps_sum<TW>(ra, lane, upper);
-      }
-      const Acc other = shfl_xor_acc2(keep, W / 2);
-      const Acc yt[2] = {upper ? other : keep, upper ? keep : other};
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        if (vr[q]) {
-          const Pair yq = acc_pair(yt[q]);
-          const Pair y2 = pair_mul(yq, yq);
-          fp = acc_add(fp, Acc{y2.h, y2.l});
-          const Pair yb{2.0f * yq.h, 2.0f * yq.l};  // exact
-#pragma unroll
-          for (int k = 0; k < B_CPT; ++k)
-            if (k < cpt) acc_fma(xbp[k], ah[q][k], al[q][k], yb.h, yb.l);
-        }
-      }
-      if ((itr & 7) == 7) {
-#pragma unroll
-        for (int k = 0; k < B_CPT; ++k) acc_renorm(xbp[k]);
-      }
+    for (int k = 0; k < B_CPT; ++k) {
+      const int j = lt + k * TEAM;
+      dst[k] = (k < cpt && v && j < n) ? __ldcs(Ar + j) : T(0);
     }
-  } else {
-    const int iters = (w.count + NT - 1) / NT;
-    // software pipeline: the next row's loads are in flight while this row computes
-    T an[B_CPT];
-    auto load_row = [&](int itr_, T* dst) {
-      const int64_t r = w.start + (int64_t)itr_ * NT + team;
-      const bool v = itr_ < iters && r < r1;
-      const T* Ar = A + (v ? r : w.start) * (int64_t)n;
+  };
+  load_row(0, an);
+  for (int itr = 0; itr < iters; ++itr) {
+    const int64_t r = w.start + (int64_t)itr * NT + team;
+    const bool valid = r < r1;
+    T av[B_CPT];
 #pragma unroll
-      for (int k = 0; k < B_CPT; ++k) {
-        const int j = lt + k * TEAM;
-        dst[k] = (k < cpt && v && j < n) ? __ldcs(Ar + j) : T(0);
+    for (int k = 0; k < B_CPT; ++k) av[k] = an[k];
+    load_row(itr + 1, an);
+    {
+      T d = T(0);
+#pragma unroll
+      for (int k = 0; k < B_CPT; ++k)
+        if (k < cpt) d = fma(av[k], xv[k], d);
+#pragma unroll
+      for (int o = (TEAM < 32 ? TEAM : 32) / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+      if constexpr (TEAM > 32) {
+        constexpr int TW = TEAM / 32;
+        T* rt = reinterpret_cast<T*>(red) + (itr & 1) * BW + team * TW;
+        if (lane == 0) rt[warp % TW] = d;
+        team_barrier<TEAM>(team);
+        d = rt[0];
+#pragma unroll
+        for (int q = 1; q < TW; ++q) d += rt[q];
       }
-    };
-    load_row(0, an);
-    for (int itr = 0; itr < iters; ++itr) {
-      const int64_t r = w.start + (int64_t)itr * NT + team;
-      const bool valid = r < r1;
-      T av[B_CPT];
-#pragma unroll
-      for (int k = 0; k < B_CPT; ++k) av[k] = an[k];
-      load_row(itr + 1, an);
-      {
-        T d = T(0);
+      if (valid) {
+        fn.add(d);
+        const T yb = T(2) * d;
 #pragma unroll
         for (int k = 0; k < B_CPT; ++k)
-          if (k < cpt) d = fma(av[k], xv[k], d);
-#pragma unroll
-        for (int o = (TEAM < 32 ? TEAM : 32) / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if constexpr (TEAM > 32) {
-          constexpr int TW = TEAM / 32;
-          T* rt = reinterpret_cast<T*>(red) + (itr & 1) * BW + team * TW;
-          if (lane == 0) rt[warp % TW] = d;
-          team_barrier<TEAM>(team);
-          d = rt[0];
-#pragma unroll
-          for (int q = 1; q < TW; ++q) d += rt[q];
-        }
-        if (valid) {
-          fn.add(d);
-          const T yb = T(2) * d;
-#pragma unroll
-          for (int k = 0; k < B_CPT; ++k)
-            if (k < cpt) xbn[k] = fma(yb, av[k], xbn[k]);
-        }
+          if (k < cpt) xbn[k] = fma(yb, av[k], xbn[k]);
       }
     }
   }
   // combine the teams' partials in team order and store the tile's partial
   __syncthreads();
-  if constexpr (PAIR) {
-    Acc* out = static_cast<Acc*>(I.partials) + (int64_t)w.tile * n;
-    if constexpr (NT == 1) {
-#pragma unroll
-      for (int k = 0; k < B_CPT; ++k) {
-        const int j = lt + k * TEAM;
-        if (j < n) out[j] = xbp[k];
-      }
-    } else {
-      Acc* ws = reinterpret_cast<Acc*>(wsp);  // [NT][TEAM * B_CPT]
-#pragma unroll
-      for (int k = 0; k < B_CPT; ++k) ws[team * TEAM * B_CPT + lt + k * TEAM] = xbp[k];
-      __syncthreads();
-      for (int j = tid; j < n; j += BT) {
-        Acc s = ws[j];
-        for (int t2 = 1; t2 < NT; ++t2) s = acc_add(s, ws[t2 * TEAM * B_CPT + j]);
-        out[j] = s;
-      }
-    }
-    // in a pair batch wsp lies in the ring: order these generic accesses before
-    // the copies that will land there
-    fence_proxy_async_smem();
-    // f of the tile: team leaders in team order
-    Acc* ra = reinterpret_cast<Acc*>(red);
-    __syncthreads();
-    if (lt == 0) ra[team] = fp;
-    __syncthreads();
-    Acc tot = ra[0];
-    for (int t2 = 1; t2 < NT; ++t2) tot = acc_add(tot, ra[t2]);
-    __syncthreads();
-    return acc_to_double(tot);
-  } else {
-    T* out = static_cast<T*>(I.partials) + (int64_t)w.tile * n;
-    if constexpr (NT == 1) {
-#pragma unroll
-      for (int k = 0; k < B_CPT; ++k) {
-        const int j = lt + k * TEAM;
-        if (j < n) out[j] = xbn[k];
-      }
-    } else {
-      T* ws = reinterpret_cast<T*>(wsp);
-#pragma unroll
-      for (int k = 0; k < B_CPT; ++k) ws[team * TEAM * B_CPT + lt + k * TEAM] = xbn[k];
-      __syncthreads();
-      for (int j = tid; j < n; j += BT) {
-        T s = ws[j];
-        for (int t2 = 1; t2 < NT; ++t2) s += ws[t2 * TEAM * B_CPT + j];
-        out[j] = s;
-      }
-    }
-    __syncthreads();
-    if (lt == 0) red[team] = fn.get();
-    __syncthreads();
-    double tot = 0.0;
-    for (int t2 = 0; t2 < NT; ++t2) tot += red[t2];
-    __syncthreads();
-    return tot;
-  }
-}
-
-// ---- dense tiles of pair batches on float-pair copies: rows staged by bulk copies ----
-// A tile's rows are contiguous, so its data arrives by 1-D bulk copies (TMA)
-// into a ring of RING_S shared-memory slots, one iteration group (the 2 NT rows
-// one iteration of the teams takes, at most 32 KB: about B_CPT columns per
-// team thread) a slot, while the teams compute on the slot before: bytes in
-// flight without registers.  A copy covers the 16-byte aligned span around its
-// rows (a row starts 8 bytes off the boundary when n is odd; those copies are
-// the batch's own, allocated 16 bytes longer), and the rows sit `off` bytes into
-// the slot.  All threads count the chunks the CTA has consumed (g), which
-// gives each slot's barrier phase across tiles; thread 0, the only one that
-// issues, counts the chunks issued (iss).  When a tile has no chunk left to
-// issue, the slots it frees take the first chunks of the CTA's next item
-// (claimed when this one started) if that is a ring tile too, so the copies
-// run on across the tile boundary.
-constexpr int RING_S = 3;
-constexpr int RING_SLOT = 32768 + 128;
-
-struct Ring {
-  unsigned char* slots;  // RING_S * RING_SLOT bytes
-  uint64_t* full;        // RING_S barriers: a slot's copy has landed
-};
-
-// The CTA's next item as ring chunks (thread 0 only); nchunks 0: not a ring tile.
-struct RingNext {
-  const double* src;   // its first row
-  int64_t chunk;       // entries a chunk (2 NT n)
-  int64_t total;       // entries of the item (count n)
-  int nchunks;
-};
-
-constexpr int RING_WS = 1024;  // Acc entries of the team combine's buffer (8 KB)
-
-__device__ __forceinline__ uint32_t ring_issue(const Ring& R, uint32_t g, const void* src, size_t bytes) {
-  const uintptr_t lo = reinterpret_cast<uintptr_t>(src) & ~uintptr_t(15);
-  const uintptr_t hi = (reinterpret_cast<uintptr_t>(src) + bytes + 15) & ~uintptr_t(15);
-  const int slot = (int)(g % RING_S);
-  mbar_arrive_expect_tx(&R.full[slot], (uint32_t)(hi - lo));
-  tma_load_1d(R.slots + slot * RING_SLOT, reinterpret_cast<const void*>(lo), (uint32_t)(hi - lo),
-              &R.full[slot]);
-  return (uint32_t)(reinterpret_cast<uintptr_t>(src) - lo);
-}
-
-// The dense_tile pair path on a prepared copy, reading its rows from the ring.
-// Returns the tile's f; sets `failed` (on all threads) when a copy did not land
-// within the wait limit, after waiting for the CTA's other copies in flight.
-// CPT > 0: the columns per team thread, ceil(n / TEAM), fixed at compile time
-// (no per-column tests but the last column's j < n); 0: at run time.
-template <int TEAM, int CPT>
-__device__ double dense_tile_ring(const BInst& I, const BItem& w, const Ring& R, uint32_t& g,
-                                  uint32_t& iss, const RingNext& nx, unsigned char* wsp, double* red,
-                                  bool& bad, bool& failed) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = I.n;
-  const double* __restrict__ A = static_cast<const double*>(I.d0);  // float pairs, 8 bytes an entry
-  const double* __restrict__ x = static_cast<const double*>(I.x);
-  constexpr int NT = BT / TEAM;
-  constexpr int W = TEAM < 32 ? TEAM : 32;  // lanes of the team inside one warp
-  const int lt = tid % TEAM, team = tid / TEAM;
-  constexpr int KM = CPT ? CPT : B_CPT;
-  const int cpt = CPT ? CPT : (n + TEAM - 1) / TEAM;
-  // column k of this thread is in the row: compile-time true below the last one
-  auto col_in = [&](int k, int j) { return (CPT && k < CPT - 1) || (k < cpt && j < n); };
-  float xh[KM], xl[KM];
-  Acc xbp[KM];
-#pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    const int j = lt + k * TEAM;
-    const double xv = col_in(k, j) ? x[j] : 0.0;
-    bad |= !pair_in_range(xv);
-    b_split<true>(xv, xh[k], xl[k]);
-    xbp[k] = acc_zero();
-  }
-  Acc fp = acc_zero();
-  const int64_t r1 = w.start + w.count;
-  const int nchunks = (w.count + 2 * NT - 1) / (2 * NT);
-  auto chunk_src = [&](int c) { return A + (w.start + (int64_t)c * 2 * NT) * n; };
-  auto chunk_bytes = [&](int c) {
-    const int64_t left = r1 - (w.start + (int64_t)c * 2 * NT);
-    return (size_t)(left < 2 * NT ? left : 2 * NT) * n * 8;
-  };
-  const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(chunk_src(0)) & 15u);
-  // chunk row starts are n * 16 bytes apart: every chunk has the same offset
-  const uint32_t g0 = g;  // this tile's chunk c is the CTA's chunk g0 + c
-  if (tid == 0)  // (the first ones may have been issued by the tile before)
-    for (; (int)(iss - g0) < nchunks && iss - g0 < (uint32_t)RING_S; ++iss)
-      ring_issue(R, iss, chunk_src((int)(iss - g0)), chunk_bytes((int)(iss - g0)));
-  const bool upper = (lane & (W / 2)) != 0;  // keeps the second row
-  for (int c = 0; c < nchunks; ++c) {
-    const int slot = (int)(g % RING_S);
-    const bool ok = mbar_wait_bounded(&R.full[slot], (g / RING_S) & 1u);
-    const unsigned char* buf = R.slots + slot * RING_SLOT + off;
-    const int64_t row0 = w.start + (int64_t)c * 2 * NT;
-    const int64_t rr[2] = {row0 + team, row0 + NT + team};
-    const bool vr[2] = {ok && rr[0] < r1, ok && rr[1] < r1};
-    float ah[2][KM], al[2][KM];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const float2* Ar = reinterpret_cast<const float2*>(buf) + (int64_t)(q * NT + team) * n;
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        const int j = lt + k * TEAM;
-        const float2 v = (vr[q] && col_in(k, j)) ? Ar[j] : make_float2(0.f, 0.f);
-        ah[q][k] = v.x;
-        al[q][k] = v.y;
-      }
-    }
-    Acc y[2] = {acc_zero(), acc_zero()};
-#pragma unroll
-    for (int k = 0; k < KM; ++k) {
-      if (CPT || k < cpt) {
-        acc_fma(y[0], ah[0][k], al[0][k], xh[k], xl[k]);
-        acc_fma(y[1], ah[1][k], al[1][k], xh[k], xl[k]);
-      }
-    }
-    Acc keep = upper ? y[1] : y[0];
-    keep = acc_add(keep, shfl_xor_acc2(upper ? y[0] : y[1], W / 2));
-#pragma unroll
-    for (int o = W / 4; o > 0; o >>= 1) keep = acc_add(keep, shfl_xor_acc2(keep, o));
-    // teams wider than a warp exchange their warps' sums through shared memory
-    // (two buffers: chunk c + 1 writes the other while chunk c's are read)
-    constexpr int TW = TEAM > 32 ? TEAM / 32 : 1;
-    Acc* ra = reinterpret_cast<Acc*>(red) + (c & 1) * 2 * BW + team * 2 * TW;  // [TW][2]
-    if constexpr (TEAM > 32)
-      if ((lane & (W / 2 - 1)) == 0) ra[(warp % TW) * 2 + (upper ? 1 : 0)] = keep;
-    // one CTA barrier a chunk: the slot's entries are in registers now, so the
-    // slot is refilled here; it also publishes the warps' sums
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0)  // do not go on with a copy into this CTA's shared memory in flight
-        for (uint32_t h = g; h < iss; ++h) mbar_wait_bounded(&R.full[h % RING_S], (h / RING_S) & 1u);
-      failed = true;
-      __syncthreads();
-      return 0.0;
-    }
-    if (tid == 0 && iss - g0 < (uint32_t)(nchunks + nx.nchunks)) {
-      const int k = (int)(iss - g0);
-      if (k < nchunks) {
-        ring_issue(R, iss, chunk_src(k), chunk_bytes(k));
-      } else {  // the next item's chunk k - nchunks
-        const int64_t e0 = (int64_t)(k - nchunks) * nx.chunk, left = nx.total - e0;
-        ring_issue(R, iss, nx.src + e0, (size_t)(left < nx.chunk ? left : nx.chunk) * 8);
-      }
-      ++iss;
-    }
-    ++g;
-    if constexpr (TEAM > 32) {
-      keep = team_warps_sum<TW>(ra, lane, upper);
-    }
-    const Acc other = shfl_xor_acc2(keep, W / 2);
-    const Acc yt[2] = {upper ? other : keep, upper ? keep : other};
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (vr[q]) {
-        const Pair yq = acc_pair(yt[q]);
-        const Pair y2 = pair_mul(yq, yq);
-        fp = acc_add(fp, Acc{y2.h, y2.l});
-        const Pair yb{2.0f * yq.h, 2.0f * yq.l};  // exact
-#pragma unroll
-        for (int k = 0; k < KM; ++k)
-          if (CPT || k < cpt) acc_fma(xbp[k], ah[q][k], al[q][k], yb.h, yb.l);
-      }
-    }
-    if ((c & 7) == 7) {
-#pragma unroll
-      for (int k = 0; k < KM; ++k) acc_renorm(xbp[k]);
-    }
-  }
-  // combine the teams' partials in team order and store the tile's partial, in
-  // two halves of the columns through RING_WS entries (outside the ring, into
-  // which the next item's copies may be landing)
-  Acc* out = static_cast<Acc*>(I.partials) + (int64_t)w.tile * n;
+  T* out = static_cast<T*>(I.partials) + (int64_t)w.tile * n;
   if constexpr (NT == 1) {
 #pragma unroll
-    for (int k = 0; k < KM; ++k) {
+    for (int k = 0; k < B_CPT; ++k) {
       const int j = lt + k * TEAM;
-      if (j < n) out[j] = xbp[k];
+      if (j < n) out[j] = xbn[k];
     }
   } else {
-    constexpr int H = B_CPT / 2;
-    static_assert(BT * H <= RING_WS, "the combine buffer holds half the columns of all teams");
-    Acc* ws = reinterpret_cast<Acc*>(wsp);  // [NT][TEAM * H]
+    T* ws = reinterpret_cast<T*>(wsp);
+#pragma unroll
+    for (int k = 0; k < B_CPT; ++k) ws[team * TEAM * B_CPT + lt + k * TEAM] = xbn[k];
+    __syncthreads();
+    for (int j = tid; j < n; j += BT) {
+      T s = ws[j];
+      for (int t2 = 1; t2 < NT; ++t2) s += ws[t2 * TEAM * B_CPT + j];
+      out[j] = s;
+    }
+  }
+  __syncthreads();
+  if (lt == 0) red[team] = fn.get();
+  __syncthreads();
+  double tot = 0.0;
+  for (int t2 = 0; t2 < NT; ++t2) tot += red[t2];
+  __syncthreads();
+  return tot;
+}
+
+// ---- dense tiles of pair batches: two rows per team and step, columns in packed pairs ----
+// Team thread lt holds the column pairs jp = lt + k TEAM, k < KM (odd n: the last
+// pair's second column is a zero).  Rows r and r + NT of a step are reduced
+// together: one transposed butterfly for both dot products (the first exchange
+// hands each half of the team one row), so the reduction and, for teams wider
+// than a warp, the barrier are paid once per two rows.  `sync` runs between the
+// warps' sums and their use; it is the barrier of teams wider than a warp, and
+// true from it (on all threads) ends the tile.
+template <int TEAM, int KM, typename Sync>
+__device__ __forceinline__ bool pair_two_rows(const Pair2 (&av)[2][KM], int kp, const Pair2 (&xp)[KM],
+                                              Acc2 (&xb)[KM], Acc& fp, const bool (&vr)[2], double* red,
+                                              int par, const Sync& sync) {
+  constexpr int W = TEAM < 32 ? TEAM : 32;  // lanes of the team inside one warp
+  constexpr int TW = TEAM > 32 ? TEAM / 32 : 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = threadIdx.x / TEAM;
+  const bool upper = (lane & (W / 2)) != 0;  // keeps the second row
+  Acc2 y2[2] = {acc2_prod(av[0][0], xp[0]), acc2_prod(av[1][0], xp[0])};
+#pragma unroll
+  for (int k = 1; k < KM; ++k) {
+    if (k < kp) {
+      acc2_fma(y2[0], av[0][k], xp[k]);
+      acc2_fma(y2[1], av[1][k], xp[k]);
+    }
+  }
+  const Acc y[2] = {acc2_sum(y2[0]), acc2_sum(y2[1])};
+  Acc keep = upper ? y[1] : y[0];
+  keep = acc_add(keep, shfl_xor_acc2(upper ? y[0] : y[1], W / 2));
+#pragma unroll
+  for (int o = W / 4; o > 0; o >>= 1) keep = acc_add(keep, shfl_xor_acc2(keep, o));
+  // two buffers: step c + 1 writes the other while step c's sums are read
+  Acc* ra = reinterpret_cast<Acc*>(red) + par * 2 * BW + team * 2 * TW;  // [TW][2]
+  if constexpr (TEAM > 32)
+    if ((lane & (W / 2 - 1)) == 0) ra[(warp % TW) * 2 + (upper ? 1 : 0)] = keep;
+  if (sync()) return true;
+  if constexpr (TEAM > 32) keep = team_warps_sum<TW>(ra, lane, upper);
+  const Acc other = shfl_xor_acc2(keep, W / 2);
+  const Acc yt[2] = {upper ? other : keep, upper ? keep : other};
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (vr[q]) {
+      const Pair yq = acc_pair(yt[q]);
+      if (TEAM <= 32 || warp % TW == 0) {  // f: the team's first warp
+        const Pair y2q = pair_mul(yq, yq);
+        fp = acc_add(fp, Acc{y2q.h, y2q.l});
+      }
+      const Pair2 yb = pair2_dup(Pair{2.0f * yq.h, 2.0f * yq.l});  // exact
+#pragma unroll
+      for (int k = 0; k < KM; ++k)
+        if (k < kp) acc2_fma(xb[k], av[q][k], yb);
+    }
+  }
+  return false;
+}
+
+// x in float pairs for the thread's column pairs.
+template <int TEAM, int KM>
+__device__ __forceinline__ void pair_load_x(const BInst& I, Pair2 (&xp)[KM], Acc2 (&xb)[KM], bool& bad) {
+  const double* __restrict__ x = static_cast<const double*>(I.x);
+  const int lt = threadIdx.x % TEAM;
+#pragma unroll
+  for (int k = 0; k < KM; ++k) {
+    const int j = 2 * (lt + k * TEAM);
+    const double x0 = j < I.n ? x[j] : 0.0, x1 = j + 1 < I.n ? x[j + 1] : 0.0;
+    bad |= !pair_in_range(x0) || !pair_in_range(x1);
+    xp[k] = pair2_of(split_f64(x0), split_f64(x1));
+    xb[k] = acc2_zero();
+  }
+}
+
+// The end of a pair tile: the teams' partials combined in team order, two column
+// pairs of every thread at a time through RING_WS entries (outside the ring, into
+// which the next item's copies may be landing), and the tile's f.
+constexpr int RING_WS = 1024;  // Acc entries of the combine buffer (8 KB)
+
+template <int TEAM, int KM>
+__device__ double pair_tile_end(const BInst& I, const BItem& w, const Acc2 (&xb)[KM], Acc fp,
+                                unsigned char* wsp, double* red) {
+  constexpr int NT = BT / TEAM, H = 2;
+  static_assert(2 * BT * H <= RING_WS, "the combine buffer holds two column pairs of all threads");
+  const int tid = threadIdx.x, lt = tid % TEAM, team = tid / TEAM;
+  const int np2 = I.pitch / 2;
+  auto entry = [](Acc2 c) {
+    const Acc a = acc2_x(c), b = acc2_y(c);
+    return make_float4(a.s, a.l, b.s, b.l);
+  };
+  float4* out = reinterpret_cast<float4*>(I.partials) + (int64_t)w.tile * np2;
+  if constexpr (NT == 1) {
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+      if (lt + k * TEAM < np2) out[lt + k * TEAM] = entry(xb[k]);
+  } else {
+    float4* ws = reinterpret_cast<float4*>(wsp);  // [NT][TEAM * H]
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
+      if (half * H * TEAM >= np2) break;
 #pragma unroll
-      for (int kk = 0; kk < H; ++kk)  // columns k >= KM are past the row's end: not read
-        if (half * H + kk < KM) ws[team * TEAM * H + lt + kk * TEAM] = xbp[half * H + kk < KM ? half * H + kk : 0];
+      for (int kk = 0; kk < H; ++kk)  // column pairs k >= KM are past the row's end: not read
+        if (half * H + kk < KM) ws[team * TEAM * H + lt + kk * TEAM] = entry(xb[half * H + kk < KM ? half * H + kk : 0]);
       __syncthreads();
       for (int jj = tid; jj < TEAM * H; jj += BT) {
-        const int j = jj % TEAM + (half * H + jj / TEAM) * TEAM;
-        if (j < n) {
-          Acc s = ws[jj];
-          for (int t2 = 1; t2 < NT; ++t2) s = acc_add(s, ws[t2 * TEAM * H + jj]);
-          out[j] = s;
+        const int jp = jj + half * H * TEAM;
+        if (jp < np2) {
+          float4 e = ws[jj];
+          Acc a{e.x, e.y}, b{e.z, e.w};
+          for (int t2 = 1; t2 < NT; ++t2) {
+            e = ws[t2 * TEAM * H + jj];
+            a = acc_add(a, Acc{e.x, e.y});
+            b = acc_add(b, Acc{e.z, e.w});
+          }
+          out[jp] = make_float4(a.s, a.l, b.s, b.l);
         }
       }
       __syncthreads();
@@ -539,6 +346,161 @@ __device__ double dense_tile_ring(const BInst& I, const BItem& w, const Ring& R,
   for (int t2 = 1; t2 < NT; ++t2) tot = acc_add(tot, ra[t2]);
   __syncthreads();
   return acc_to_double(tot);
+}
+
+// Rows of a pair-batch instance without a float-pair copy: FP64 data, split on
+// every load, in the ring path's order of operations (the same bits).
+template <int TEAM>
+__device__ double dense_tile_split(const BInst& I, const BItem& w, unsigned char* wsp, double* red, bool& bad) {
+  constexpr int NT = BT / TEAM, KM = B_CPT / 2;
+  const int lt = threadIdx.x % TEAM, team = threadIdx.x / TEAM;
+  const double* __restrict__ A = static_cast<const double*>(I.d0);
+  const int n = I.n, kp = (I.pitch / 2 + TEAM - 1) / TEAM;
+  Pair2 xp[KM];
+  Acc2 xb[KM];
+  pair_load_x<TEAM>(I, xp, xb, bad);
+  Acc fp = acc_zero();
+  const int64_t r1 = w.start + w.count;
+  const int steps = (w.count + 2 * NT - 1) / (2 * NT);
+  for (int c = 0; c < steps; ++c) {
+    const int64_t row0 = w.start + (int64_t)c * 2 * NT;
+    const int64_t rr[2] = {row0 + team, row0 + NT + team};
+    const bool vr[2] = {rr[0] < r1, rr[1] < r1};
+    Pair2 av[2][KM];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double* Ar = A + (vr[q] ? rr[q] : w.start) * (int64_t)n;
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const int j = 2 * (lt + k * TEAM);
+        const double v0 = vr[q] && j < n ? __ldcs(Ar + j) : 0.0;
+        const double v1 = vr[q] && j + 1 < n ? __ldcs(Ar + j + 1) : 0.0;
+        av[q][k] = pair2_of(split_f64(v0), split_f64(v1));
+      }
+    }
+    pair_two_rows<TEAM>(av, kp, xp, xb, fp, vr, red, c & 1, [&] {
+      if constexpr (TEAM > 32) team_barrier<TEAM>(team);
+      return false;
+    });
+    if ((c & 7) == 7) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) acc2_renorm(xb[k]);
+    }
+  }
+  __syncthreads();
+  return pair_tile_end<TEAM>(I, w, xb, fp, wsp, red);
+}
+
+// ---- ... on float-pair copies: rows staged by bulk copies ----
+// A tile's rows are contiguous, so its data arrives by 1-D bulk copies (TMA)
+// into a ring of RING_S shared-memory slots, one iteration group (the 2 NT rows
+// one step of the teams takes, at most 32 KB: 4 column pairs a team thread) a
+// slot, while the teams compute on the slot before: bytes in flight without
+// registers.  Rows of a copy are `pitch` entries, so they start on 16-byte
+// boundaries.  All threads count the chunks the CTA has consumed (g), which
+// gives each slot's barrier phase across tiles; thread 0, the only one that
+// issues, counts the chunks issued (iss).  When a tile has no chunk left to
+// issue, the slots it frees take the first chunks of the CTA's next item
+// (claimed when this one started) if that is a ring tile too, so the copies
+// run on across the tile boundary.
+constexpr int RING_S = 3;
+constexpr int RING_SLOT = 32768;
+
+struct Ring {
+  unsigned char* slots;  // RING_S * RING_SLOT bytes
+  uint64_t* full;        // RING_S barriers: a slot's copy has landed
+};
+
+// The CTA's next item as ring chunks (thread 0 only); nchunks 0: not a ring tile.
+struct RingNext {
+  const double* src;   // its first row
+  int64_t chunk;       // entries a chunk (2 NT pitch)
+  int64_t total;       // entries of the item (count pitch)
+  int nchunks;
+};
+
+__device__ __forceinline__ void ring_issue(const Ring& R, uint32_t g, const void* src, size_t bytes) {
+  const int slot = (int)(g % RING_S);
+  mbar_arrive_expect_tx(&R.full[slot], (uint32_t)bytes);
+  tma_load_1d(R.slots + slot * RING_SLOT, src, (uint32_t)bytes, &R.full[slot]);
+}
+
+// Rows of an instance with a copy, read from the ring.  Returns the tile's f;
+// sets `failed` (on all threads) when a copy did not land within the wait limit,
+// after waiting for the CTA's other copies in flight.
+// KP > 0: the column pairs per team thread, ceil(pitch / 2 / TEAM), fixed at
+// compile time (no test but the last pair's); 0: at run time.
+template <int TEAM, int KP>
+__device__ double dense_tile_ring(const BInst& I, const BItem& w, const Ring& R, uint32_t& g,
+                                  uint32_t& iss, const RingNext& nx, unsigned char* wsp, double* red,
+                                  bool& bad, bool& failed) {
+  const int tid = threadIdx.x;
+  const double* __restrict__ A = static_cast<const double*>(I.d0);  // float pairs, 8 bytes an entry
+  constexpr int NT = BT / TEAM, KM = KP ? KP : B_CPT / 2;
+  const int lt = tid % TEAM, team = tid / TEAM;
+  const int np = I.pitch, np2 = np / 2;
+  const int kp = KP ? KP : (np2 + TEAM - 1) / TEAM;
+  // pair k of this thread is in the row: compile-time true below the last one
+  auto in_row = [&](int k) { return (KP && k < KP - 1) || lt + k * TEAM < np2; };
+  Pair2 xp[KM];
+  Acc2 xb[KM];
+  pair_load_x<TEAM>(I, xp, xb, bad);
+  Acc fp = acc_zero();
+  const int64_t r1 = w.start + w.count;
+  const int nchunks = (w.count + 2 * NT - 1) / (2 * NT);
+  auto chunk_src = [&](int c) { return A + (w.start + (int64_t)c * 2 * NT) * np; };
+  auto chunk_bytes = [&](int c) {
+    const int64_t left = r1 - (w.start + (int64_t)c * 2 * NT);
+    return (size_t)(left < 2 * NT ? left : 2 * NT) * np * 8;
+  };
+  const uint32_t g0 = g;  // this tile's chunk c is the CTA's chunk g0 + c
+  if (tid == 0)  // (the first ones may have been issued by the tile before)
+    for (; (int)(iss - g0) < nchunks && iss - g0 < (uint32_t)RING_S; ++iss)
+      ring_issue(R, iss, chunk_src((int)(iss - g0)), chunk_bytes((int)(iss - g0)));
+  for (int c = 0; c < nchunks; ++c) {
+    const int slot = (int)(g % RING_S);
+    const bool ok = mbar_wait_bounded(&R.full[slot], (g / RING_S) & 1u);
+    const float4* buf = reinterpret_cast<const float4*>(R.slots + slot * RING_SLOT);
+    const int64_t row0 = w.start + (int64_t)c * 2 * NT;
+    const bool vr[2] = {ok && row0 + team < r1, ok && row0 + NT + team < r1};
+    Pair2 av[2][KM];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float4* Ar = buf + (q * NT + team) * np2;
+#pragma unroll
+      for (int k = 0; k < KM; ++k)
+        av[q][k] = vr[q] && in_row(k) ? pair2_load(Ar + lt + k * TEAM) : Pair2{f2_zero(), f2_zero()};
+    }
+    // one CTA barrier a chunk: the slot's entries are in registers by then, so the
+    // slot is refilled behind it; it also publishes the warps' sums
+    const bool lost = pair_two_rows<TEAM>(av, kp, xp, xb, fp, vr, red, c & 1, [&] {
+      if (__syncthreads_or(!ok)) return true;
+      if (tid == 0 && iss - g0 < (uint32_t)(nchunks + nx.nchunks)) {
+        const int k = (int)(iss - g0);
+        if (k < nchunks) {
+          ring_issue(R, iss, chunk_src(k), chunk_bytes(k));
+        } else {  // the next item's chunk k - nchunks
+          const int64_t e0 = (int64_t)(k - nchunks) * nx.chunk, left = nx.total - e0;
+          ring_issue(R, iss, nx.src + e0, (size_t)(left < nx.chunk ? left : nx.chunk) * 8);
+        }
+        ++iss;
+      }
+      return false;
+    });
+    if (lost) {
+      if (tid == 0)  // do not go on with a copy into this CTA's shared memory in flight
+        for (uint32_t h = g; h < iss; ++h) mbar_wait_bounded(&R.full[h % RING_S], (h / RING_S) & 1u);
+      failed = true;
+      __syncthreads();
+      return 0.0;
+    }
+    ++g;
+    if ((c & 7) == 7) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) acc2_renorm(xb[k]);
+    }
+  }
+  return pair_tile_end<TEAM>(I, w, xb, fp, wsp, red);
 }
 
 // Elements [w.start, w.start + w.count) of a tet instance; returns the tile's f.
@@ -619,92 +581,110 @@ __device__ double tet_tile(const BInst& I, const BItem& w, const float4* tab, co
   }
 }
 
-template <typename T, bool PAIR>
-__device__ __forceinline__ double dense_dispatch(const BInst& I, const BItem& w, unsigned char* wsp,
-                                                 double* red, bool& bad) {
-  switch (I.team) {
-    case 4: return dense_tile<T, PAIR, 4>(I, w, wsp, red, bad);
-    case 8: return dense_tile<T, PAIR, 8>(I, w, wsp, red, bad);
-    case 16: return dense_tile<T, PAIR, 16>(I, w, wsp, red, bad);
-    case 32: return dense_tile<T, PAIR, 32>(I, w, wsp, red, bad);
-    case 64: return dense_tile<T, PAIR, 64>(I, w, wsp, red, bad);
-    case 128: return dense_tile<T, PAIR, 128>(I, w, wsp, red, bad);
-    default: return dense_tile<T, PAIR, BT>(I, w, wsp, red, bad);
+// Calls go.template run<TEAM>() with the instance's team width.
+template <typename Go>
+__device__ __forceinline__ double with_team(int team, const Go& go) {
+  switch (team) {
+    case 4: return go.template run<4>();
+    case 8: return go.template run<8>();
+    case 16: return go.template run<16>();
+    case 32: return go.template run<32>();
+    case 64: return go.template run<64>();
+    case 128: return go.template run<128>();
+    default: return go.template run<BT>();
   }
 }
 
-// The team is the smallest power of two (>= 4) with 8 columns a thread, so
-// above 4 threads a team thread has 5 to 8 columns.
-template <int TEAM>
-__device__ __forceinline__ double dense_ring_cpt(const BInst& I, const BItem& w, const Ring& R, uint32_t& g,
-                                                 uint32_t& iss, const RingNext& nx, unsigned char* wsp,
-                                                 double* red, bool& bad, bool& failed) {
-  switch ((I.n + TEAM - 1) / TEAM) {
-    case 5: return dense_tile_ring<TEAM, 5>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 6: return dense_tile_ring<TEAM, 6>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 7: return dense_tile_ring<TEAM, 7>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 8: return dense_tile_ring<TEAM, 8>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    default: return dense_tile_ring<TEAM, 0>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-  }
-}
+template <typename T>
+struct NativeTile {
+  const BInst& I;
+  const BItem& w;
+  unsigned char* wsp;
+  double* red;
+  template <int TEAM>
+  __device__ __forceinline__ double run() const { return dense_tile<T, TEAM>(I, w, wsp, red); }
+};
 
-__device__ __forceinline__ double dense_ring_dispatch(const BInst& I, const BItem& w, const Ring& R,
-                                                      uint32_t& g, uint32_t& iss, const RingNext& nx,
-                                                      unsigned char* wsp, double* red, bool& bad,
-                                                      bool& failed) {
-  switch (I.team) {
-    case 4: return dense_tile_ring<4, 0>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 8: return dense_ring_cpt<8>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 16: return dense_ring_cpt<16>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 32: return dense_ring_cpt<32>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 64: return dense_ring_cpt<64>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    case 128: return dense_ring_cpt<128>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-    default: return dense_ring_cpt<BT>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-  }
-}
+struct SplitTile {
+  const BInst& I;
+  const BItem& w;
+  unsigned char* wsp;
+  double* red;
+  bool& bad;
+  template <int TEAM>
+  __device__ __forceinline__ double run() const { return dense_tile_split<TEAM>(I, w, wsp, red, bad); }
+};
 
-// Last tile of an instance: sum the tile partials in tile order.
-template <typename T, bool PAIR>
-__device__ void finalize(const BInst& I, double* red) {
-  const int tid = threadIdx.x;
-  if (I.kind == BK_DENSE) {
-    const int n = I.n;
-    for (int j = tid; j < n; j += BT) {
-      if constexpr (PAIR) {
-        const Acc* P = static_cast<const Acc*>(I.partials);
-        Acc s = acc_zero();
-        for (int t = 0; t < I.ntiles; ++t) {
-          const float2 v = __ldcg(reinterpret_cast<const float2*>(P + (int64_t)t * n + j));
-          s = acc_add(s, Acc{v.x, v.y});
-          if ((t & 31) == 31) acc_renorm(s);
-        }
-        static_cast<double*>(I.gx)[j] = pair_to_double_fast(acc_pair(s));
-      } else {
-        const T* P = static_cast<const T*>(I.partials);
-        T s = T(0);
-        for (int t = 0; t < I.ntiles; ++t) s += __ldcg(P + (int64_t)t * n + j);
-        static_cast<T*>(I.gx)[j] = s;
-      }
+struct RingTile {
+  const BInst& I;
+  const BItem& w;
+  const Ring& R;
+  uint32_t &g, &iss;
+  const RingNext& nx;
+  unsigned char* wsp;
+  double* red;
+  bool &bad, &failed;
+  // the team is the smallest power of two (>= 4) with 4 column pairs a thread, so
+  // above 4 threads a team thread has 3 or 4
+  template <int TEAM>
+  __device__ __forceinline__ double run() const {
+    if constexpr (TEAM > 4) {
+      const int kp = (I.pitch / 2 + TEAM - 1) / TEAM;
+      if (kp == 4) return dense_tile_ring<TEAM, 4>(I, w, R, g, iss, nx, wsp, red, bad, failed);
+      if (kp == 3) return dense_tile_ring<TEAM, 3>(I, w, R, g, iss, nx, wsp, red, bad, failed);
     }
+    return dense_tile_ring<TEAM, 0>(I, w, R, g, iss, nx, wsp, red, bad, failed);
   }
-  if (tid == 0 && I.f) {
-    double fs = 0.0;
-    for (int t = 0; t < I.ntiles; ++t) fs += __ldcg(I.fpart + t);
-    *static_cast<T*>(I.f) = (T)fs;
+};
+
+// The instance's f from its tile partials: lane l of warp 0 adds tiles l, l + 32, ..., then
+// a butterfly (call with warp 0 only).
+template <typename T>
+__device__ __forceinline__ void sum_f(const BInst& I) {
+  double fs = 0.0;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < I.ntiles; t += 32) fs += __ldcg(I.fpart + t);
+  fs = warp_sum(fs);
+  if (threadIdx.x == 0 && I.f) *static_cast<T*>(I.f) = (T)fs;
+}
+
+// Columns [j0, j0 + cols) of a dense instance's gradient: a thread per column adds the
+// tile partials in tile order, eight loads in flight.
+template <typename T, bool PAIR>
+__device__ void sum_columns(const BInst& I, int j0, int cols) {
+  using P = std::conditional_t<PAIR, float2, T>;
+  using S = std::conditional_t<PAIR, Acc, T>;
+  const P* parts = static_cast<const P*>(I.partials);
+  const int64_t pitch = PAIR ? I.pitch : I.n;
+  for (int j = j0 + threadIdx.x; j < j0 + cols; j += BT) {
+    S s{};
+    for (int t = 0; t < I.ntiles; t += 8) {
+      P v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = t + u < I.ntiles ? __ldcg(parts + (t + u) * pitch + j) : P{};
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if constexpr (PAIR) s = acc_add(s, Acc{v[u].x, v[u].y});
+        else s += v[u];
+      }
+      if constexpr (PAIR)
+        if ((t & 24) == 24) acc_renorm(s);
+    }
+    if constexpr (PAIR) static_cast<double*>(I.gx)[j] = pair_to_double_fast(acc_pair(s));
+    else static_cast<T*>(I.gx)[j] = s;
   }
 }
 
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
-  // PAIR: [log table][ring: RING_S slots][ring combine buffer][red][ring barriers];
-  // the other dense tiles of a pair batch combine inside the ring (idle then).
+  // PAIR: [log table][ring: RING_S slots][combine buffer][red][ring barriers].
   // Otherwise [wsp][red].
   extern __shared__ __align__(16) unsigned char smem[];
   float4* tab = reinterpret_cast<float4*>(smem);
-  unsigned char* wsp = smem + (PAIR ? kLogTableSize * sizeof(float4) : 0);
-  unsigned char* rws = wsp + (PAIR ? (size_t)RING_S * RING_SLOT : 0);
-  double* red = reinterpret_cast<double*>(PAIR ? rws + RING_WS * sizeof(Acc) : wsp + (size_t)BT * B_CPT * 8);
-  Ring R{wsp, reinterpret_cast<uint64_t*>(red + 64)};
+  unsigned char* slots = smem + (PAIR ? kLogTableSize * sizeof(float4) : 0);
+  unsigned char* rws = slots + (PAIR ? (size_t)RING_S * RING_SLOT : 0);  // combine buffer
+  double* red = reinterpret_cast<double*>(rws + (PAIR ? RING_WS * sizeof(Acc) : (size_t)BT * B_CPT * 8));
+  Ring R{slots, reinterpret_cast<uint64_t*>(red + 64)};
   uint32_t g = 0, iss = 0;  // ring chunks consumed by this CTA; issued (thread 0)
   __shared__ int s_item, s_last;
   const int tid = threadIdx.x;
@@ -731,17 +711,45 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
       if (PAIR && nit < a.nitems) {
         const BItem wn = a.items[nit];
         const BInst& In = a.insts[wn.inst];
-        if (In.kind == BK_DENSE && In.prep) {
-          const int64_t rows = 2 * (BT / In.team);
-          nx.src = static_cast<const double*>(In.d0) + wn.start * (int64_t)In.n;
-          nx.chunk = rows * In.n;
-          nx.total = (int64_t)wn.count * In.n;
+        if (In.kind == BK_DENSE && In.prep && wn.tile >= 0) {
+          const int64_t rows = 2 * (BT / In.team);  // a step's
+          nx.src = static_cast<const double*>(In.d0) + wn.start * (int64_t)In.pitch;
+          nx.chunk = rows * In.pitch;
+          nx.total = (int64_t)wn.count * In.pitch;
           nx.nchunks = (int)((wn.count + rows - 1) / rows);
         }
       }
     }
     const BItem w = a.items[it];
     const BInst I = a.insts[w.inst];
+    if (w.tile < 0) {
+      // every tile item comes before the sum items and is held by a running CTA (this
+      // one has none left), so the wait ends
+      if (tid == 0) {
+        const uint64_t t0 = global_ns();
+        s_last = 1;
+        while (ld_acquire_u32(I.done) < (unsigned)I.ntiles) {
+          if (global_ns() - t0 > kWaitLimitNs) {
+            set_error(a.err, ERRBIT_TIMEOUT);
+            s_last = 0;
+            break;
+          }
+        }
+        __threadfence();
+      }
+      __syncthreads();
+      if (s_last) {
+        if (w.start == 0 && tid < 32) sum_f<T>(I);
+        sum_columns<T, PAIR>(I, (int)w.start, w.count);
+      }
+      __syncthreads();
+      if (tid == 0 && atomicAdd(I.done + 1, 1u) == (unsigned)I.nsum - 1u) {  // all have waited
+        I.done[0] = 0u;
+        I.done[1] = 0u;
+      }
+      it = s_item;
+      continue;
+    }
     // the tile's contiguous data into L2 while the first loads are in flight (not
     // for the ring's tiles: their copies stream it, and whole-tile prefetches of
     // every CTA exceed L2 and are evicted before use)
@@ -759,14 +767,14 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
     const bool prep = PAIR && I.prep;
     if (I.kind == BK_DENSE) {
       if constexpr (PAIR) {
-        ft = prep ? dense_ring_dispatch(I, w, R, g, iss, nx, rws, red, bad, failed)
-                  : dense_dispatch<T, PAIR>(I, w, wsp, red, bad);
+        ft = prep ? with_team(I.team, RingTile{I, w, R, g, iss, nx, rws, red, bad, failed})
+                  : with_team(I.team, SplitTile{I, w, rws, red, bad});
         if (failed) {  // a copy did not land: this CTA leaves the queue
           if (tid == 0) set_error(a.err, ERRBIT_TIMEOUT);
           break;
         }
       } else {
-        ft = dense_dispatch<T, PAIR>(I, w, wsp, red, bad);
+        ft = with_team(I.team, NativeTile<T>{I, w, rws, red});
       }
     } else {
       if (a.warpc)
@@ -781,9 +789,10 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
     __syncthreads();
     if (tid == 0) s_last = atomicAdd(I.done, 1u) == (unsigned)I.ntiles - 1u;
     __syncthreads();
-    if (s_last) {
+    if (s_last && I.nsum == 0) {
       __threadfence();
-      finalize<T, PAIR>(I, red);
+      if (tid < 32) sum_f<T>(I);
+      if (I.kind == BK_DENSE) sum_columns<T, PAIR>(I, 0, I.n);
       if (tid == 0) *I.done = 0u;
     }
     it = s_item;  // written by thread 0 before the barriers above
@@ -796,6 +805,18 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
       a.head[1] = 0u;
       __threadfence();
     }
+  }
+}
+
+// The float pairs of m rows of n (odd) doubles, n + 1 entries a row, the last a zero.
+__global__ void pair_rows_kernel(const double* __restrict__ A, float4* __restrict__ out, int64_t m, int n) {
+  const int np2 = (n + 1) / 2;
+  const int64_t count = m * np2, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
+    const int64_t r = i / np2;
+    const int j = 2 * (int)(i - r * np2);
+    const double* a = A + r * n + j;
+    out[i] = pair2_entry(split_f64(a[0]), split_f64(j + 1 < n ? a[1] : 0.0));
   }
 }
 
@@ -877,6 +898,7 @@ namespace {
 struct Plan {
   std::vector<BInst> insts;
   std::vector<BItem> items;
+  std::vector<BItem> sums;       // after all tiles, in the order of their instances' size
   std::vector<int> tet_ids;
   std::vector<size_t> part_off;  // byte offset of each dense instance's partials
   std::vector<size_t> fpart_off; // index of each instance's first f partial
@@ -891,11 +913,33 @@ struct Tuning {
 int default_rows(int n) { return n <= 64 ? 128 : n <= 256 ? 64 : (n <= 1024 ? 16 : 8); }
 int default_elems(int64_t) { return 4096; }
 
+// Bytes a work item streams, the tets' weighted by their lower rate.
+double item_cost(const kg_problem* p, int64_t count, size_t es) {
+  return p->kind == KG_QUADFORM ? (double)count * p->n * es : 1.7 * (double)count * (16.0 + 12.0 * es);
+}
+
+// Dense instances of more tiles than this are summed by items of their own, by all CTAs
+// that have no tile left: the last tile's CTA alone reads 256 columns of 8 partials in
+// about a microsecond, 48 partials of 2035 columns in 50, at the end of the batch.
+constexpr int B_SUM_TILES = 16;
+// No tile is larger than a CTA's share of the batch / B_SHARE, so that a batch of few
+// large instances still fills the grid: the autotuner's tiles (up to 256 rows, right for
+// batches of thousands) gave 128 dense and 16 tet instances two items a CTA.  Measured on
+// that batch, 630 MB: shares of 2, 3, 4 and 6 take 183, 174, 172 and 185 us (tuned tiles
+// of 128 rows), 172, 171, 174 and 183 us (of 64).
+constexpr int B_SHARE = 3;
+
 // prep[i]: the float-pair copy of problem i's A (dense) or G (tet) that the
-// batch streams, or NULL (the FP64 data, split per load).
+// batch streams, or NULL (the FP64 data, split per load).  grid > 0: tiles are
+// cut so that none exceeds a CTA's share of these instances / B_SHARE.
 Plan make_plan(const std::vector<kg_problem*>& probs, const std::vector<const void*>& prep,
-               const std::vector<int>& ids, const Tuning& tu, bool pair, size_t es) {
+               const std::vector<int>& ids, const Tuning& tu, bool pair, size_t es, int grid) {
   Plan P;
+  double cap = 0.0;
+  if (grid > 0) {
+    for (int i : ids) cap += item_cost(probs[i], probs[i]->m, es);
+    cap /= (double)B_SHARE * grid;
+  }
   struct Cost {
     double c;
     BItem it;
@@ -906,6 +950,7 @@ Plan make_plan(const std::vector<kg_problem*>& probs, const std::vector<const vo
     BInst I{};
     I.kind = p->kind == KG_QUADFORM ? BK_DENSE : BK_TET;
     I.n = (int)p->n;
+    I.pitch = (int)(p->n + (p->n & 1));
     I.m = p->m;
     I.d0 = p->data0;
     I.d1 = p->data1;
@@ -927,24 +972,38 @@ Plan make_plan(const std::vector<kg_problem*>& probs, const std::vector<const vo
       I.team = 0;
       P.tet_ids.push_back(idx);
     }
+    if (cap > 0.0) {  // whole steps of the row teams (2 rows each) or of the CTA's threads, 4 at least
+      const int64_t unit = I.kind == BK_DENSE ? 2 * (BT / I.team) : BT;
+      const int64_t most = (int64_t)(cap / item_cost(p, unit, es)) * unit;
+      per = std::min(per, std::max(most, 4 * unit));
+    }
     I.ntiles = (int)((I.m + per - 1) / per);
+    if (I.kind == BK_DENSE && I.ntiles > B_SUM_TILES) {
+      for (int j = 0; j < I.n; j += BT) {
+        P.sums.push_back(BItem{idx, -1, j, std::min(BT, I.n - j)});
+        ++I.nsum;
+      }
+    }
     P.fpart_off.push_back(P.fparts);
     P.fparts += I.ntiles;
     P.part_off.push_back(P.part_bytes);
     if (I.kind == BK_DENSE) {
-      const size_t b = (size_t)I.ntiles * I.n * (pair ? sizeof(Acc) : es);
+      const size_t b = (size_t)I.ntiles * (pair ? I.pitch * sizeof(Acc) : I.n * es);
       P.part_bytes += (b + 255) & ~size_t(255);
     }
     for (int t = 0; t < I.ntiles; ++t) {
       BItem it{idx, t, (int64_t)t * per, (int)std::min<int64_t>(per, I.m - (int64_t)t * per)};
-      const double bytes = I.kind == BK_DENSE ? (double)it.count * I.n * es
-                                              : (double)it.count * (16.0 + 12.0 * es);
-      all.push_back({bytes, it});
+      all.push_back({item_cost(p, it.count, es), it});
     }
     P.insts.push_back(I);
   }
   std::stable_sort(all.begin(), all.end(), [](const Cost& a, const Cost& b) { return a.c > b.c; });
   for (const auto& c : all) P.items.push_back(c.it);
+  // instances whose tiles come first are summed first
+  std::stable_sort(P.sums.begin(), P.sums.end(), [&](const BItem& a, const BItem& b) {
+    return P.insts[a.inst].m * P.insts[a.inst].n > P.insts[b.inst].m * P.insts[b.inst].n;
+  });
+  P.items.insert(P.items.end(), P.sums.begin(), P.sums.end());
   return P;
 }
 
@@ -980,17 +1039,17 @@ kg_status devplan_alloc(DevPlan& D, Plan& P, cudaStream_t s) {
   if ((rc = al((void**)&D.items, sizeof(BItem) * P.items.size(), "work table")) != KG_OK) return rc;
   if ((rc = al((void**)&D.tet_ids, sizeof(int) * std::max<size_t>(1, P.tet_ids.size()), "tet ids")) != KG_OK) return rc;
   if ((rc = al((void**)&D.head, 16, "queue head")) != KG_OK) return rc;
-  if ((rc = al((void**)&D.done, sizeof(unsigned) * P.insts.size(), "arrival counters")) != KG_OK) return rc;
+  if ((rc = al((void**)&D.done, 2 * sizeof(unsigned) * P.insts.size(), "arrival counters")) != KG_OK) return rc;
   if ((rc = al((void**)&D.parts, std::max<size_t>(256, P.part_bytes), "partials")) != KG_OK) return rc;
   if ((rc = al((void**)&D.fpart, sizeof(double) * std::max<size_t>(1, P.fparts), "f partials")) != KG_OK) return rc;
   for (int i = 0; i < D.ninst; ++i) {
     P.insts[i].partials = D.parts + P.part_off[i];
     P.insts[i].fpart = D.fpart + P.fpart_off[i];
-    P.insts[i].done = D.done + i;
+    P.insts[i].done = D.done + 2 * i;
   }
   cudaError_t e;
   if ((e = cudaMemsetAsync(D.head, 0, 16, s)) != cudaSuccess) return cuda_fail(e, "batch set-up");
-  if ((e = cudaMemsetAsync(D.done, 0, sizeof(unsigned) * P.insts.size(), s)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(D.done, 0, 2 * sizeof(unsigned) * P.insts.size(), s)) != cudaSuccess)
     return cuda_fail(e, "batch set-up");
   if ((e = cudaMemcpyAsync(D.items, P.items.data(), sizeof(BItem) * P.items.size(),
                            cudaMemcpyHostToDevice, s)) != cudaSuccess)
@@ -1020,6 +1079,16 @@ int batched_grid(bool pair) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batched_kernel<double, false>, BT, smem);
   if (e != cudaSuccess || per < 1) per = 2;
   return num_sms() * std::min(per, 4);
+}
+
+// The float-pair copy of m rows of n doubles, rows padded to whole column pairs.
+kg_status pair_prepare_rows(const double* src, void* dst, int64_t m, int64_t n, cudaStream_t s) {
+  if (n % 2 == 0) return pair_prepare(src, dst, m * n, s);
+  const int64_t count = m * ((n + 1) / 2);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((count + 255) / 256, (int64_t)num_sms() * 8));
+  pair_rows_kernel<<<grid, 256, 0, s>>>(src, static_cast<float4*>(dst), m, (int)n);
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? KG_OK : cuda_fail(e, "prepare float pairs");
 }
 
 // Launches the zero kernel (tet gradients) and the persistent kernel on s.
@@ -1097,7 +1166,7 @@ std::string gpu_name() {
 // Times the persistent kernel on the instances `ids` with tuning `tu`.
 kg_status time_plan(kg_batch* b, const std::vector<int>& ids, const Tuning& tu, cudaStream_t s,
                     void* xbuf, void* gbuf, float* ms) {
-  Plan P = make_plan(b->probs, b->prep, ids, tu, b->pair, b->es);
+  Plan P = make_plan(b->probs, b->prep, ids, tu, b->pair, b->es, b->grid);
   DevPlan D;
   kg_status rc = devplan_alloc(D, P, s);
   if (rc == KG_OK) {
@@ -1135,9 +1204,11 @@ kg_status time_plan(kg_batch* b, const std::vector<int>& ids, const Tuning& tu, 
 // Chooses rows (dense) / elements (tet) per item for every size bucket of the
 // batch: each candidate runs on a sample of the bucket's instances large
 // enough that the largest candidate still gives four items per CTA of the
-// persistent grid (or on all of them); the fastest wins.  A smaller sample
-// would favour small tiles for want of parallelism that the whole batch has.
-// Choices are cached by GPU name, kind, dtype, arithmetic and bucket.
+// persistent grid (or on all of them); the largest tile within 3% of the
+// fastest wins.  A smaller sample favours small tiles for want of parallelism
+// that the whole batch has (make_plan cuts them to a CTA's share anyway): there
+// the largest within 10% wins (on 128 dense and 16 tet instances the fastest
+// ones made tiles of 16 rows and 187 us, these 171).  Choices are cached by GPU name, kind, dtype, arithmetic and bucket.
 kg_status autotune(kg_batch* b, cudaStream_t s) {
   std::map<std::pair<int, int>, std::vector<int>> groups;  // (kind, bucket) -> instance ids
   for (int i = 0; i < (int)b->probs.size(); ++i) {
@@ -1148,8 +1219,8 @@ kg_status autotune(kg_batch* b, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   std::map<std::string, int> cache = cache_read();
   bool dirty = false;
-  // "k3": dense tiles of pair batches stream float-pair copies through a ring; larger samples
-  const std::string prefix = b->gpu + "|k3|" + (b->dtype == KG_F64 ? "f64" : "f32") + "|" +
+  // "k4": dense tiles of pair batches in packed column pairs through a ring of bulk copies
+  const std::string prefix = b->gpu + "|k4|" + (b->dtype == KG_F64 ? "f64" : "f32") + "|" +
                              (b->pair ? "pair" : "native") + "|";
   const std::vector<int> dense_cands{4, 8, 16, 32, 64, 128, 256}, tet_cands{1024, 2048, 4096, 8192, 16384};
   std::map<std::pair<int, int>, std::vector<int>> sample;
@@ -1187,19 +1258,20 @@ kg_status autotune(kg_batch* b, cudaStream_t s) {
     }
     const std::vector<int>& ids = sample[g.first];
     const std::vector<int>& cands = kind == BK_DENSE ? dense_cands : tet_cands;
-    int best = cands[0];
-    float best_ms = 1e30f;
-    for (int c : cands) {
+    std::vector<float> ms(cands.size(), 0.f);
+    for (size_t i = 0; i < cands.size() && rc == KG_OK; ++i) {
       Tuning tu;
-      (kind == BK_DENSE ? tu.dense_rows : tu.tet_elems)[bucket] = c;
-      float ms = 0.f;
-      if ((rc = time_plan(b, ids, tu, s, xbuf, gbuf, &ms)) != KG_OK) break;
-      if (ms < best_ms) {
-        best_ms = ms;
-        best = c;
-      }
+      (kind == BK_DENSE ? tu.dense_rows : tu.tet_elems)[bucket] = cands[i];
+      rc = time_plan(b, ids, tu, s, xbuf, gbuf, &ms[i]);
     }
     if (rc != KG_OK) break;
+    int64_t items = 0;
+    for (int i : ids) items += (b->probs[i]->m + cands.back() - 1) / cands.back();
+    const float slack = items >= 4 * (int64_t)b->grid ? 1.03f : 1.10f;
+    const float least = *std::min_element(ms.begin(), ms.end());
+    int best = cands[0];
+    for (size_t i = 0; i < cands.size(); ++i)
+      if (ms[i] <= slack * least) best = cands[i];
     (kind == BK_DENSE ? b->tune.dense_rows : b->tune.tet_elems)[bucket] = best;
     cache[key] = best;
     dirty = true;
@@ -1293,13 +1365,13 @@ kg_status kg_batch_create(kg_batch** out, kg_problem* const* probs, int count,
       const size_t bytes = 8 * (size_t)p->m * (size_t)p->n;
       if (bytes > budget) continue;
       void* q = nullptr;
-      // 16 bytes beyond the end: the ring's copies read whole 16-byte units
-      if (dev_alloc(&q, bytes + 16) != cudaSuccess) {
+      // rows of odd n are padded by a zero to whole column pairs
+      if (dev_alloc(&q, 8 * (size_t)p->m * (size_t)(p->n + (p->n & 1))) != cudaSuccess) {
         rc = fail(KG_ERR_OOM, "kg_batch_create: float-pair copy of A");
         break;
       }
       b->own_preps.push_back(q);
-      if ((rc = pair_prepare(static_cast<const double*>(p->data0), q, p->m * p->n, s)) != KG_OK) break;
+      if ((rc = pair_prepare_rows(static_cast<const double*>(p->data0), q, p->m, p->n, s)) != KG_OK) break;
       b->prep[i] = q;
       budget -= bytes;
     }
@@ -1321,7 +1393,7 @@ kg_status kg_batch_create(kg_batch** out, kg_problem* const* probs, int count,
   if (rc == KG_OK) {
     std::vector<int> ids(count);
     for (int i = 0; i < count; ++i) ids[i] = i;
-    b->plan = make_plan(b->probs, b->prep, ids, b->tune, b->pair, b->es);
+    b->plan = make_plan(b->probs, b->prep, ids, b->tune, b->pair, b->es, b->grid);
     rc = devplan_alloc(b->dev, b->plan, s);
   }
   if (rc == KG_OK) {
@@ -1414,7 +1486,7 @@ kg_status kg_grad_batched_loop(kg_batch* b, const void* const* x, void* const* f
 kg_status kg_batch_get_config(const kg_batch* b, int* arith, int* items, int* grid) {
   if (!b) return fail(KG_ERR_INVALID_ARG, "kg_batch_get_config: NULL batch");
   if (arith) *arith = b->pair ? KG_ARITH_PAIR : KG_ARITH_NATIVE;
-  if (items) *items = b->dev.nitems;
+  if (items) *items = b->dev.nitems - (int)b->plan.sums.size();
   if (grid) *grid = b->grid;
   return KG_OK;
 }

@@ -4,8 +4,9 @@
 // kernels keep their data in FP64 memory and compute on pairs of floats
 // (hi + lo):
 //   - split_f64 turns a double into hi (its leading 24 significant bits,
-//     truncated) and lo (the next 23 bits) with integer instructions only;
-//     the pair holds the double to within 2^-46 relative for
+//     truncated) and lo (the rest, rounded to 23 bits) with integer
+//     instructions only; the pair holds the double to within 2^-47 relative,
+//     without bias (lo truncated, a dot product came out 2e-14 short), for
 //     2^-60 <= |d| < 2^40 (pair_in_range) and maps +-0 to +-0; callers check
 //     the range of their inputs.
 //   - products use the FMA error-free transformation: for floats a, b,
@@ -73,8 +74,9 @@ __host__ __device__ __forceinline__ uint32_t fshl3(uint32_t lo, uint32_t hi) {
 //       in its top 9 bits and (e - 896) = (e mod 512 + 128) mod 512 for every
 //       e in [897, 1150], so adding 2^30 re-biases the field; e = 0 (+-0) is
 //       kept as a signed zero by the select.
-//   lo: m[28:6] * 2^(E - 46), built as (1.m' * 2^k) - 2^k with 2^k = 2^(E-23)
-//       taken from hi's exponent field, so the subtraction is exact.
+//   lo: m[28:0] rounded at bit 6, times 2^(E - 46), built as (1.m' * 2^k) - 2^k
+//       with 2^k = 2^(E-23) taken from hi's exponent field, so the subtraction is
+//       exact (a carry out of the rounding goes into that field: 2^(k+1) - 2^k).
 // For d = +-0 the low word is 0 and lo = s - s = 0.
 __host__ __device__ __forceinline__ Pair split_f64(double d) {
   uint32_t lo, hi;
@@ -83,7 +85,7 @@ __host__ __device__ __forceinline__ Pair split_f64(double d) {
   const uint32_t t = fshl3(lo, hi);
   const uint32_t hb = (hi & 0x7FF00000u) ? ((t + 0x40000000u) | sign) : sign;
   const uint32_t fs = (hb & 0xFF800000u) - (23u << 23);
-  const uint32_t lb = fs | ((lo >> 6) & 0x007FFFFFu);
+  const uint32_t lb = fs + (((lo & 0x1FFFFFFFu) + 32u) >> 6);
   Pair p;
   p.h = u2f(hb);
   p.l = u2f(lb) - u2f(fs);

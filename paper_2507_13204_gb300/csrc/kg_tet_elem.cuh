@@ -252,7 +252,7 @@ __device__ __forceinline__ void elem_pair_core(const Pair (&G)[12], const Pair (
 }
 
 // One element in float-pair arithmetic (FP64 data).  Gs points at the
-// element's 12 doubles, or (PREP) at its 12 float pairs (h, l) prepared once.
+// element's 12 doubles, or (PREP) at its 12 float pairs prepared once, two as (h0, h1, l0, l1).
 // USPLIT: u points at float pairs of the vertex values, split (and range
 // checked) once per call by pair_split_vec instead of once per gather.
 template <int MODE, typename Sink, bool PREP = false, bool USPLIT = false>
@@ -265,8 +265,8 @@ __device__ __forceinline__ void elem_pair(const int4 c, const double* __restrict
   for (int i = 0; i < 12; i += 2) {
     if constexpr (PREP) {
       const float4 q = *reinterpret_cast<const float4*>(Gs + i);
-      G[i] = Pair{q.x, q.y};
-      G[i + 1] = Pair{q.z, q.w};
+      G[i] = Pair{q.x, q.z};
+      G[i + 1] = Pair{q.y, q.w};
     } else {
       const double2 v = *reinterpret_cast<const double2*>(Gs + i);
       G[i] = split_f64(v.x);
@@ -396,8 +396,8 @@ __device__ __forceinline__ void elem_pair_hvp(const int4 c, const double* __rest
   for (int i = 0; i < 12; i += 2) {
     if constexpr (PREP) {
       const float4 q = *reinterpret_cast<const float4*>(Gs + i);
-      G[i] = Pair{q.x, q.y};
-      G[i + 1] = Pair{q.z, q.w};
+      G[i] = Pair{q.x, q.z};
+      G[i + 1] = Pair{q.y, q.w};
     } else {
       const double2 q = *reinterpret_cast<const double2*>(Gs + i);
       G[i] = split_f64(q.x);

@@ -12,7 +12,10 @@
 //   - consumer thread t owns the column pairs jp = t + 512 k; it splits A's
 //     doubles into float pairs (integer instructions), writes the split values
 //     back in place so the reverse pass does not split again, and accumulates
-//     with FMA two-product / TwoSum on the FP32 units;
+//     with FMA two-product / TwoSum on the FP32 units, a column pair at a time in
+//     packed instructions (kg_pair2.cuh; scalar ones kept 36 instructions an entry
+//     against HBM: 10000 x 10000 value and gradient 144.5 -> 134.2 us, 118 us of
+//     them the bytes);
 //   - PREP: when the problem holds A already split into float pairs (made once
 //     by kg_create, same 8 bytes per entry), rows of that copy stream instead
 //     and no split or write-back runs in the row loop (about a fifth of the
@@ -32,6 +35,7 @@
 #include "kg_device.cuh"
 #include "kg_internal.h"
 #include "kg_pair.cuh"
+#include "kg_pair2.cuh"
 
 namespace kg {
 
@@ -41,7 +45,7 @@ constexpr int QP_THREADS = QP_CT;
 constexpr int QP_BAR = 1;                    // named barrier id
 
 struct QpArgs {
-  const double* A;   // FP64 rows, or (PREP) rows of float pairs (h0, l0, h1, l1, ...)
+  const double* A;   // FP64 rows, or (PREP) rows of float pairs, two entries as (h0, h1, l0, l1)
   const double* x;
   int64_t m;
   int n;  // even
@@ -103,7 +107,7 @@ __global__ void __launch_bounds__(QP_THREADS, 1) qf_pair_kernel(QpArgs a) {
 
   // ------------------------------------------------------------ consumers
   const int t = threadIdx.x;
-  float xh[PPT][2], xl[PPT][2];
+  Pair2 xp[PPT];
   bool bad = false;
 #pragma unroll
   for (int k = 0; k < PPT; ++k) {
@@ -111,20 +115,16 @@ __global__ void __launch_bounds__(QP_THREADS, 1) qf_pair_kernel(QpArgs a) {
     double2 xv = make_double2(0.0, 0.0);
     if (jp < npairs) xv = reinterpret_cast<const double2*>(a.x)[jp];
     bad |= !pair_in_range(xv.x) || !pair_in_range(xv.y);
-    const Pair p0 = split_f64(xv.x), p1 = split_f64(xv.y);
-    xh[k][0] = p0.h;
-    xl[k][0] = p0.l;
-    xh[k][1] = p1.h;
-    xl[k][1] = p1.l;
+    xp[k] = pair2_of(split_f64(xv.x), split_f64(xv.y));
   }
   const double fb = a.seed ? *a.seed : 1.0;
   if (FUSED) bad |= !pair_in_range(2.0 * fb);
   if (bad) set_error(a.err, ERRBIT_RANGE);
   const Pair fb2 = split_f64(2.0 * fb);
 
-  Acc xb[PPT][2];
+  Acc2 xb[PPT];
 #pragma unroll
-  for (int k = 0; k < PPT; ++k) xb[k][0] = xb[k][1] = acc_zero();
+  for (int k = 0; k < PPT; ++k) xb[k] = acc2_zero();
   Acc facc = acc_zero();
 
   for (int it = 0; it < nrows; ++it) {
@@ -132,29 +132,26 @@ __global__ void __launch_bounds__(QP_THREADS, 1) qf_pair_kernel(QpArgs a) {
     const bool ok = mbar_wait_bounded(&full[s], (it >> 1) & 1);
     double2* rowd = reinterpret_cast<double2*>(s ? stage1 : stage0);
     float4* rowf = reinterpret_cast<float4*>(rowd);
-    Acc yc[4] = {acc_zero(), acc_zero(), acc_zero(), acc_zero()};  // independent chains
+    Acc2 yc[2] = {acc2_zero(), acc2_zero()};  // independent chains
     if (ok) {
 #pragma unroll
       for (int k = 0; k < PPT; ++k) {
         const int jp = t + QP_CT * k;
         if (jp < npairs) {
-          Pair p0, p1;
+          Pair2 q;
           if (PREP) {
-            const float4 q = rowf[jp];
-            p0 = Pair{q.x, q.y};
-            p1 = Pair{q.z, q.w};
+            q = pair2_load(rowf + jp);
           } else {
             const double2 v = rowd[jp];
-            p0 = split_f64(v.x);
-            p1 = split_f64(v.y);
-            if (FUSED) rowf[jp] = make_float4(p0.h, p0.l, p1.h, p1.l);
+            const Pair p0 = split_f64(v.x), p1 = split_f64(v.y);
+            q = pair2_of(p0, p1);
+            if (FUSED) rowf[jp] = pair2_entry(p0, p1);
           }
-          acc_fma(yc[2 * (k & 1)], p0.h, p0.l, xh[k][0], xl[k][0]);
-          acc_fma(yc[2 * (k & 1) + 1], p1.h, p1.l, xh[k][1], xl[k][1]);
+          acc2_fma(yc[k & 1], q, xp[k]);
         }
       }
     }
-    Acc yv = acc_add(acc_add(yc[0], yc[1]), acc_add(yc[2], yc[3]));
+    Acc yv = acc_add(acc2_sum(yc[0]), acc2_sum(yc[1]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) yv = acc_add(yv, shfl_xor_acc(yv, o));
     if (lane == 0) red[(it & 1) * QP_CW + warp] = yv;
@@ -176,22 +173,15 @@ __global__ void __launch_bounds__(QP_THREADS, 1) qf_pair_kernel(QpArgs a) {
       facc = acc_add(facc, Acc{y2.h, y2.l});
     }
     if (FUSED) {
-      const Pair yb = pair_mul(fb2, y);
+      const Pair2 yb = pair2_dup(pair_mul(fb2, y));
 #pragma unroll
       for (int k = 0; k < PPT; ++k) {
         const int jp = t + QP_CT * k;
-        if (jp < npairs) {
-          const float4 q = rowf[jp];
-          acc_fma(xb[k][0], q.x, q.y, yb.h, yb.l);
-          acc_fma(xb[k][1], q.z, q.w, yb.h, yb.l);
-        }
+        if (jp < npairs) acc2_fma(xb[k], pair2_load(rowf + jp), yb);
       }
       if ((it & 15) == 15) {
 #pragma unroll
-        for (int k = 0; k < PPT; ++k) {
-          acc_renorm(xb[k][0]);
-          acc_renorm(xb[k][1]);
-        }
+        for (int k = 0; k < PPT; ++k) acc2_renorm(xb[k]);
       }
       if (!PREP) fence_proxy_async_smem();  // split values were written with generic stores
     }
@@ -225,7 +215,7 @@ __global__ void __launch_bounds__(QP_THREADS, 1) qf_pair_kernel(QpArgs a) {
     for (int k = 0; k < PPT; ++k) {
       const int jp = t + QP_CT * k;
       if (jp < npairs) {
-        const Pair p0 = acc_pair(xb[k][0]), p1 = acc_pair(xb[k][1]);
+        const Pair p0 = acc_pair(acc2_x(xb[k])), p1 = acc_pair(acc2_y(xb[k]));
         out[jp] = make_float4(p0.h, p0.l, p1.h, p1.l);
       }
     }
@@ -400,7 +390,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
   if (warp < WS_DW) {
     // ------------------------------------------------------------- dot role
     const int t = threadIdx.x;
-    float xh[KPD][2], xl[KPD][2];
+    Pair2 xp[KPD];
     bool bad = false;
 #pragma unroll
     for (int k = 0; k < KPD; ++k) {
@@ -408,11 +398,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
       double2 xv = make_double2(0.0, 0.0);
       if (jp < npairs) xv = reinterpret_cast<const double2*>(a.x)[jp];
       bad |= !pair_in_range(xv.x) || !pair_in_range(xv.y);
-      const Pair p0 = split_f64(xv.x), p1 = split_f64(xv.y);
-      xh[k][0] = p0.h;
-      xl[k][0] = p0.l;
-      xh[k][1] = p1.h;
-      xl[k][1] = p1.l;
+      xp[k] = pair2_of(split_f64(xv.x), split_f64(xv.y));
     }
     if (bad) set_error(a.err, ERRBIT_RANGE);
     for (int r = 0; r < nrows; ++r) {
@@ -427,21 +413,20 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
       }
       const float4* buf0 = slots + s0 * H;
       const float4* buf1 = slots + s1 * H;
-      Acc yc[4] = {acc_zero(), acc_zero(), acc_zero(), acc_zero()};
+      Acc2 yc[2] = {acc2_zero(), acc2_zero()};
 #pragma unroll
       for (int k = 0; k < KPD; ++k) {
         const int jp = t + TD * k;
         if (TD * (k + 1) <= 2 * H || jp < 2 * H) {  // the test is compiled for the last k only
           // which chunk: known at compile time for all k but the one whose
           // threads straddle the chunk boundary
-          const float4 q = TD * (k + 1) <= H ? buf0[jp]
-                           : TD * k >= H     ? buf1[jp - H]
-                                             : (jp < H ? buf0[jp] : buf1[jp - H]);
-          acc_fma(yc[2 * (k & 1)], q.x, q.y, xh[k][0], xl[k][0]);
-          acc_fma(yc[2 * (k & 1) + 1], q.z, q.w, xh[k][1], xl[k][1]);
+          const float4* e = TD * (k + 1) <= H ? buf0 + jp
+                            : TD * k >= H     ? buf1 + (jp - H)
+                                              : (jp < H ? buf0 + jp : buf1 + (jp - H));
+          acc2_fma(yc[k & 1], pair2_load(e), xp[k]);
         }
       }
-      Acc yv = acc_add(acc_add(yc[0], yc[1]), acc_add(yc[2], yc[3]));
+      Acc yv = acc_add(acc2_sum(yc[0]), acc2_sum(yc[1]));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) yv = acc_add(yv, shfl_xor_acc(yv, o));
       if (lane == 0) {
@@ -456,9 +441,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
     const double fb = a.seed ? *a.seed : 1.0;
     if (t == 0 && !pair_in_range(2.0 * fb)) set_error(a.err, ERRBIT_RANGE);
     const Pair fb2 = split_f64(2.0 * fb);
-    Acc xb[KP][2];
+    Acc2 xb[KP];
 #pragma unroll
-    for (int k = 0; k < KP; ++k) xb[k][0] = xb[k][1] = acc_zero();
+    for (int k = 0; k < KP; ++k) xb[k] = acc2_zero();
     Acc facc = acc_zero();
     for (int r = 0; r < nrows; ++r) {
       if (*abort_flag) break;
@@ -476,7 +461,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
         const Pair y2 = pair_mul(y, y);
         facc = acc_add(facc, Acc{y2.h, y2.l});
       }
-      const Pair yb = pair_mul(fb2, y);
+      const Pair2 yb = pair2_dup(pair_mul(fb2, y));
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const int g = 2 * r + c, slot = g % WS_SLOTS;
@@ -487,9 +472,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
 #pragma unroll
           for (int kk = 0; kk < KP / 2; ++kk) {
             const int k = c * (KP / 2) + kk;
-            const float4 q = buf[t + TU * kk];
-            acc_fma(xb[k][0], q.x, q.y, yb.h, yb.l);
-            acc_fma(xb[k][1], q.z, q.w, yb.h, yb.l);
+            acc2_fma(xb[k], pair2_load(buf + t + TU * kk), yb);
           }
         }
         __syncwarp();
@@ -502,10 +485,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
       }
       if ((r & 15) == 15) {
 #pragma unroll
-        for (int k = 0; k < KP; ++k) {
-          acc_renorm(xb[k][0]);
-          acc_renorm(xb[k][1]);
-        }
+        for (int k = 0; k < KP; ++k) acc2_renorm(xb[k]);
       }
     }
     float4* out = a.partials + (int64_t)blockIdx.x * npairs;
@@ -513,7 +493,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
     for (int k = 0; k < KP; ++k) {
       const int jp = t + TU * k;
       if (jp < npairs) {
-        const Pair p0 = acc_pair(xb[k][0]), p1 = acc_pair(xb[k][1]);
+        const Pair p0 = acc_pair(acc2_x(xb[k])), p1 = acc_pair(acc2_y(xb[k]));
         out[jp] = make_float4(p0.h, p0.l, p1.h, p1.l);
       }
     }
@@ -563,15 +543,15 @@ __global__ void __launch_bounds__(512) qf_pair_reduce_kernel(const float4* __res
   if (blockIdx.x == 0 && f) reduce_f_partials(fpart, nparts, f, fred);
 }
 
-// The prepared copy of A: every double split into its float pair (h, l).
-// count doubles; an odd count's last one is split by thread 0 of block 0.
+// The prepared copy of A: every double split into its float pair, two neighbouring
+// entries as (h0, h1, l0, l1) (an odd count's last one, by thread 0 of block 0, as (h, l)).
 __global__ void pair_prepare_kernel(const double2* __restrict__ A, float4* __restrict__ out,
                                     int64_t count) {
   const int64_t n2 = count / 2, stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += stride) {
     const double2 v = __ldcs(A + i);
     const Pair p0 = split_f64(v.x), p1 = split_f64(v.y);
-    __stcs(out + i, make_float4(p0.h, p0.l, p1.h, p1.l));
+    __stcs(out + i, pair2_entry(p0, p1));
   }
   if ((count & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
     const Pair q = split_f64(reinterpret_cast<const double*>(A)[count - 1]);

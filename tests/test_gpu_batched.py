@@ -292,3 +292,34 @@ def test_batch_tiny_and_odd_rows_through_the_ring(api, tmp_path, monkeypatch):
         assert rel_scalar(f.item(), f_ref) <= TOL["f64"]
         assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f64"]
     batch.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_batch_of_many_tiles_an_instance(api, dtype, tmp_path, monkeypatch):
+    # few instances: tiles are cut to a CTA's share of the batch, the instances of more than
+    # 16 tiles are summed by items of their own (256 columns each: one, a full one and a
+    # remainder, several), the others by their last tile; rows of odd length, one-row instances
+    monkeypatch.setenv("KG_NO_AUTOTUNE", "1")
+    td = torch.float64 if dtype == "f64" else torch.float32
+    rnd = (lambda a: a) if dtype == "f64" else f32_round
+    shapes = [(20000, 33), (4000, 257), (2500, 512), (3000, 1023), (1200, 2047), (1, 2048), (1, 1), (700, 300)]
+    probs, host, xs = [], [], []
+    for k, (m, n) in enumerate(shapes):
+        A, x = W.quadform_inputs(n, m=m, seed=50 + k)
+        A, x = rnd(A), rnd(x)
+        host.append((A, x))
+        probs.append(api.QuadForm(torch.tensor(A, dtype=td, device="cuda")))
+        xs.append(torch.tensor(x, dtype=td, device="cuda"))
+    fs = [torch.empty((), dtype=td, device="cuda") for _ in shapes]
+    gs = [torch.empty_like(x) for x in xs]
+    batch = api.Batch(probs)
+    batch.grad(xs, fs, gs)
+    first = [g.clone() for g in gs]
+    batch.grad(xs, fs, gs)
+    batch.sync()
+    for (A, x), f, g, g1 in zip(host, fs, gs, first):
+        f_ref, g_ref = O.quadform_grad(A, x)
+        assert rel_scalar(f.item(), f_ref) <= TOL[dtype], A.shape
+        assert rel_l2(g.cpu().numpy(), g_ref) <= TOL[dtype], A.shape
+        assert torch.equal(g, g1)
+    batch.close()
