@@ -166,6 +166,13 @@ int qf_pair_grid(const kg_problem* p, int* band);
 bool qf_pair_coop_fits(const kg_problem* p);
 // The same for the FP32 streamed gradient (quadform_f32.cu).
 bool qf_f32_coop_fits(const kg_problem* p);
+// ... several rows a step (quadform_pair_rows.cu)
+bool qf_pair_rows_supported(int64_t m, int64_t n, bool eval);
+int qf_pair_rows_grid(const kg_problem* p);
+bool qf_pair_rows_coop_fits(const kg_problem* p);
+kg_status qf_pair_rows_eval(kg_problem* p, const void* x, void* f, cudaStream_t s);
+kg_status qf_pair_rows_grad(kg_problem* p, const void* x, void* f, void* gx, const void* seed,
+                            int accumulate, cudaStream_t s);
 kg_status qf_pair_eval(kg_problem* p, const void* x, void* f, cudaStream_t s);
 kg_status qf_pair_grad(kg_problem* p, const void* x, void* f, void* gx, const void* seed,
                        int accumulate, cudaStream_t s);

@@ -350,7 +350,7 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
       return fail(KG_ERR_UNSUPPORTED, "QUADFORM PAIR arithmetic needs the FUSED strategy, even n "
                                       "and 1024 <= n <= 12288");
     if (shape_ok) {
-      kg_status rc = ws_common(p, num_sms(), s);
+      kg_status rc = ws_common(p, qf_pair_rows_supported(p->m, p->n, false) ? 2 * num_sms() : num_sms(), s);
       if (rc != KG_OK) return rc;
       bool in_range = false;
       if ((rc = qf_pair_range_ok(p, s, &in_range)) != KG_OK) return rc;
@@ -364,11 +364,17 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
     p->arith = KG_ARITH_PAIR;
     p->strategy = KG_STRATEGY_FUSED;
     QfConfig& c = p->qf;
-    c.grid = qf_pair_grid(p, &c.rows_per_cta);
-    c.team = c.block = 512;
-    kg_status rc = ws_alloc(p, &p->partials, 8 * (size_t)c.grid * p->n, "xbar partials (pairs)");
+    const bool rows = qf_pair_rows_supported(p->m, p->n, false);
+    c.grid = rows ? qf_pair_rows_grid(p) : qf_pair_grid(p, &c.rows_per_cta);
+    c.team = c.block = rows ? 256 : 512;
+    kg_status rc = KG_OK;
+    if (c.grid > p->fpart_len) {
+      rc = ws_alloc(p, (void**)&p->fpart, sizeof(double) * (size_t)c.grid, "f partials");
+      p->fpart_len = c.grid;
+    }
+    if (rc == KG_OK) rc = ws_alloc(p, &p->partials, 8 * (size_t)c.grid * p->n, "xbar partials (pairs)");
     if (rc == KG_OK) rc = qf_pair_prepare(p, s);
-    if (rc == KG_OK) c.coop = qf_pair_coop_fits(p) ? 1 : 0;
+    if (rc == KG_OK) c.coop = (rows ? qf_pair_rows_coop_fits(p) : qf_pair_coop_fits(p)) ? 1 : 0;
     return rc;
   }
   if (p->arith == KG_ARITH_AUTO || p->dtype == KG_F32) p->arith = KG_ARITH_NATIVE;

@@ -22,6 +22,8 @@
 //     instructions per entry);
 //   - the private xbar partials (float pairs) of each CTA go to a workspace that
 //     a second kernel sums in a fixed order: bitwise reproducible.
+// Rows of up to 4096 entries (the forward: 8192) run the kernels of quadform_pair_rows.cu,
+// those of more than 2048 when the matrix has enough of them.
 // For 2048 < n <= 10240 on the prepared A the fused pass runs qf_pair_ws_kernel
 // instead, with dot-product, update and copy roles in separate warps (described
 // at the kernel); the forward and all other shapes use qf_pair_kernel.
@@ -576,7 +578,7 @@ __global__ void pair_range_scan_kernel(const double2* __restrict__ p, int64_t co
 // ---------------------------------------------------------------- host ----
 static int pair_ppt(int64_t n) {
   const int64_t need = (n / 2 + QP_CT - 1) / QP_CT;
-  for (int p : {1, 2, 4, 6, 8, 10, 12})
+  for (int p : {4, 6, 8, 10, 12})
     if (need <= p) return p;
   return -1;
 }
@@ -633,8 +635,6 @@ static cudaError_t launch_pair(int grid, size_t smem, cudaStream_t s, const QpAr
 template <bool FUSED, bool PREP>
 static cudaError_t dispatch_ppt(int ppt, int grid, size_t smem, cudaStream_t s, const QpArgs& a) {
   switch (ppt) {
-    case 1: return launch_pair<1, FUSED, PREP>(grid, smem, s, a);
-    case 2: return launch_pair<2, FUSED, PREP>(grid, smem, s, a);
     case 4: return launch_pair<4, FUSED, PREP>(grid, smem, s, a);
     case 6: return launch_pair<6, FUSED, PREP>(grid, smem, s, a);
     case 8: return launch_pair<8, FUSED, PREP>(grid, smem, s, a);
@@ -689,6 +689,7 @@ static QpArgs pair_args(kg_problem* p, const void* x, const void* seed) {
 kg_status qf_pair_eval(kg_problem* p, const void* x, void* f, cudaStream_t s) {
   if ((reinterpret_cast<uintptr_t>(x) & 15u) != 0)
     return fail(KG_ERR_INVALID_ARG, "QUADFORM pair kernels need a 16-byte aligned x");
+  if (qf_pair_rows_supported(p->m, p->n, true)) return qf_pair_rows_eval(p, x, f, s);
   QpArgs a = pair_args(p, x, nullptr);
   a.f = static_cast<double*>(f);
   prof_begin(s, p->aprep ? "qf_pair_kernel<eval, prepared A>" : "qf_pair_kernel<eval>");
@@ -778,6 +779,7 @@ kg_status qf_pair_grad(kg_problem* p, const void* x, void* f, void* gx, const vo
                        int accumulate, cudaStream_t s) {
   if ((reinterpret_cast<uintptr_t>(x) & 15u) != 0 || (reinterpret_cast<uintptr_t>(gx) & 15u) != 0)
     return fail(KG_ERR_INVALID_ARG, "QUADFORM pair kernels need 16-byte aligned x and gx");
+  if (qf_pair_rows_supported(p->m, p->n, false)) return qf_pair_rows_grad(p, x, f, gx, seed, accumulate, s);
   QpArgs a = pair_args(p, x, seed);
   const int kp = ws_kp(p);
   cudaError_t e;

@@ -78,3 +78,40 @@ def test_infinite_x_and_ragged_row_group(api, m, n):
     p.sync()
     assert f.item() == np.inf and bool((g == np.inf).all())
     p.close()
+
+
+@pytest.mark.parametrize("m,n", [(1, 1024), (3, 1026), (4, 1536), (5, 1538), (1217, 2046), (1300, 2048), (9001, 1500),
+                                 (611, 2050), (700, 2562), (1001, 3074), (613, 3586), (1216, 4096), (609, 4098),
+                                 (615, 5122), (700, 6146), (801, 7170), (608, 8192)])
+def test_float_pair_rows_paths_agree_bitwise(api, m, n, monkeypatch):
+    # float pairs, several rows a step: every width of a thread, ragged steps of four or two
+    # rows, one and many CTAs; prepared and per-load split, one launch and two (also taken by
+    # grids of up to 64 CTAs), give the same bits
+    from paper_2507_13204_gb300 import _lib as L
+    A, x = W.quadform_inputs(n, m=m, seed=2 * m + n)
+    f_ref, g_ref = O.quadform_grad(A, x, fbar=0.5)
+    At, xt = torch.tensor(A, device="cuda"), torch.tensor(x, device="cuda")
+    seed = torch.tensor(0.5, dtype=torch.float64, device="cuda")
+    out = []
+    for coop, budget in ((1, 0), (0, 0), (1, 8)):  # a budget of 8 bytes: no prepared copy
+        if coop:
+            monkeypatch.delenv("KG_TEST_NO_COOP", raising=False)
+        else:
+            monkeypatch.setenv("KG_TEST_NO_COOP", "1")
+        p = api.QuadForm(At, tape_budget_bytes=budget)
+        assert p.config == ("fused", "recompute", "pair")
+        f, g = p.grad(xt, seed=seed)
+        assert L.kg_last_launch_count() == (1 if coop and m > 256 else 2) or budget and n > 4096
+        g2 = torch.full_like(g, 0.25)
+        p.grad(xt, gx=g2, seed=seed, accumulate=True)
+        fe = p.eval(xt)
+        p.sync()
+        out.append((f.item(), g.cpu().numpy(), g2.cpu().numpy(), fe.item()))
+        p.close()
+    f, g, g2, fe = out[0]
+    assert rel_scalar(f, f_ref) <= TOL["f64"] and rel_scalar(fe, f_ref) <= TOL["f64"]
+    assert rel_l2(g, g_ref) <= TOL["f64"] and np.array_equal(g2, 0.25 + g)
+    for o in out[1:]:
+        assert o[3] == fe
+        if n <= 4096 or o is out[1]:  # (longer rows: the per-load split's gradient is another kernel)
+            assert o[0] == f and np.array_equal(o[1], g) and np.array_equal(o[2], g2)
