@@ -155,3 +155,37 @@ def test_checkpoint_resume_reproduces_the_uninterrupted_run(mods, tmp_path):
                                   every=3, resume=True)
     assert torch.equal(full, resumed)
     assert torch.load(ck)["step"] == 9
+
+
+@pytest.mark.parametrize("strategy", ["atomic", "warp", "tile", "csr", "shared"])
+@pytest.mark.parametrize("mode,policy", [("tape", "tape"), ("tape", "auto"), ("recompute", "auto"),
+                                         ("tape", "recompute")])
+def test_descent_direct_steps_match_autograd_steps(mods, strategy, mode, policy):
+    # the descent's direct calls against the same loop through KGTetEnergy: value and
+    # trajectory to the parity bound over three steps; u0 is left alone; policy "tape" without a
+    # tape and a gradient whose shape autograd refuses are refused as before
+    api, ag = mods
+    mesh = W.tet_mesh(5, jitter_seed=2, perm_seed=4)
+    p = _tet(api, mesh, strategy=strategy, mode=mode)
+    u0 = torch.tensor(np.random.default_rng(3).uniform(-1, 1, mesh.nv), device="cuda")
+    keep = u0.clone()
+    hist = []
+    got = ag.gradient_descent(p, u0, ETA, 3, policy=policy, history=hist)
+    u, ref = u0.clone(), []
+    for _ in range(3):
+        ut = u.clone().requires_grad_(True)
+        f = ag.KGTetEnergy.apply(ut, p, policy)
+        (g,) = torch.autograd.grad(f, ut)
+        ref.append(f.item())
+        u = u - ETA * g
+    assert torch.equal(u0, keep) and not got.requires_grad
+    assert rel_l2(got.cpu().numpy(), u.cpu().numpy()) <= TOL["f64"]
+    assert [h.shape for h in hist] == [torch.Size([])] * 3
+    assert max(rel_scalar(h.item(), r) for h, r in zip(hist, ref)) <= TOL["f64"]
+    if mode == "recompute":
+        with pytest.raises(ValueError):
+            ag.gradient_descent(p, u0, ETA, 1, policy="tape")
+    with pytest.raises(RuntimeError):
+        ag.gradient_descent(p, u0.view(-1, 1), ETA, 1, policy=policy)
+    with torch.no_grad(), pytest.raises(RuntimeError):
+        ag.gradient_descent(p, u0, ETA, 1, policy=policy)
