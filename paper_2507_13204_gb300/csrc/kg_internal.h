@@ -103,6 +103,7 @@ struct kg_problem {
   kg::QfConfig qf;           // dense launch configuration
   int tet_block = 256, tet_grid = 1;
   int sq_team = 8, sq_col_team = 8;  // sparse: lanes per row team / per column team
+  int sq_stream = 0;         // sparse: lanes per row of the row-block kernels (spquad_stream.cu); 0: row teams
   cudaStream_t last_stream = nullptr;
 };
 
@@ -227,6 +228,17 @@ void scan_exclusive(int* data, int n, cudaStream_t s);
 // Buckets of positions by key (transposed index lists; tet.cu), synchronises s.
 kg_status build_buckets(const int* keys, int64_t count, int nbins, int* binptr, int* perm,
                         cudaStream_t s);
+
+// row passes of the sparse ||A x||^2 by blocks of rows (spquad_stream.cu)
+struct SpqStreamCall {
+  const void *x, *seed;
+  void *f, *gx, *gval;
+  int accumulate;
+};
+int spq_stream_team(double avg);
+bool spq_stream_takes(const kg_problem* p, int mode, bool gval);
+int spq_stream_grid(int64_t m, int tw);
+cudaError_t spq_stream(const kg_problem* p, int mode, const SpqStreamCall& c, cudaStream_t s);
 
 // sparse ||A x||^2 (spquadform.cu)
 kg_status spq_setup(kg_problem* p, cudaStream_t s);

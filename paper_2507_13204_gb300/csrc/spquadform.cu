@@ -6,6 +6,8 @@
 // of x through the index map col becomes a scatter-add xbar[col[p]] += val[p]
 // ybar_i (Sec. 3.3), and valbar[p] = x[col[p]] ybar_i.
 //
+// Most row passes run a block of rows at a time (spquad_stream.cu); the kernels
+// here serve a caller's own team width, long rows and FP32 forwards and row passes.
 // A team of TW lanes works on one row (32 / TW rows per warp, grid-stride over
 // row groups so that every lane of a warp runs the same iterations); the team
 // reduces its row sum with xor shuffles, a fixed order.
@@ -401,7 +403,8 @@ kg_status spq_setup(kg_problem* p, cudaStream_t s) {
   const double cover = p->dtype == KG_F32 ? 0.5 : 1.5;
   p->sq_team = team_for((double)p->nnz / (double)p->m, t, cover);
   p->sq_col_team = team_for((double)p->nnz / (double)p->n, t, cover);
-  const int grid = sq_grid(p->m, p->sq_team);
+  if (!t) p->sq_stream = spq_stream_team((double)p->nnz / (double)p->m);  // a given team: row teams
+  const int grid = std::max(sq_grid(p->m, p->sq_team), p->sq_stream ? spq_stream_grid(p->m, p->sq_stream) : 0);
   kg_status rc = ws_common(p, grid, s);
   if (rc != KG_OK) return rc;
   const int* rowptr = static_cast<const int*>(p->data0);
@@ -478,6 +481,8 @@ kg_status spq_setup(kg_problem* p, cudaStream_t s) {
 
 template <typename T, int MODE>
 static cudaError_t launch_row(const kg_problem* p, const SqArgs<T>& a, cudaStream_t s) {
+  if (spq_stream_takes(p, MODE, a.gval != nullptr))
+    return spq_stream(p, MODE, SpqStreamCall{a.x, a.seed, a.f, a.gx, a.gval, a.accumulate}, s);
   const int g = sq_grid(p->m, p->sq_team);
   switch (p->sq_team) {
     case 2: spq_row_kernel<T, 2, MODE><<<g, SQ_THREADS, 0, s>>>(a); break;
@@ -508,6 +513,8 @@ static cudaError_t launch_col(const kg_problem* p, const T* y, const T* seed, T*
 
 template <int MODE>
 static cudaError_t launch_row_pair(const kg_problem* p, const SqPairArgs& a, cudaStream_t s) {
+  if (spq_stream_takes(p, MODE, a.gval != nullptr))
+    return spq_stream(p, MODE, SpqStreamCall{a.x, a.seed, a.f, a.gx, a.gval, a.accumulate}, s);
   const int g = sq_grid(p->m, p->sq_team);
   switch (p->sq_team) {
     case 2: spq_row_pair_kernel<2, MODE><<<g, SQ_THREADS, 0, s>>>(a); break;

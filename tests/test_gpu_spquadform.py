@@ -190,3 +190,52 @@ def test_full_size_workload_f64(api):
         assert rel_scalar(f.item(), f_ref) <= TOL["f64"], strategy
         assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f64"], strategy
         p.close()
+
+
+def _csr_of_degrees(deg, n, seed):
+    rng = np.random.default_rng(seed)
+    rowptr = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
+    nnz = int(rowptr[-1])
+    return W.CsrMatrix(rowptr, rng.integers(0, n, nnz).astype(np.int32), rng.standard_normal(nnz), len(deg), n)
+
+
+# Row blocks: 256 / TW rows, TW the power of two with 2.4 to 4.8 entries a lane; at most 1536
+# entries in a block, longer ones by a warp per row
+BLOCKS = {
+    "capacity": [48] * 32 + [48] * 31 + [49] + [0] * 30 + [3, 97] + [1] * 5,  # 1536, 1537, ragged last block
+    "tw1": [3] * 300 + [0] * 7, "tw2": [9] * 200, "tw4": [17] * 131, "tw16": [70] * 33 + [0, 1, 140],
+    "tw32": [150] * 19 + [192] * 8 + [1, 0], "row teams": [300, 1, 170],
+    "one long row": [2] * 500 + [4000] + [2] * 500,
+}
+
+
+@pytest.mark.parametrize("name", sorted(BLOCKS))
+@pytest.mark.parametrize("kind", ["pair", "native", "f32"])
+@pytest.mark.parametrize("strategy", ["atomic", "transpose"])
+def test_row_blocks(api, name, kind, strategy):
+    A = _csr_of_degrees(BLOCKS[name], 211, seed=len(name))
+    x = np.random.default_rng(5).uniform(-1, 1, A.n)
+    dt = torch.float32 if kind == "f32" else torch.float64
+    tol = TOL["f32" if kind == "f32" else "f64"]
+    if kind == "f32":
+        A.val, x = f32_round(A.val), f32_round(x)
+    f_ref, g_ref, gv_ref = O.spquadform_grad(A.rowptr, A.col, A.val, x, fbar=0.5, want_gval=True)
+    p = _problem(api, A, dt, strategy=strategy, arith="auto" if kind == "f32" else kind)
+    xt = torch.tensor(x, dtype=dt, device="cuda")
+    seed = torch.tensor(0.5, dtype=dt, device="cuda")
+    gv = torch.full((A.nnz,), 0.25, dtype=dt, device="cuda")
+    f, g = p.grad(xt, gdata=gv, seed=seed, accumulate=False)
+    f2, g2 = p.grad(xt, gdata=gv, gx=g.clone(), seed=seed, accumulate=True)
+    fe = p.eval(xt)
+    p.sync()
+    for v in (f, f2, fe):
+        assert rel_scalar(v.item(), f_ref) <= tol
+    assert rel_l2(g.cpu().numpy(), g_ref) <= tol
+    assert rel_l2(g2.cpu().numpy(), 2 * g_ref) <= tol
+    assert rel_l2(gv.cpu().numpy(), 2 * gv_ref) <= tol
+    if strategy == "transpose":
+        g3 = p.grad(xt, gdata=gv, seed=seed)[1].clone()
+        assert torch.equal(f, f2) and torch.equal(g3, g)
+        g4, g5 = p.grad(xt, seed=seed)[1].clone(), p.grad(xt, seed=seed)[1]
+        assert torch.equal(g4, g5) and rel_l2(g4.cpu().numpy(), g_ref) <= tol
+    p.close()
