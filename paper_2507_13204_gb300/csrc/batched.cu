@@ -512,26 +512,24 @@ __device__ double tet_tile(const BInst& I, const BItem& w, const float4* tab, co
   const T* G = static_cast<const T*>(I.d1);
   const T* u = static_cast<const T*>(I.x);
   T* gu = static_cast<T*>(I.gx);
-  Acc fp = acc_zero();
+  LogSum lsum = log_sum_zero();
   T fn = T(0);
   const int64_t e1 = w.start + w.count;
-  int cnt = 0;
   if constexpr (!WARPC) {  // one atomic per contribution
-    for (int64_t e = w.start + tid; e < e1; e += BT, ++cnt) {
+    for (int64_t e = w.start + tid; e < e1; e += BT) {
       const int4 c = __ldcs(conn + e);
       if constexpr (PAIR) {
         elem_pair<TS_GRAD, AtomicSink<double>, PREP>(
             c, reinterpret_cast<const double*>(G) + e * 12, reinterpret_cast<const double*>(u),
-            Pair{2.0f, 0.0f}, tab, K, fp, AtomicSink<double>{reinterpret_cast<double*>(gu)}, nullptr,
+            Pair{2.0f, 0.0f}, tab, K, lsum, AtomicSink<double>{reinterpret_cast<double*>(gu)}, nullptr,
             bad);
-        if ((cnt & 31) == 31) acc_renorm(fp);
       } else {
         elem_native<T, TS_GRAD>(c, G + e * 12, u, T(1), fn, AtomicSink<T>{gu}, nullptr);
       }
     }
   }
   // WARPC: block-uniform loop, so that every lane reaches the warp-level combine
-  for (int64_t e0 = w.start; WARPC && e0 < e1; e0 += BT, ++cnt) {
+  for (int64_t e0 = w.start; WARPC && e0 < e1; e0 += BT) {
     const int64_t e = e0 + tid;
     const bool act = e < e1;
     T cv[4];
@@ -542,8 +540,7 @@ __device__ double tet_tile(const BInst& I, const BItem& w, const float4* tab, co
       if constexpr (PAIR) {
         elem_pair<TS_GRAD, CollectSink<T>, PREP>(
             c, reinterpret_cast<const double*>(G) + e * 12, reinterpret_cast<const double*>(u),
-            Pair{2.0f, 0.0f}, tab, K, fp, CollectSink<T>{cv, cpr}, nullptr, bad);
-        if ((cnt & 31) == 31) acc_renorm(fp);
+            Pair{2.0f, 0.0f}, tab, K, lsum, CollectSink<T>{cv, cpr}, nullptr, bad);
       } else {
         elem_native<T, TS_GRAD>(c, G + e * 12, u, T(1), fn, CollectSink<T>{cv, cpr}, nullptr);
       }
@@ -565,6 +562,7 @@ __device__ double tet_tile(const BInst& I, const BItem& w, const float4* tab, co
   }
   __syncthreads();
   if constexpr (PAIR) {
+    Acc fp = log_sum_get(lsum, tab, K);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) fp = acc_add(fp, shfl_xor_acc2(fp, o));
     Acc* ra = reinterpret_cast<Acc*>(red);

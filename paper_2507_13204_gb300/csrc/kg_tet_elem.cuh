@@ -17,6 +17,7 @@
 
 #include "kg_device.cuh"
 #include "kg_pair.cuh"
+#include "kg_pair2.cuh"
 
 namespace kg {
 
@@ -213,84 +214,126 @@ __device__ __forceinline__ void elem_native(const int4 c, const T* __restrict__ 
   }
 }
 
-// The arithmetic of one element in float pairs, from its G_e (12 pairs) and
-// gathered vertex values U (4 pairs): g = G_e u_e, f_e = log1p(|g|^2) added to
-// facc, and (MODE != TS_EVAL) the element adjoint
-// cp[k] = (G_e^T (2 fbar g / (1 + |g|^2)))_k, with fb2 = 2 fbar as a pair.
+// Sum of log1p(s_e) over a thread's elements, s_e >= 0 as normalised pairs.  The elements'
+// factors are multiplied, (1 + q)(1 + s) = 1 + (q + s + q s), with q kept instead of 1 + q so
+// that small values keep their relative accuracy, and one log1p(q) is taken for eight of
+// them: 29 FP32 operations an element instead of log1p's 130.  A factor above 2^30 is not
+// multiplied on, so q stays below 2^61 + 2^31 for every s that is.
+struct LogSum {
+  Acc f;
+  Pair q;
+  int n;
+};
+
+__device__ __forceinline__ LogSum log_sum_zero() { return LogSum{acc_zero(), Pair{0.f, 0.f}, 0}; }
+
+__device__ __forceinline__ void log_sum_flush(LogSum& L, const float4* __restrict__ tab, const LogConsts& K) {
+  Pair t;
+  const Pair lf = pair_log1p(L.q, tab, K, t);
+  L.f = acc_add(L.f, Acc{lf.h, lf.l});
+  acc_renorm(L.f);
+}
+
+__device__ __forceinline__ void log_sum_add(LogSum& L, Pair s, const float4* __restrict__ tab, const LogConsts& K) {
+  constexpr float kBig = 1073741824.0f;  // 2^30
+  if ((++L.n & 7) == 0 || s.h > kBig || L.q.h > kBig) {
+    log_sum_flush(L, tab, K);
+    L.q = s;
+  } else {
+    L.q = pair_add(pair_add(L.q, s), pair_mul(L.q, s));
+  }
+}
+
+// The thread's sum (call once, after its last element).
+__device__ __forceinline__ Acc log_sum_get(LogSum& L, const float4* __restrict__ tab, const LogConsts& K) {
+  log_sum_flush(L, tab, K);
+  return L.f;
+}
+
+// The arithmetic of one element in float pairs, from its G_e (row r: G[2r] holds columns 0
+// and 1, G[2r + 1] columns 2 and 3) and gathered vertex values (U[0]: 0 and 1, U[1]: 2 and 3):
+// g = G_e u_e, f_e = log1p(|g|^2) added to L, and (MODE != TS_EVAL) the element adjoint
+// cp = G_e^T (2 fbar g / (1 + |g|^2)), with fb2 = 2 fbar as a pair.  Two columns at a time in
+// packed instructions.
 template <int MODE>
-__device__ __forceinline__ void elem_pair_core(const Pair (&G)[12], const Pair (&U)[4], Pair fb2,
+__device__ __forceinline__ void elem_pair_core(const Pair2 (&G)[6], const Pair2 (&U)[2], Pair fb2,
                                                const float4* __restrict__ tab, const LogConsts& K,
-                                               Acc& facc, Pair (&cp)[4]) {
+                                               LogSum& L, Pair (&cp)[4]) {
   Pair g[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    Acc a = acc_prod(G[4 * r].h, G[4 * r].l, U[0].h, U[0].l);
-#pragma unroll
-    for (int k = 1; k < 4; ++k) acc_fma(a, G[4 * r + k].h, G[4 * r + k].l, U[k].h, U[k].l);
-    g[r] = acc_pair(a);
+    Acc2 a = acc2_prod(G[2 * r], U[0]);
+    acc2_fma(a, G[2 * r + 1], U[1]);
+    g[r] = acc_pair(acc2_sum(a));
   }
-  Acc sa = acc_prod(g[0].h, g[0].l, g[0].h, g[0].l);
-#pragma unroll
-  for (int r = 1; r < 3; ++r) acc_fma(sa, g[r].h, g[r].l, g[r].h, g[r].l);
+  const Pair2 g01 = pair2_of(g[0], g[1]);
+  Acc sa = acc2_sum(acc2_prod(g01, g01));
+  acc_fma(sa, g[2].h, g[2].l, g[2].h, g[2].l);
   const Pair s = acc_pair(sa);
-  Pair t;
-  const Pair lf = pair_log1p(s, tab, K, t);
-  facc = acc_add(facc, Acc{lf.h, lf.l});
+  log_sum_add(L, s, tab, K);
   if constexpr (MODE != TS_EVAL) {
+    Pair t;  // 1 + s, normalised
+    two_sum(1.0f, s.h, t.h, t.l);
+    t.l += s.l;
+    fast_two_sum(t.h, t.l, t.h, t.l);
     const Pair w = pair_mul(fb2, pair_recip(t));
-    Pair wg[3];
+    const Pair2 w01 = pair2_mul(pair2_dup(w), g01);
+    const Pair2 wg[3] = {pair2_dup(pair2_x(w01)), pair2_dup(pair2_y(w01)), pair2_dup(pair_mul(w, g[2]))};
 #pragma unroll
-    for (int r = 0; r < 3; ++r) wg[r] = pair_mul(w, g[r]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      Acc a = acc_prod(G[k].h, G[k].l, wg[0].h, wg[0].l);
-#pragma unroll
-      for (int r = 1; r < 3; ++r) acc_fma(a, G[4 * r + k].h, G[4 * r + k].l, wg[r].h, wg[r].l);
-      cp[k] = acc_pair(a);
+    for (int h = 0; h < 2; ++h) {
+      Acc2 a = acc2_prod(G[h], wg[0]);
+      acc2_fma(a, G[2 + h], wg[1]);
+      acc2_fma(a, G[4 + h], wg[2]);
+      const Pair2 c = acc2_pair(a);
+      cp[2 * h] = pair2_x(c);
+      cp[2 * h + 1] = pair2_y(c);
     }
   }
 }
 
-// One element in float-pair arithmetic (FP64 data).  Gs points at the
-// element's 12 doubles, or (PREP) at its 12 float pairs prepared once, two as (h0, h1, l0, l1).
-// USPLIT: u points at float pairs of the vertex values, split (and range
-// checked) once per call by pair_split_vec instead of once per gather.
+// G_e (Gs: 12 doubles, or with PREP the 12 float pairs prepared once, two as (h0, h1, l0, l1)).
+template <bool PREP>
+__device__ __forceinline__ void elem_pair_load_G(const double* __restrict__ Gs, Pair2 (&G)[6]) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    if constexpr (PREP) {
+      G[i] = pair2_load(reinterpret_cast<const float4*>(Gs) + i);
+    } else {
+      const double2 v = reinterpret_cast<const double2*>(Gs)[i];
+      G[i] = pair2_of(split_f64(v.x), split_f64(v.y));
+    }
+  }
+}
+
+// The element's vertex values (USPLIT: u points at float pairs split and range checked once
+// per call, instead of once per gather here).
+template <bool USPLIT>
+__device__ __forceinline__ void elem_pair_load_u(const int4 c, const double* __restrict__ u, Pair2 (&U)[2],
+                                                 bool& bad) {
+  if constexpr (USPLIT) {
+    const float2* up = reinterpret_cast<const float2*>(u);
+    const float2 q0 = __ldg(up + c.x), q1 = __ldg(up + c.y), q2 = __ldg(up + c.z), q3 = __ldg(up + c.w);
+    U[0] = Pair2{f2(q0.x, q1.x), f2(q0.y, q1.y)};
+    U[1] = Pair2{f2(q2.x, q3.x), f2(q2.y, q3.y)};
+  } else {
+    const double u0 = __ldg(u + c.x), u1 = __ldg(u + c.y), u2 = __ldg(u + c.z), u3 = __ldg(u + c.w);
+    bad |= !pair_in_range(u0) || !pair_in_range(u1) || !pair_in_range(u2) || !pair_in_range(u3);
+    U[0] = pair2_of(split_f64(u0), split_f64(u1));
+    U[1] = pair2_of(split_f64(u2), split_f64(u3));
+  }
+}
+
+// One element in float-pair arithmetic (FP64 data).
 template <int MODE, typename Sink, bool PREP = false, bool USPLIT = false>
 __device__ __forceinline__ void elem_pair(const int4 c, const double* __restrict__ Gs,
                                           const double* __restrict__ u, Pair fb2,
                                           const float4* __restrict__ tab, const LogConsts& K,
-                                          Acc& facc, const Sink& gu, double* tape_e, bool& bad) {
-  Pair G[12];
-#pragma unroll
-  for (int i = 0; i < 12; i += 2) {
-    if constexpr (PREP) {
-      const float4 q = *reinterpret_cast<const float4*>(Gs + i);
-      G[i] = Pair{q.x, q.z};
-      G[i + 1] = Pair{q.y, q.w};
-    } else {
-      const double2 v = *reinterpret_cast<const double2*>(Gs + i);
-      G[i] = split_f64(v.x);
-      G[i + 1] = split_f64(v.y);
-    }
-  }
-  Pair U[4];
-  if constexpr (USPLIT) {
-    const float2* up = reinterpret_cast<const float2*>(u);
-    const float2 q0 = __ldg(up + c.x), q1 = __ldg(up + c.y), q2 = __ldg(up + c.z), q3 = __ldg(up + c.w);
-    U[0] = Pair{q0.x, q0.y};
-    U[1] = Pair{q1.x, q1.y};
-    U[2] = Pair{q2.x, q2.y};
-    U[3] = Pair{q3.x, q3.y};
-  } else {
-    const double ud[4] = {__ldg(u + c.x), __ldg(u + c.y), __ldg(u + c.z), __ldg(u + c.w)};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      bad |= !pair_in_range(ud[k]);
-      U[k] = split_f64(ud[k]);
-    }
-  }
+                                          LogSum& L, const Sink& gu, double* tape_e, bool& bad) {
+  Pair2 G[6], U[2];
+  elem_pair_load_G<PREP>(Gs, G);
+  elem_pair_load_u<USPLIT>(c, u, U, bad);
   Pair cp[4];
-  elem_pair_core<MODE>(G, U, fb2, tab, K, facc, cp);
+  elem_pair_core<MODE>(G, U, fb2, tab, K, L, cp);
   if constexpr (MODE != TS_EVAL) {
     if constexpr (MODE == TS_GRAD) {
       sink_pair(gu, 0, c.x, cp[0]);
@@ -342,30 +385,23 @@ __device__ __forceinline__ void elem_native_hvp(const int4 c, const T* __restric
 
 // The Hessian-vector arithmetic of one element in float pairs, from its G_e
 // and the gathered U (point) and V (direction): hc[k] = (G_e^T (wd g + w gd))_k.
-__device__ __forceinline__ void elem_pair_hvp_core(const Pair (&G)[12], const Pair (&U)[4],
-                                                   const Pair (&V)[4], Pair fb2, Pair (&hc)[4]) {
+__device__ __forceinline__ void elem_pair_hvp_core(const Pair2 (&G)[6], const Pair2 (&U)[2],
+                                                   const Pair2 (&V)[2], Pair fb2, Pair (&hc)[4]) {
   Pair g[3], gd[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    Acc a = acc_prod(G[4 * r].h, G[4 * r].l, U[0].h, U[0].l);
-    Acc b = acc_prod(G[4 * r].h, G[4 * r].l, V[0].h, V[0].l);
-#pragma unroll
-    for (int k = 1; k < 4; ++k) {
-      acc_fma(a, G[4 * r + k].h, G[4 * r + k].l, U[k].h, U[k].l);
-      acc_fma(b, G[4 * r + k].h, G[4 * r + k].l, V[k].h, V[k].l);
-    }
-    g[r] = acc_pair(a);
-    gd[r] = acc_pair(b);
+    Acc2 a = acc2_prod(G[2 * r], U[0]), b = acc2_prod(G[2 * r], V[0]);
+    acc2_fma(a, G[2 * r + 1], U[1]);
+    acc2_fma(b, G[2 * r + 1], V[1]);
+    g[r] = acc_pair(acc2_sum(a));
+    gd[r] = acc_pair(acc2_sum(b));
   }
-  Acc sa = acc_prod(g[0].h, g[0].l, g[0].h, g[0].l);
-  Acc sda = acc_prod(g[0].h, g[0].l, gd[0].h, gd[0].l);
+  // s = |g|^2 and g . gd, one on each half
+  Acc2 sa = acc2_prod(pair2_dup(g[0]), pair2_of(g[0], gd[0]));
 #pragma unroll
-  for (int r = 1; r < 3; ++r) {
-    acc_fma(sa, g[r].h, g[r].l, g[r].h, g[r].l);
-    acc_fma(sda, g[r].h, g[r].l, gd[r].h, gd[r].l);
-  }
-  const Pair s = acc_pair(sa);
-  Pair sd = acc_pair(sda);
+  for (int r = 1; r < 3; ++r) acc2_fma(sa, pair2_dup(g[r]), pair2_of(g[r], gd[r]));
+  const Pair s = acc_pair(acc2_x(sa));
+  Pair sd = acc_pair(acc2_y(sa));
   sd.h *= 2.0f;  // exact
   sd.l *= 2.0f;
   const Pair rt = pair_recip(pair_add(Pair{1.0f, 0.0f}, s));
@@ -373,15 +409,20 @@ __device__ __forceinline__ void elem_pair_hvp_core(const Pair (&G)[12], const Pa
   Pair wd = pair_mul(pair_mul(w, sd), rt);
   wd.h = -wd.h;
   wd.l = -wd.l;
-  Pair h[3];
+  Pair2 h[3];
 #pragma unroll
-  for (int r = 0; r < 3; ++r) h[r] = pair_add(pair_mul(wd, g[r]), pair_mul(w, gd[r]));
+  for (int r = 0; r < 3; ++r) {
+    const Pair2 m = pair2_mul(pair2_of(wd, w), pair2_of(g[r], gd[r]));
+    h[r] = pair2_dup(pair_add(pair2_x(m), pair2_y(m)));
+  }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    Acc a = acc_prod(G[k].h, G[k].l, h[0].h, h[0].l);
-#pragma unroll
-    for (int r = 1; r < 3; ++r) acc_fma(a, G[4 * r + k].h, G[4 * r + k].l, h[r].h, h[r].l);
-    hc[k] = acc_pair(a);
+  for (int c = 0; c < 2; ++c) {
+    Acc2 a = acc2_prod(G[c], h[0]);
+    acc2_fma(a, G[2 + c], h[1]);
+    acc2_fma(a, G[4 + c], h[2]);
+    const Pair2 q = acc2_pair(a);
+    hc[2 * c] = pair2_x(q);
+    hc[2 * c + 1] = pair2_y(q);
   }
 }
 
@@ -391,39 +432,16 @@ __device__ __forceinline__ void elem_pair_hvp(const int4 c, const double* __rest
                                               const double* __restrict__ u,
                                               const double* __restrict__ v, Pair fb2,
                                               const Sink& gu, bool& bad) {
-  Pair G[12];
-#pragma unroll
-  for (int i = 0; i < 12; i += 2) {
-    if constexpr (PREP) {
-      const float4 q = *reinterpret_cast<const float4*>(Gs + i);
-      G[i] = Pair{q.x, q.z};
-      G[i + 1] = Pair{q.y, q.w};
-    } else {
-      const double2 q = *reinterpret_cast<const double2*>(Gs + i);
-      G[i] = split_f64(q.x);
-      G[i + 1] = split_f64(q.y);
-    }
-  }
-  const int idx[4] = {c.x, c.y, c.z, c.w};
-  Pair U[4], V[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    if constexpr (USPLIT) {
-      const float2 qu = __ldg(reinterpret_cast<const float2*>(u) + idx[k]);
-      const float2 qv = __ldg(reinterpret_cast<const float2*>(v) + idx[k]);
-      U[k] = Pair{qu.x, qu.y};
-      V[k] = Pair{qv.x, qv.y};
-    } else {
-      const double uk = __ldg(u + idx[k]), vk = __ldg(v + idx[k]);
-      bad |= !pair_in_range(uk) || !pair_in_range(vk);
-      U[k] = split_f64(uk);
-      V[k] = split_f64(vk);
-    }
-  }
+  Pair2 G[6], U[2], V[2];
+  elem_pair_load_G<PREP>(Gs, G);
+  elem_pair_load_u<USPLIT>(c, u, U, bad);
+  elem_pair_load_u<USPLIT>(c, v, V, bad);
   Pair hc[4];
   elem_pair_hvp_core(G, U, V, fb2, hc);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) sink_pair(gu, k, idx[k], hc[k]);
+  sink_pair(gu, 0, c.x, hc[0]);
+  sink_pair(gu, 1, c.y, hc[1]);
+  sink_pair(gu, 2, c.z, hc[2]);
+  sink_pair(gu, 3, c.w, hc[3]);
 }
 
 }  // namespace kg

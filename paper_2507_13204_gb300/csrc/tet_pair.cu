@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(TS_THREADS) tet_staged_kernel(TsArgs<T> a) {
   }
 
   T facc_n = T(0);
-  Acc facc_p = acc_zero();
+  LogSum lsum = log_sum_zero();
   bool bad = false;
   const T fb = REV ? load_seed(a.seed) : T(1);
   Pair fb2{2.0f, 0.0f};
@@ -198,9 +198,8 @@ __global__ void __launch_bounds__(TS_THREADS) tet_staged_kernel(TsArgs<T> a) {
           } else if constexpr (PAIR) {
             elem_pair<MODE, std::decay_t<decltype(sink)>, PREP, MODE == TS_GRAD>(
                             c, reinterpret_cast<const double*>(Gs),
-                            reinterpret_cast<const double*>(a.u), fb2, tab, a.K, facc_p, sink,
+                            reinterpret_cast<const double*>(a.u), fb2, tab, a.K, lsum, sink,
                             reinterpret_cast<double*>(a.tape) + e * 4, bad);
-            if ((i & 31) == 31) acc_renorm(facc_p);
           } else {
             elem_native<T, MODE>(c, Gs, a.u, fb, facc_n, sink, a.tape + e * 4);
           }
@@ -264,6 +263,7 @@ __global__ void __launch_bounds__(TS_THREADS) tet_staged_kernel(TsArgs<T> a) {
   // CTA sum of f (deterministic), then the last CTA sums the CTA partials.
   double fcta;
   if constexpr (PAIR) {
+    Acc facc_p = MODE == TS_HVP ? acc_zero() : log_sum_get(lsum, tab, a.K);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) facc_p = acc_add(facc_p, shfl_xor_acc2(facc_p, o));
     Acc* ra = reinterpret_cast<Acc*>(red);
@@ -311,7 +311,7 @@ __global__ void pair_split_vec_kernel(const double* __restrict__ u, const double
 // trip count, so the warp combine can run).  GRAD and HVP read u (and v) as
 // float pairs split once per call.
 template <int MODE, bool WARPC>
-__global__ void __launch_bounds__(TS_THREADS) tet_direct_pair_kernel(TsArgs<double> a) {
+__global__ void __launch_bounds__(TS_THREADS, MODE == TS_HVP ? 3 : 4) tet_direct_pair_kernel(TsArgs<double> a) {
   __shared__ float4 tab[kLogTableSize];
   __shared__ double red[2 * TS_WARPS];
   constexpr bool REV = MODE == TS_GRAD || MODE == TS_HVP;
@@ -326,16 +326,21 @@ __global__ void __launch_bounds__(TS_THREADS) tet_direct_pair_kernel(TsArgs<doub
     bad |= !pair_in_range(2.0 * fb);
     fb2 = split_f64(2.0 * fb);
   }
-  Acc fa = acc_zero();
-  int cnt = 0;
+  LogSum lsum = log_sum_zero();
   const double* Gp = reinterpret_cast<const double*>(a.G);
   const double* u = reinterpret_cast<const double*>(a.u);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < a.ne;
-       base += stride, ++cnt) {
-    const int64_t e = base + lane;
+  // the forward and the taping forward load the next element's vertices a step ahead, so that
+  // its gathers need not wait for them (6e6 elements: 119.5 -> 114.3 and 155 -> 148 us); the
+  // scattering modes would spill for it (189 -> 198 us)
+  const int4 none = make_int4(-1, -1, -1, -1);
+  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int4 cn = !REV && e < a.ne ? __ldcs(a.conn + e) : none;
+  for (int64_t base = e - lane; base < a.ne; base += stride, e += stride) {
     const bool act = e < a.ne;
-    const int4 c = act ? __ldcs(a.conn + e) : make_int4(-1, -1, -1, -1);
+    int4 c = cn;
+    if constexpr (REV) c = act ? __ldcs(a.conn + e) : none;
+    else cn = e + stride < a.ne ? __ldcs(a.conn + e + stride) : none;
     double wv[4];
     Pair wp[4];
     if (act) {
@@ -345,13 +350,12 @@ __global__ void __launch_bounds__(TS_THREADS) tet_direct_pair_kernel(TsArgs<doub
               c, Gp + e * 12, u, reinterpret_cast<const double*>(a.v), fb2, sink, bad);
         else
           elem_pair<MODE, std::decay_t<decltype(sink)>, true, USPLIT>(
-              c, Gp + e * 12, u, fb2, tab, a.K, fa, sink, reinterpret_cast<double*>(a.tape) + e * 4,
+              c, Gp + e * 12, u, fb2, tab, a.K, lsum, sink, reinterpret_cast<double*>(a.tape) + e * 4,
               bad);
       };
       if constexpr (WARPC) run(CollectSink<double>{wv, wp});
       else run(AtomicSink<double>{reinterpret_cast<double*>(a.gu)});
     }
-    if ((cnt & 31) == 31) acc_renorm(fa);
     if constexpr (WARPC) {
       const int key[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
@@ -363,6 +367,7 @@ __global__ void __launch_bounds__(TS_THREADS) tet_direct_pair_kernel(TsArgs<doub
     }
   }
   if (bad) set_error(a.err, ERRBIT_RANGE);
+  Acc fa = MODE == TS_HVP ? acc_zero() : log_sum_get(lsum, tab, a.K);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) fa = acc_add(fa, shfl_xor_acc2(fa, o));
   Acc* ra = reinterpret_cast<Acc*>(red);

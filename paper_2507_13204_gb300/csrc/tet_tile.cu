@@ -164,7 +164,7 @@ struct TileArgs {
 // in ascending order and issues one global reduction -- or, STORE (the
 // reproducible CSR strategy), writes the sum to the tile's partials instead.
 template <int MODE, bool STORE>
-__global__ void __launch_bounds__(TL_THREADS, 4) tet_tile_pair_kernel(TileArgs a) {
+__global__ void __launch_bounds__(TL_THREADS, MODE == TS_HVP ? 3 : 4) tet_tile_pair_kernel(TileArgs a) {
   __shared__ float4 tab[kLogTableSize];
   __shared__ __align__(16) float2 c_s[TL_THREADS / 32][TL_C];  // float4 stores
   __shared__ double red[2 * (TL_THREADS / 32)];
@@ -175,12 +175,11 @@ __global__ void __launch_bounds__(TL_THREADS, 4) tet_tile_pair_kernel(TileArgs a
   const double fb = load_seed(a.seed);
   bool bad = !pair_in_range(2.0 * fb);
   const Pair fb2 = split_f64(2.0 * fb);
-  Acc fa = acc_zero();
-  int cnt = 0;
+  LogSum lsum = log_sum_zero();
   float2* cw = c_s[warp];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < a.ne;
-       base += stride, ++cnt) {
+       base += stride) {
     const int64_t e = base + lane;
     // the tile's transposed connectivity, loaded before the element arithmetic so
     // that its latency overlaps it: lane l holds incidence bytes 4l .. 4l + 3 and
@@ -197,7 +196,7 @@ __global__ void __launch_bounds__(TL_THREADS, 4) tet_tile_pair_kernel(TileArgs a
       double wv[4];
       Pair wp[4];
       if constexpr (GRAD)
-        elem_pair<TS_GRAD, CollectSink<double>, true, true>(c, a.G + e * 12, a.u, fb2, tab, a.K, fa,
+        elem_pair<TS_GRAD, CollectSink<double>, true, true>(c, a.G + e * 12, a.u, fb2, tab, a.K, lsum,
                                                              CollectSink<double>{wv, wp}, nullptr, bad);
       else
         elem_pair_hvp<CollectSink<double>, true, true>(c, a.G + e * 12, a.u, a.v, fb2,
@@ -206,7 +205,6 @@ __global__ void __launch_bounds__(TL_THREADS, 4) tet_tile_pair_kernel(TileArgs a
       cs[0] = make_float4(wp[0].h, wp[0].l, wp[1].h, wp[1].l);
       cs[1] = make_float4(wp[2].h, wp[2].l, wp[3].h, wp[3].l);
     }
-    if ((cnt & 31) == 31) acc_renorm(fa);
     __syncwarp();
     {  // tile vertex `lane`: incidence bytes from the lanes' registers
       const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)(p1 - p0));
@@ -240,6 +238,7 @@ __global__ void __launch_bounds__(TL_THREADS, 4) tet_tile_pair_kernel(TileArgs a
   }
   if (bad) set_error(a.err, ERRBIT_RANGE);
   if constexpr (GRAD) {
+    Acc fa = log_sum_get(lsum, tab, a.K);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) fa = acc_add(fa, shfl_xor_acc2(fa, o));
     Acc* ra = reinterpret_cast<Acc*>(red);

@@ -388,3 +388,27 @@ def test_warp_combine_odd_counts_and_repeated_elements(api, dtype):
         assert rel_scalar(f.item(), f_ref) <= tol, len(rows)
         assert rel_l2(g.cpu().numpy(), g_ref) <= tol, len(rows)
         assert rel_l2(hv.cpu().numpy(), h_ref) <= tol, len(rows)
+
+
+@pytest.mark.parametrize("scale", [1e-9, 1e-4, 1.0, 1e4, 3e5, 1e9])
+@pytest.mark.parametrize("strategy", ["warp", "tile", "csr"])
+def test_value_over_the_range_of_element_energies(api, scale, strategy):
+    # float pairs take one log1p for eight elements' factors, and a factor above 2^30 by itself:
+    # energies from 1e-18 (relative accuracy of small values) over 2^30 (scale 3e5) to 1e18,
+    # also mixed within a thread's elements; more elements than the grid has threads
+    mesh = W.tet_mesh(40, 41, 39, perm_seed=2)
+    rng = np.random.default_rng(6)
+    p = _problem(api, mesh, torch.float64, strategy=strategy, arith="pair")
+    for mixed in (False, True):
+        u = rng.uniform(-1, 1, mesh.nv) * scale
+        if mixed:
+            u[rng.random(mesh.nv) < 0.5] *= 2.0 ** -8  # (|u| stays above 2^-60)
+        f_ref, g_ref = O.tet_grad(mesh.conn, mesh.G, u)
+        ut = torch.tensor(u, device="cuda")
+        f, g = p.grad(ut)
+        fe = p.eval(ut)
+        p.sync()
+        assert rel_scalar(f.item(), f_ref) <= TOL["f64"]
+        assert rel_scalar(fe.item(), f_ref) <= TOL["f64"]
+        assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f64"]
+    p.close()
