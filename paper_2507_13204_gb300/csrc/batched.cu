@@ -128,70 +128,78 @@ __device__ __forceinline__ Acc team_warps_sum(const Acc* ra, int lane, bool uppe
   return k;
 }
 
-// Rows [w.start, w.start + w.count) of a dense instance in native arithmetic;
-// returns the tile's f.
-template <typename T, int TEAM>
+// Rows [w.start, w.start + w.count) of a dense instance in native arithmetic, B_NR rows per
+// team and step: their loads go out together and one transposed butterfly reduces them all
+// (a butterfly per row is five FP64 adds a lane for eight columns' products).  Returns the
+// tile's f.  CPT > 0: ceil(n / TEAM) columns a thread, no test but the last one's; 0: at run
+// time (teams of 4).
+constexpr int B_NR = 4;
+
+template <typename T, int TEAM, int CPT>
 __device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp, double* red) {
+  constexpr int R = B_NR, WL = TEAM < 32 ? TEAM : 32, GL = WL / R;  // lanes of a row's total in a warp
+  constexpr int NT = BT / TEAM, KM = CPT ? CPT : B_CPT, TW = TEAM > 32 ? TEAM / 32 : 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = I.n;
   const T* __restrict__ A = static_cast<const T*>(I.d0);
   const T* __restrict__ x = static_cast<const T*>(I.x);
-  constexpr int NT = BT / TEAM;
   const int lt = tid % TEAM, team = tid / TEAM;
-  const int cpt = (n + TEAM - 1) / TEAM;  // <= B_CPT, uniform over the item
-  T xv[B_CPT], xbn[B_CPT];
+  auto col_in = [&](int k) { return (CPT && k < CPT - 1) || lt + k * TEAM < n; };
+  T xv[KM], xbn[KM];
 #pragma unroll
-  for (int k = 0; k < B_CPT; ++k) {
-    const int j = lt + k * TEAM;
-    xv[k] = (k < cpt && j < n) ? x[j] : T(0);
+  for (int k = 0; k < KM; ++k) {
+    xv[k] = col_in(k) ? x[lt + k * TEAM] : T(0);
     xbn[k] = T(0);
   }
   FSum<T> fn;
+  const int row = (lane % WL) / GL;  // whose total this lane holds
   const int64_t r1 = w.start + w.count;
-  const int iters = (w.count + NT - 1) / NT;
-  // software pipeline: the next row's loads are in flight while this row computes
-  T an[B_CPT];
-  auto load_row = [&](int itr_, T* dst) {
-    const int64_t r = w.start + (int64_t)itr_ * NT + team;
-    const bool v = itr_ < iters && r < r1;
-    const T* Ar = A + (v ? r : w.start) * (int64_t)n;
+  const int steps = (w.count + R * NT - 1) / (R * NT);
+  for (int c = 0; c < steps; ++c) {
+    const int64_t r0 = w.start + ((int64_t)c * NT + team) * R;
+    const int rows = r0 < r1 ? (int)(r1 - r0 < R ? r1 - r0 : R) : 0;
+    const T* Ar = A + (rows > 0 ? r0 : w.start) * (int64_t)n + lt;
+    T av[R][KM], d[R];
 #pragma unroll
-    for (int k = 0; k < B_CPT; ++k) {
-      const int j = lt + k * TEAM;
-      dst[k] = (k < cpt && v && j < n) ? __ldcs(Ar + j) : T(0);
+    for (int r = 0; r < R; ++r) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) av[r][k] = r < rows && col_in(k) ? __ldcs(Ar + k * TEAM) : T(0);
+      Ar += n;
     }
-  };
-  load_row(0, an);
-  for (int itr = 0; itr < iters; ++itr) {
-    const int64_t r = w.start + (int64_t)itr * NT + team;
-    const bool valid = r < r1;
-    T av[B_CPT];
 #pragma unroll
-    for (int k = 0; k < B_CPT; ++k) av[k] = an[k];
-    load_row(itr + 1, an);
-    {
-      T d = T(0);
+    for (int r = 0; r < R; ++r) {
+      d[r] = av[r][0] * xv[0];
 #pragma unroll
-      for (int k = 0; k < B_CPT; ++k)
-        if (k < cpt) d = fma(av[k], xv[k], d);
+      for (int k = 1; k < KM; ++k) d[r] = fma(av[r][k], xv[k], d[r]);
+    }
+    int o = WL / 2;
 #pragma unroll
-      for (int o = (TEAM < 32 ? TEAM : 32) / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      if constexpr (TEAM > 32) {
-        constexpr int TW = TEAM / 32;
-        T* rt = reinterpret_cast<T*>(red) + (itr & 1) * BW + team * TW;
-        if (lane == 0) rt[warp % TW] = d;
-        team_barrier<TEAM>(team);
-        d = rt[0];
+    for (int q = R / 2; q > 0; q >>= 1, o >>= 1) {
+      const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int q = 1; q < TW; ++q) d += rt[q];
-      }
-      if (valid) {
-        fn.add(d);
-        const T yb = T(2) * d;
+      for (int i = 0; i < q; ++i)
+        d[i] = (up ? d[i + q] : d[i]) + __shfl_xor_sync(0xffffffffu, up ? d[i] : d[i + q], o);
+    }
 #pragma unroll
-        for (int k = 0; k < B_CPT; ++k)
-          if (k < cpt) xbn[k] = fma(yb, av[k], xbn[k]);
-      }
+    for (; o > 0; o >>= 1) d[0] += __shfl_xor_sync(0xffffffffu, d[0], o);
+    T tot = d[0];
+    if constexpr (TEAM > 32) {
+      static_assert(TW <= GL, "the butterfly over the warps stays inside a row's lanes");
+      T* rt = reinterpret_cast<T*>(red) + ((c & 1) * BW + team * TW) * R;  // [TW][R]
+      if (lane % GL == 0) rt[(warp % TW) * R + row] = tot;
+      team_barrier<TEAM>(team);
+      tot = rt[(lane % TW) * R + row];
+#pragma unroll
+      for (int q = TW / 2; q > 0; q >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, q);
+    }
+    if (row >= rows) tot = T(0);  // past the tile's end: 0 times an infinite x is no row's value
+    if (TEAM <= 32 || warp % TW == 0) fn.add(tot);
+    const T ybl = T(2) * tot;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const T yb = __shfl_sync(0xffffffffu, ybl, (lane & ~(WL - 1)) + r * GL);
+#pragma unroll
+      for (int k = 0; k < KM; ++k) xbn[k] = fma(yb, av[r][k], xbn[k]);
     }
   }
   // combine the teams' partials in team order and store the tile's partial
@@ -199,14 +207,12 @@ __device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp,
   T* out = static_cast<T*>(I.partials) + (int64_t)w.tile * n;
   if constexpr (NT == 1) {
 #pragma unroll
-    for (int k = 0; k < B_CPT; ++k) {
-      const int j = lt + k * TEAM;
-      if (j < n) out[j] = xbn[k];
-    }
+    for (int k = 0; k < KM; ++k)
+      if (col_in(k)) out[lt + k * TEAM] = xbn[k];
   } else {
     T* ws = reinterpret_cast<T*>(wsp);
 #pragma unroll
-    for (int k = 0; k < B_CPT; ++k) ws[team * TEAM * B_CPT + lt + k * TEAM] = xbn[k];
+    for (int k = 0; k < KM; ++k) ws[team * TEAM * B_CPT + lt + k * TEAM] = xbn[k];
     __syncthreads();
     for (int j = tid; j < n; j += BT) {
       T s = ws[j];
@@ -214,13 +220,11 @@ __device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp,
       out[j] = s;
     }
   }
+  // f: each row's total once, one lane of the team's first warp
+  const bool counts = lane % GL == 0 && (TEAM <= 32 || warp % TW == 0);
+  const double f = block_sum(counts ? fn.get() : 0.0, red);
   __syncthreads();
-  if (lt == 0) red[team] = fn.get();
-  __syncthreads();
-  double tot = 0.0;
-  for (int t2 = 0; t2 < NT; ++t2) tot += red[t2];
-  __syncthreads();
-  return tot;
+  return f;
 }
 
 // ---- dense tiles of pair batches: two rows per team and step, columns in packed pairs ----
@@ -599,8 +603,21 @@ struct NativeTile {
   const BItem& w;
   unsigned char* wsp;
   double* red;
+  // the team is the smallest power of two (>= 4) with 8 columns a thread, so above 4
+  // threads a team thread has 5 to 8
   template <int TEAM>
-  __device__ __forceinline__ double run() const { return dense_tile<T, TEAM>(I, w, wsp, red); }
+  __device__ __forceinline__ double run() const {
+    if constexpr (TEAM > 4) {
+      switch ((I.n + TEAM - 1) / TEAM) {
+        case 5: return dense_tile<T, TEAM, 5>(I, w, wsp, red);
+        case 6: return dense_tile<T, TEAM, 6>(I, w, wsp, red);
+        case 7: return dense_tile<T, TEAM, 7>(I, w, wsp, red);
+        default: return dense_tile<T, TEAM, 8>(I, w, wsp, red);
+      }
+    } else {
+      return dense_tile<T, TEAM, 0>(I, w, wsp, red);
+    }
+  }
 };
 
 struct SplitTile {
@@ -970,8 +987,8 @@ Plan make_plan(const std::vector<kg_problem*>& probs, const std::vector<const vo
       I.team = 0;
       P.tet_ids.push_back(idx);
     }
-    if (cap > 0.0) {  // whole steps of the row teams (2 rows each) or of the CTA's threads, 4 at least
-      const int64_t unit = I.kind == BK_DENSE ? 2 * (BT / I.team) : BT;
+    if (cap > 0.0) {  // whole steps of the row teams or of the CTA's threads, 4 at least
+      const int64_t unit = I.kind == BK_DENSE ? (pair ? 2 : B_NR) * (BT / I.team) : BT;
       const int64_t most = (int64_t)(cap / item_cost(p, unit, es)) * unit;
       per = std::min(per, std::max(most, 4 * unit));
     }

@@ -46,7 +46,7 @@ struct QfConfig {
   int cpt = 1;      // columns per team thread (compile-time variant)
   int grid = 1;     // CTAs
   int rows_per_cta = 1;
-  int rgrid = 0;     // CTAs of the several-rows-a-step kernels (quadform_rows.cu); 0: not used
+  int rgrid = 0;     // CTAs of the native forward and fused kernels (quadform_rows.cu)
   int streamed = 0;  // 1: FP32 TMA-streamed kernel (quadform_f32.cu)
   int coop = 0;      // 1: the streamed gradient (pair, FP32) reduces its partials in one cooperative launch
 };
@@ -114,7 +114,7 @@ kg_status qf_eval(kg_problem* p, const void* x, void* f, cudaStream_t s);
 kg_status qf_grad(kg_problem* p, const void* x, void* f, void* gx, void* gA, const void* seed,
                   int accumulate, cudaStream_t s);
 
-// Native dense kernels for rows of up to 2048 entries (quadform_rows.cu).
+// Native dense kernels (quadform_rows.cu).
 template <typename T>
 struct QfRowsCall {
   const T* A;
@@ -131,7 +131,6 @@ struct QfRowsCall {
   T* gA;
   int accumulate;
 };
-bool qf_rows_supported(int64_t n);
 int qf_rows_grid(int dtype, int64_t m, int64_t n, int team);
 template <typename T>
 kg_status qf_rows_eval(const QfRowsCall<T>& c, cudaStream_t s);

@@ -31,141 +31,8 @@ struct QfArgs {
   int cpt;           // columns per team thread actually used (<= CPT_MAX)
   int rows_per_cta;  // contiguous band of rows per CTA
   const T* seed;     // nullable device scalar (fbar)
-  T* partials;       // FUSED: [gridDim.x][n] private xbar partials
-  double* fpart;     // per-CTA f partials
-  unsigned* counter; // arrival counter for the last-CTA reduction
-  T* y;              // nullable: forward row values
-  T* f;              // EVAL: output
-  T* gA;             // FUSED, nullable: gradient w.r.t. A
-  int accumulate;
+  const T* y;        // forward row values
 };
-
-enum { QF_EVAL = 0, QF_FUSED = 1 };
-
-// Sum over a team of TEAM threads; every thread of the CTA calls it in the same
-// iteration.  red: shared [2][nteams][TEAM/32], double-buffered by `par`.
-template <typename T, int TEAM>
-__device__ __forceinline__ T team_sum(T v, T* red, int par) {
-  v = warp_sum(v);
-  if constexpr (TEAM == 32) {
-    return v;
-  } else {
-    constexpr int W = TEAM / 32;
-    const int team = threadIdx.x / TEAM, w = (threadIdx.x % TEAM) >> 5;
-    const int nteams = blockDim.x / TEAM;
-    T* r = red + (par * nteams + team) * W;
-    if ((threadIdx.x & 31) == 0) r[w] = v;
-    __syncthreads();
-    // lane l takes warp l mod W's sum, and a butterfly over W lanes gives every lane the
-    // same total: log2(W) adds a thread instead of W (FP64 adds are scarce on GB300)
-    T s = r[(threadIdx.x & 31) % W];
-#pragma unroll
-    for (int o = W / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-  }
-}
-
-// Team-per-row kernel.  Team thread lt owns columns j = lt + k*TEAM, k < cpt.
-// EVAL: y_i and f.  FUSED: additionally ybar_i = 2 fbar y_i and the private
-// partial xbar_j += ybar_i A_ij (and Abar_ij when gA is given), with the
-// row's A values still in registers: A is read once.
-template <typename T, int TEAM, int CPT_MAX, int MODE>
-__global__ void __launch_bounds__(512) qf_team_kernel(QfArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int n = a.n;
-  const int nteams = blockDim.x / TEAM;
-  const int team = threadIdx.x / TEAM, lt = threadIdx.x % TEAM;
-  T* xs = reinterpret_cast<T*>(smem_raw);                  // CPT_MAX*TEAM (x, later xbar)
-  T* red = xs + CPT_MAX * TEAM;                            // 2*nteams*(TEAM/32)
-  double* fs = reinterpret_cast<double*>(red + 2 * nteams * (TEAM / 32) + 2);  // nteams + 32
-  fs = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(fs) + 7) & ~uintptr_t(7));
-
-  for (int j = threadIdx.x; j < CPT_MAX * TEAM; j += blockDim.x) xs[j] = j < n ? a.x[j] : T(0);
-  __syncthreads();
-
-  const T fb = MODE == QF_FUSED ? load_seed(a.seed) : T(1);
-  T xb[CPT_MAX];
-#pragma unroll
-  for (int k = 0; k < CPT_MAX; ++k) xb[k] = T(0);
-  FSum<T> fsum;
-
-  const int64_t r0 = (int64_t)blockIdx.x * a.rows_per_cta;
-  const int64_t r1 = r0 + a.rows_per_cta < a.m ? r0 + a.rows_per_cta : a.m;
-  const int iters = r1 > r0 ? (int)((r1 - r0 + nteams - 1) / nteams) : 0;
-  for (int it = 0; it < iters; ++it) {
-    const int64_t row = r0 + (int64_t)it * nteams + team;
-    const bool valid = row < r1;
-    const T* Ar = a.A + (valid ? row : r0) * (int64_t)n;
-    T av[CPT_MAX];
-#pragma unroll
-    for (int k = 0; k < CPT_MAX; ++k) {
-      const int j = lt + k * TEAM;
-      av[k] = (k < a.cpt && valid && j < n) ? ld_stream(Ar + j) : T(0);
-    }
-    T d = T(0);
-#pragma unroll
-    for (int k = 0; k < CPT_MAX; ++k)
-      if (k < a.cpt) d = fma(av[k], xs[lt + k * TEAM], d);
-    const T yv = team_sum<T, TEAM>(d, red, it & 1);
-    if (valid) {
-      if (lt == 0) {
-        fsum.add(yv);
-        if (a.y) a.y[row] = yv;
-      }
-      if constexpr (MODE == QF_FUSED) {
-        const T yb = T(2) * fb * yv;
-#pragma unroll
-        for (int k = 0; k < CPT_MAX; ++k)
-          if (k < a.cpt) xb[k] = fma(yb, av[k], xb[k]);
-        if (a.gA) {
-          T* gr = a.gA + row * (int64_t)n;
-#pragma unroll
-          for (int k = 0; k < CPT_MAX; ++k) {
-            const int j = lt + k * TEAM;
-            if (k < a.cpt && j < n) {
-              const T v = yb * xs[j];
-              gr[j] = a.accumulate ? gr[j] + v : v;
-            }
-          }
-        }
-      }
-    }
-  }
-
-  // CTA's f partial: team leaders in team order.
-  __syncthreads();
-  if (lt == 0) fs[team] = fsum.get();
-  __syncthreads();
-  double fcta = 0.0;
-  for (int t = 0; t < nteams; ++t) fcta += fs[t];
-
-  if constexpr (MODE == QF_EVAL) {
-    finish_sum<T>(fcta, a.fpart, a.counter, a.f, 0, fs + nteams);
-  } else {
-    if (threadIdx.x == 0) a.fpart[blockIdx.x] = fcta;
-    // combine the teams' private xbar in team order, then store this CTA's partial
-    T* out = a.partials + (int64_t)blockIdx.x * n;
-    if (nteams == 1) {
-#pragma unroll
-      for (int k = 0; k < CPT_MAX; ++k) {
-        const int j = lt + k * TEAM;
-        if (k < a.cpt && j < n) out[j] = xb[k];
-      }
-    } else {
-      for (int t = 0; t < nteams; ++t) {
-        if (team == t) {
-#pragma unroll
-          for (int k = 0; k < CPT_MAX; ++k) {
-            const int j = lt + k * TEAM;
-            if (k < a.cpt) xs[j] = t == 0 ? xb[k] : xs[j] + xb[k];
-          }
-        }
-        __syncthreads();
-      }
-      for (int j = threadIdx.x; j < n; j += blockDim.x) out[j] = xs[j];
-    }
-  }
-}
 
 // Reverse with the forward schedule (the paper's atomic scatter): each team
 // re-reads its row and adds ybar_i A_ij into gx[j] (a global red); ybar_i comes from
@@ -218,16 +85,18 @@ __global__ void __launch_bounds__(256) qf_transpose_kernel(const T* __restrict__
 }
 
 // Sum of the private partials in a fixed order, a dependent launch: a block of 512
-// threads takes 64 bytes of columns, thread (cx, py) sums partials py, py + PY, ... of
+// threads takes CX columns (64 bytes), thread (cx, py) sums partials py, py + PY, ... of
 // column cx (eight loads in flight); the lanes of a warp that hold the same column add by
 // a butterfly, then the 16 warps' sums are added in warp order.  Block 0 also sums the
 // per-CTA f partials into *f.  Narrow blocks spread the loads of a short row of partials
-// over the chip: 304 partials of 255 doubles took 7.0 us in 8 blocks of 32 columns.
-template <typename T>
+// over the chip: 304 partials of 255 doubles took 7.0 us in 8 blocks of 32 columns.  Up to
+// 64 partials take 32 columns a block (CX): 64 bytes would leave half the threads idle in
+// four times the blocks (30 partials of 9001 doubles: 3 us more).
+template <typename T, int CX>
 __global__ void __launch_bounds__(512) qf_reduce_kernel(const T* __restrict__ partials, int nparts,
                                                         int n, const double* __restrict__ fpart,
                                                         int nf, T* gx, T* f, int accumulate) {
-  constexpr int CX = 64 / (int)sizeof(T), PY = 512 / CX;
+  constexpr int PY = 512 / CX;
   __shared__ T red[16][CX];
   __shared__ double fred[32];
   grid_dependency_wait();  // the partials are written and visible
@@ -258,8 +127,8 @@ __global__ void __launch_bounds__(512) qf_reduce_kernel(const T* __restrict__ pa
 
 // ---------------------------------------------------------------- host ----
 // Variants: (TEAM, CPT_MAX, block).  Team thread count x CPT_MAX bounds n.
-// Rows of up to 2048 entries go to the kernels of quadform_rows.cu; their variants here
-// size the atomic adjoint and say which teams hold a row.
+// The forward and the fused gradient are quadform_rows.cu's; the variants here are the
+// atomic adjoint's and say which teams hold a row.
 struct QfVariant {
   int team, cpt_max, block;
 };
@@ -278,36 +147,6 @@ static int pick_variant(int64_t n, int team_hint) {
     if (n <= (int64_t)kVariants[v].team * kVariants[v].cpt_max) return v;
   }
   return -1;
-}
-
-template <typename T>
-static size_t qf_smem_bytes(const QfVariant& v) {
-  const int nteams = v.block / v.team;
-  return sizeof(T) * ((size_t)v.cpt_max * v.team + 2 * nteams * (v.team / 32) + 2) + 8 +
-         sizeof(double) * (nteams + 32);
-}
-
-template <typename T, int MODE>
-static cudaError_t launch_team(int var, dim3 grid, cudaStream_t s, const QfArgs<T>& a) {
-  const QfVariant& v = kVariants[var];
-  const size_t smem = qf_smem_bytes<T>(v);
-  cudaError_t e = cudaSuccess;
-  auto go = [&](auto kern) {
-    e = set_smem_once(kern, smem);
-    if (e == cudaSuccess) {
-      prof_begin(s, MODE == QF_FUSED ? "qf_team_kernel<fused>" : "qf_team_kernel<eval>");
-      kern<<<grid, v.block, smem, s>>>(a);
-      prof_end(s);
-      e = cudaGetLastError();
-    }
-  };
-  switch (var) {
-    case 3: go(qf_team_kernel<T, 512, 20, MODE>); break;
-    case 4: go(qf_team_kernel<T, 512, 24, MODE>); break;
-    default: e = cudaErrorInvalidValue;
-  }
-  count_launch();
-  return e;
 }
 
 template <typename T>
@@ -384,8 +223,12 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
     c.streamed = 1;
     c.grid = qf_f32_grid(p, &c.rows_per_cta);
     c.team = c.block = 512;
-    kg_status rc = ws_common(p, c.grid, s);
-    if (rc == KG_OK) rc = ws_alloc(p, &p->partials, 4 * (size_t)c.grid * p->n, "xbar partials (FP32)");
+    // short rows: several at a step instead (40000 x 1024 96.8 -> 32 us, 40000 x 2048 97.6 -> 56);
+    // with fewer rows than CTAs of the streamed kernel, one a CTA is as good
+    if (p->n <= 2048 && p->m >= 2 * (int64_t)num_sms()) c.rgrid = qf_rows_grid(KG_F32, p->m, p->n, 0);
+    const int most = std::max(c.grid, c.rgrid);
+    kg_status rc = ws_common(p, most, s);
+    if (rc == KG_OK) rc = ws_alloc(p, &p->partials, 4 * (size_t)most * p->n, "xbar partials (FP32)");
     if (rc == KG_OK) c.coop = qf_f32_coop_fits(p) ? 1 : 0;
     return rc;
   }
@@ -408,13 +251,12 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
   if (p->opt.tile > 0) rows = p->opt.tile;
   c.rows_per_cta = (int)rows;
   c.grid = (int)((p->m + rows - 1) / rows);
-  if (qf_rows_supported(p->n))
-    c.rgrid = p->opt.tile > 0 ? c.grid : qf_rows_grid(p->dtype, p->m, p->n, p->opt.team);
+  c.rgrid = p->opt.tile > 0 ? c.grid : qf_rows_grid(p->dtype, p->m, p->n, p->opt.team);
   int fp = std::max({c.grid, c.rgrid, transpose_chunks(p)});
   kg_status rc = ws_common(p, fp, s);
   if (rc != KG_OK) return rc;
   if (p->strategy == KG_STRATEGY_FUSED || p->strategy == KG_STRATEGY_TRANSPOSE) {
-    int parts = p->strategy != KG_STRATEGY_FUSED ? transpose_chunks(p) : c.rgrid ? c.rgrid : c.grid;
+    int parts = p->strategy != KG_STRATEGY_FUSED ? transpose_chunks(p) : c.rgrid;
     rc = ws_alloc(p, &p->partials, p->esize * (size_t)parts * p->n, "xbar partials");
     if (rc != KG_OK) return rc;
   }
@@ -435,9 +277,7 @@ static QfArgs<T> make_args(kg_problem* p, const void* x, const void* seed) {
   a.cpt = p->qf.cpt;
   a.rows_per_cta = p->qf.rows_per_cta;
   a.seed = static_cast<const T*>(seed);
-  a.partials = static_cast<T*>(p->partials);
-  a.fpart = p->fpart;
-  a.counter = p->counter;
+  a.y = static_cast<const T*>(p->y);
   return a;
 }
 
@@ -460,9 +300,10 @@ static QfRowsCall<T> rows_call(kg_problem* p, const void* x, void* f) {
 template <typename T>
 kg_status qf_reduce_partials(const T* partials, int nparts, int n, const double* fpart, int nf, T* gx,
                              T* f, int accumulate, cudaStream_t s) {
-  constexpr int CX = 64 / (int)sizeof(T);
+  const bool few = nparts <= 64;
+  const int cx = few ? 32 : 64 / (int)sizeof(T);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((n + CX - 1) / CX);
+  cfg.gridDim = dim3((n + cx - 1) / cx);
   cfg.blockDim = dim3(512);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -470,8 +311,8 @@ kg_status qf_reduce_partials(const T* partials, int nparts, int n, const double*
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, qf_reduce_kernel<T>, partials, nparts, n, fpart, nf, gx, f,
-                                     accumulate);
+  auto kern = few ? qf_reduce_kernel<T, 32> : qf_reduce_kernel<T, 64 / (int)sizeof(T)>;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, partials, nparts, n, fpart, nf, gx, f, accumulate);
   count_launch();
   return e == cudaSuccess ? KG_OK : cuda_fail(e, "qf reduce kernel");
 }
@@ -482,23 +323,21 @@ template kg_status qf_reduce_partials<float>(const float*, int, int, const doubl
 
 template <typename T>
 static kg_status qf_eval_t(kg_problem* p, const void* x, void* f, T* y, cudaStream_t s) {
-  if (p->qf.rgrid) {
-    QfRowsCall<T> r = rows_call<T>(p, x, f);
-    r.y = y;
-    return qf_rows_eval(r, s);
-  }
-  QfArgs<T> a = make_args<T>(p, x, nullptr);
-  a.f = static_cast<T*>(f);
-  a.y = y;
-  const int var = pick_variant(p->n, p->qf.team);
-  cudaError_t e = launch_team<T, QF_EVAL>(var, dim3(p->qf.grid), s, a);
-  if (e != cudaSuccess) return cuda_fail(e, "qf forward kernel");
-  return KG_OK;
+  QfRowsCall<T> r = rows_call<T>(p, x, f);
+  r.y = y;
+  return qf_rows_eval(r, s);
+}
+
+// FP32 problems of the streamed kernel's shapes ask for aligned vectors whichever kernel runs.
+static const char* const kF32Align = "QUADFORM FP32 streamed kernels need 16-byte aligned x and gx";
+static bool aligned16(const void* a, const void* b) {
+  return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15u) == 0;
 }
 
 kg_status qf_eval(kg_problem* p, const void* x, void* f, cudaStream_t s) {
   if (p->arith == KG_ARITH_PAIR) return qf_pair_eval(p, x, f, s);
-  if (p->qf.streamed) return qf_f32_eval(p, x, f, s);
+  if (p->qf.streamed && !p->qf.rgrid) return qf_f32_eval(p, x, f, s);
+  if (p->qf.streamed && !aligned16(x, x)) return fail(KG_ERR_INVALID_ARG, kF32Align);
   return p->dtype == KG_F64 ? qf_eval_t<double>(p, x, f, nullptr, s)
                             : qf_eval_t<float>(p, x, f, nullptr, s);
 }
@@ -510,21 +349,12 @@ static kg_status qf_grad_t(kg_problem* p, const void* x, void* f, void* gx, void
   const int n = (int)p->n;
   cudaError_t e;
   if (p->strategy == KG_STRATEGY_FUSED) {
-    if (p->qf.rgrid) {
-      QfRowsCall<T> r = rows_call<T>(p, x, f);
-      r.seed = static_cast<const T*>(seed);
-      r.gx = static_cast<T*>(gx);
-      r.gA = static_cast<T*>(gA);
-      r.accumulate = accumulate;
-      return qf_rows_grad(r, s);
-    }
-    QfArgs<T> a = make_args<T>(p, x, seed);
-    a.gA = static_cast<T*>(gA);
-    a.accumulate = accumulate;
-    e = launch_team<T, QF_FUSED>(var, dim3(p->qf.grid), s, a);
-    if (e != cudaSuccess) return cuda_fail(e, "qf fused kernel");
-    return qf_reduce_partials<T>(static_cast<const T*>(p->partials), p->qf.grid, n, p->fpart, p->qf.grid,
-                                 static_cast<T*>(gx), static_cast<T*>(f), accumulate, s);
+    QfRowsCall<T> r = rows_call<T>(p, x, f);
+    r.seed = static_cast<const T*>(seed);
+    r.gx = static_cast<T*>(gx);
+    r.gA = static_cast<T*>(gA);
+    r.accumulate = accumulate;
+    return qf_rows_grad(r, s);
   }
   if (gA) return fail(KG_ERR_UNSUPPORTED, "QUADFORM: gradient w.r.t. A needs the FUSED strategy");
   // forward with y stored (f written by the last CTA)
@@ -537,7 +367,6 @@ static kg_status qf_grad_t(kg_problem* p, const void* x, void* f, void* gx, void
       if (e != cudaSuccess) return cuda_fail(e, "zero gx");
     }
     QfArgs<T> a = make_args<T>(p, x, seed);
-    a.y = static_cast<T*>(p->y);
     e = launch_atomic<T>(var, dim3(p->qf.grid), s, a, static_cast<T*>(gx));
     if (e != cudaSuccess) return cuda_fail(e, "qf atomic adjoint kernel");
     return KG_OK;
@@ -566,49 +395,22 @@ static kg_status qf_grad_t(kg_problem* p, const void* x, void* f, void* gx, void
 kg_status qf_native_fused_on_scratch(const double* A, int64_t m, int64_t n, const double* x,
                                      double* f, double* gx, double* scratch,
                                      size_t scratch_doubles, cudaStream_t s) {
-  const int var = pick_variant(n, 0);
-  if (var < 0) return fail(KG_ERR_INVALID_ARG, "n must be <= 12288");
+  if (pick_variant(n, 0) < 0) return fail(KG_ERR_INVALID_ARG, "n must be <= 12288");
   const int64_t max_grid = (int64_t)(scratch_doubles / ((size_t)n + 1));
   if (max_grid < 1)
     return fail(KG_ERR_INVALID_ARG, "scratch of " + std::to_string(scratch_doubles) +
                                         " doubles is too small for n = " + std::to_string(n));
-  if (qf_rows_supported(n)) {
-    QfRowsCall<double> r{};  // no arrival counter: more than one CTA's partials in a second launch
-    r.A = A;
-    r.x = x;
-    r.m = m;
-    r.n = n;
-    r.grid = (int)std::min<int64_t>(qf_rows_grid(KG_F64, m, n, 0), max_grid);
-    r.partials = scratch;
-    r.fpart = scratch + (size_t)r.grid * n;
-    r.f = f;
-    r.gx = gx;
-    return qf_rows_grad(r, s);
-  }
-  const QfVariant& v = kVariants[var];
-  const int nteams = v.block / v.team;
-  const int resident = v.block >= 512 ? 1 : 2;
-  const int64_t target = (int64_t)num_sms() * resident;
-  const int64_t rows = std::max<int64_t>({(int64_t)nteams, (m + target - 1) / target,
-                                          (m + max_grid - 1) / max_grid});
-  const int grid = (int)((m + rows - 1) / rows);
-  const size_t need = (size_t)grid * (size_t)n + (size_t)grid;
-  if (need > scratch_doubles)
-    return fail(KG_ERR_INVALID_ARG, "problem needs " + std::to_string(need) +
-                                        " scratch doubles, more than the " +
-                                        std::to_string(scratch_doubles) + " available");
-  QfArgs<double> a{};
-  a.A = A;
-  a.x = x;
-  a.m = m;
-  a.n = (int)n;
-  a.cpt = (int)((n + v.team - 1) / v.team);
-  a.rows_per_cta = (int)rows;
-  a.partials = scratch;
-  a.fpart = scratch + (size_t)grid * n;
-  cudaError_t e = launch_team<double, QF_FUSED>(var, dim3(grid), s, a);
-  if (e != cudaSuccess) return cuda_fail(e, "qf fused kernel");
-  return qf_reduce_partials<double>(scratch, grid, (int)n, a.fpart, grid, gx, f, 0, s);
+  QfRowsCall<double> r{};  // no arrival counter: more than one CTA's partials in a second launch
+  r.A = A;
+  r.x = x;
+  r.m = m;
+  r.n = n;
+  r.grid = (int)std::min<int64_t>(qf_rows_grid(KG_F64, m, n, 0), max_grid);
+  r.partials = scratch;
+  r.fpart = scratch + (size_t)r.grid * n;
+  r.f = f;
+  r.gx = gx;
+  return qf_rows_grad(r, s);
 }
 
 kg_status qf_grad(kg_problem* p, const void* x, void* f, void* gx, void* gA, const void* seed,
@@ -623,7 +425,8 @@ kg_status qf_grad(kg_problem* p, const void* x, void* f, void* gx, void* gA, con
     if (gA)
       return fail(KG_ERR_UNSUPPORTED, "QUADFORM: the gradient w.r.t. A is produced by the register "
                                       "team kernels (pass team=block size)");
-    return qf_f32_grad(p, x, f, gx, seed, accumulate, s);
+    if (!p->qf.rgrid) return qf_f32_grad(p, x, f, gx, seed, accumulate, s);
+    if (!aligned16(x, gx)) return fail(KG_ERR_INVALID_ARG, kF32Align);
   }
   return p->dtype == KG_F64 ? qf_grad_t<double>(p, x, f, gx, gA, seed, accumulate, s)
                             : qf_grad_t<float>(p, x, f, gx, gA, seed, accumulate, s);

@@ -1,5 +1,5 @@
-// Dense ||A x||^2 for rows of up to 2048 entries in native arithmetic (FP64, FP32):
-// forward and fused value-and-gradient, several rows per team and step.
+// Dense ||A x||^2 in native arithmetic (FP64, FP32): forward and fused value-and-gradient,
+// several rows per team and step.
 //
 // What bounds it: FP32, the stream of A from HBM; FP64, GB300's 2 DFMA a clock and SM
 // (two DFMA an entry are 2.7 times the HBM time of its 8 bytes).  Neither leaves room
@@ -13,16 +13,18 @@
 //     all R rows;
 //   - only teams wider than a warp (n > 256) exchange through shared memory, once per
 //     R rows.
-// CPL is ceil(n / (32 W)) at compile time, so that no column slot but the last is
-// tested or idle.  Groups of R rows go round-robin over all teams of the grid; xbar is
+// CPL is fixed at compile time, ceil(n / (32 W)) up to n = 4096 and even above, so that
+// at most the last two column slots are tested or idle.  Groups of R rows go round-robin over all teams of the grid; xbar is
 // accumulated in registers, combined over the CTA's teams in team order and, for grids
 // of one CTA, written as the gradient; larger grids write a row of partials per CTA,
 // summed in a fixed order by the CTA that finishes last (few partials) or by
 // qf_reduce_kernel: bitwise reproducible.
 //
 // Measured (value and gradient, one call, against one row a team and step with a butterfly
-// per row): FP64 150001 x 255 857 -> 160 us (its DFMAs take 122), FP32 400000 x 100
-// 121 -> 36.6 us (its bytes take 23.6).
+// per row): FP64 150001 x 255 857 -> 160 us (its DFMAs take 122), 20000 x 2051 963 -> 250
+// (131), 10000 x 5001 484 -> 243 (160), 10000 x 9999 478 -> 475 (320); FP32 400000 x 100
+// 121 -> 36.6 us (its bytes take 23.6), 40000 x 1024 96.8 -> 31 (24), 20000 x 4095
+// 157 -> 72 (48).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,9 +35,6 @@
 #include "kg_pair.cuh"
 
 namespace kg {
-
-constexpr int QR_THREADS = 256;
-constexpr int QR_WARPS = QR_THREADS / 32;
 
 template <typename T>
 struct QrArgs {
@@ -75,25 +74,45 @@ __device__ __forceinline__ T reduce_rows(T (&d)[R]) {
   return d[0];
 }
 
-// FP64: two CTAs an SM (128 registers, R * CPL doubles of A in them); FP32: three.
-template <typename T, int W, int CPL, int R, bool FUSED>
-__global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_kernel(QrArgs<T> a) {
-  constexpr int TEAM = 32 * W, NT = QR_WARPS / W, G = 32 / R;  // G lanes hold a row's total
-  static_assert(W <= G, "the cross-warp butterfly stays inside a row's lanes");
-  __shared__ T xbs[FUSED ? QR_THREADS * CPL : 1];
-  __shared__ T red[W > 1 ? 2 * QR_WARPS * R : 1];
+// One kernel's shape: W warps a team, CPL columns a lane (the first FULL of them inside every
+// row that runs it), R rows a step.  Teams of up to 8 warps share CTAs of 256 threads, a team
+// of 16 is a CTA.  XS: x in shared memory, where a lane's columns leave no registers for it.
+template <int W_, int CPL_, int FULL_, int R_, bool XS_>
+struct QrShape {
+  static constexpr int W = W_, CPL = CPL_, FULL = FULL_, R = R_;
+  static constexpr bool XS = XS_;
+  static constexpr int THREADS = W_ > 8 ? 512 : 256, WARPS = THREADS / 32, NT = WARPS / W_;
+};
+
+// FP64: 16 warps an SM (128 registers, R * CPL doubles of A in them); FP32 teams of up to 8
+// warps: 24.
+template <typename T, typename S, bool FUSED>
+__global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) == 8 ? 2 : 3)
+    qf_rows_kernel(QrArgs<T> a) {
+  constexpr int W = S::W, CPL = S::CPL, R = S::R, NT = S::NT, THREADS = S::THREADS, WARPS = S::WARPS;
+  constexpr int TEAM = 32 * W, G = 32 / R, WG = W < G ? W : G;  // G lanes hold a row's total
+  __shared__ T xbs[FUSED ? (NT > 1 ? THREADS * CPL : THREADS) : 1];
+  __shared__ T red[W > 1 ? 2 * WARPS * R : 1];
   __shared__ double fred[32];
   __shared__ bool s_last;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  T* xs = reinterpret_cast<T*>(dyn);  // XS: [CPL][THREADS], each thread its own entries
   const int n = a.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int team = warp / W, lt = threadIdx.x % TEAM;
-  auto col_in = [&](int k) { return k < CPL - 1 || lt + k * TEAM < n; };
+  auto col_in = [&](int k) { return k < S::FULL || lt + k * TEAM < n; };
 
-  T xv[CPL], xb[CPL];
+  T xr[S::XS ? 1 : CPL], xb[CPL];
 #pragma unroll
   for (int k = 0; k < CPL; ++k) {
-    xv[k] = col_in(k) ? a.x[lt + k * TEAM] : T(0);
+    const T v = col_in(k) ? a.x[lt + k * TEAM] : T(0);
+    if constexpr (S::XS) xs[k * THREADS + threadIdx.x] = v;
+    else xr[k] = v;
     xb[k] = T(0);
   }
+  auto xv = [&](int k) {
+    if constexpr (S::XS) return xs[k * THREADS + threadIdx.x];
+    else return xr[k];
+  };
   const T fb2 = FUSED ? T(2) * load_seed(a.seed) : T(0);
   FSum<T> fsum;  // of row lane / G of every group (counted once per row below)
 
@@ -119,29 +138,31 @@ __global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_ke
     T d[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      d[r] = av[r][0] * xv[0];
+      d[r] = av[r][0] * xv(0);
 #pragma unroll
-      for (int k = 1; k < CPL; ++k) d[r] = fma(av[r][k], xv[k], d[r]);
+      for (int k = 1; k < CPL; ++k) d[r] = fma(av[r][k], xv(k), d[r]);
     }
     T tot = reduce_rows<R>(d);
     const int row = lane / G;
     if constexpr (W > 1) {
-      T* rd = red + par * QR_WARPS * R + team * W * R;
+      T* rd = red + par * WARPS * R + team * W * R;
       if (lane % G == 0) rd[(warp % W) * R + row] = tot;
       __syncthreads();
-      tot = rd[(lane % W) * R + row];
+      tot = rd[(lane % WG) * R + row];
 #pragma unroll
-      for (int o = W / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+      for (int i = G; i < W; i += G) tot += rd[(i + lane % G) * R + row];
+#pragma unroll
+      for (int o = WG / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     }
     if (row >= rows) tot = T(0);  // past the end: 0 times an infinite x is no row's value
-    fsum.add(tot);
+    if (W == 1 || warp % W == 0) fsum.add(tot);  // one warp of the team: an FP64 instruction a row
     if constexpr (!FUSED) {
       if (a.y && row < rows && lane % G == 0 && (W == 1 || warp % W == 0)) a.y[r0 + row] = tot;
     } else {
       const T ybl = fb2 * tot;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const T yb = __shfl_sync(0xffffffffu, ybl, r * G);
+        const T yb = R == 1 ? ybl : __shfl_sync(0xffffffffu, ybl, r * G);
 #pragma unroll
         for (int k = 0; k < CPL; ++k) xb[k] = fma(yb, av[r][k], xb[k]);
         if (a.gA && r < rows) {
@@ -149,7 +170,7 @@ __global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_ke
 #pragma unroll
           for (int k = 0; k < CPL; ++k)
             if (col_in(k)) {
-              const T v = yb * xv[k];
+              const T v = yb * xv(k);
               gr[k * TEAM] = a.accumulate ? gr[k * TEAM] + v : v;
             }
         }
@@ -164,16 +185,24 @@ __global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_ke
     finish_sum<T>(fcta, a.fpart, a.counter, a.f, 0, fred);
     return;
   } else {
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) xbs[team * TEAM * CPL + lt + k * TEAM] = xb[k];
-    __syncthreads();
     const bool one = gridDim.x == 1;
     T* out = one ? a.gx : a.partials + (int64_t)blockIdx.x * n;
-    for (int j = threadIdx.x; j < n; j += QR_THREADS) {
-      T s = xbs[j];
+    if constexpr (NT == 1) {
 #pragma unroll
-      for (int t = 1; t < NT; ++t) s += xbs[t * TEAM * CPL + j];
-      out[j] = one && a.accumulate ? out[j] + s : s;
+      for (int k = 0; k < CPL; ++k) {
+        const int j = lt + k * TEAM;
+        if (col_in(k)) out[j] = one && a.accumulate ? out[j] + xb[k] : xb[k];
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < CPL; ++k) xbs[team * TEAM * CPL + lt + k * TEAM] = xb[k];
+      __syncthreads();
+      for (int j = threadIdx.x; j < n; j += THREADS) {
+        T s = xbs[j];
+#pragma unroll
+        for (int t = 1; t < NT; ++t) s += xbs[t * TEAM * CPL + j];
+        out[j] = one && a.accumulate ? out[j] + s : s;
+      }
     }
     if (threadIdx.x == 0) {
       if (one) {
@@ -183,8 +212,8 @@ __global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_ke
       }
     }
     if (one || !a.last) return;
-    // few partials: the CTA that arrives last sums them, thread (cx, pg) partials pg,
-    // pg + PG, ... of column cx, the PG sums then in pg order
+    // few partials of few columns: the CTA that arrives last sums them, thread (j, pg)
+    // partials pg, pg + PG, ... of column j, the PG sums then in pg order
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) s_last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
@@ -193,25 +222,22 @@ __global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_ke
     __threadfence();
     const int parts = gridDim.x;
     int cw = 32;
-    while (cw < n && cw < QR_THREADS) cw *= 2;
-    const int pgs = QR_THREADS / cw, cx = threadIdx.x % cw, pg = threadIdx.x / cw;
-    for (int jb = 0; jb < n; jb += cw) {
-      const int j = jb + cx;
-      T s = T(0);
-      if (j < n) {
+    while (cw < n) cw *= 2;  // n <= 128 here
+    const int pgs = THREADS / cw, j = threadIdx.x % cw, pg = threadIdx.x / cw;
+    T s = T(0);
+    if (j < n) {
 #pragma unroll 8
-        for (int c = pg; c < parts; c += pgs) s += __ldcg(a.partials + (int64_t)c * n + j);
-      }
-      __syncthreads();
-      xbs[threadIdx.x] = s;
-      __syncthreads();
-      if (pg == 0 && j < n) {
-        for (int q = 1; q < pgs; ++q) s += xbs[q * cw + cx];
-        a.gx[j] = a.accumulate ? a.gx[j] + s : s;
-      }
+      for (int c = pg; c < parts; c += pgs) s += __ldcg(a.partials + (int64_t)c * n + j);
+    }
+    __syncthreads();
+    xbs[threadIdx.x] = s;
+    __syncthreads();
+    if (pg == 0 && j < n) {
+      for (int q = 1; q < pgs; ++q) s += xbs[q * cw + j];
+      a.gx[j] = a.accumulate ? a.gx[j] + s : s;
     }
     double fs = 0.0;
-    for (int i = threadIdx.x; i < parts; i += QR_THREADS) fs += __ldcg(a.fpart + i);
+    for (int i = threadIdx.x; i < parts; i += THREADS) fs += __ldcg(a.fpart + i);
     fs = block_sum(fs, fred);
     if (threadIdx.x == 0) {
       if (a.f) *a.f = (T)fs;
@@ -221,53 +247,84 @@ __global__ void __launch_bounds__(QR_THREADS, sizeof(T) == 8 ? 2 : 3) qf_rows_ke
 }
 
 // ---------------------------------------------------------------- host ----
-// Warps per team for rows of n entries (8 columns a lane at most); team: the
-// caller's threads per team (0: the smallest that holds the row).
-static int qr_warps(int64_t n, int team) {
-  if (team) return team / 32;
-  int w = 1;
-  while ((int64_t)256 * w < n) w *= 2;
-  return w;
-}
-
-// Rows per step: R * CPL values of A in a lane's registers, up to 32; a team of 8 warps
-// takes 4 rows (the cross-warp butterfly needs W lanes a row).
-constexpr int qr_rows(int cpl, int w) { return cpl <= 4 && w < 8 ? 8 : 4; }
-
-// Calls go(kernel, rows per step, teams per CTA) with the kernel of this row length.
-template <typename T, bool FUSED, int W, typename Go>
-static void qr_with_cpl(int64_t n, const Go& go) {
+// Calls go(shape) with the shape for rows of n entries.  team: the caller's threads per team
+// (0: the smallest that holds the row in 8 columns a lane; 512 threads above 2048 entries).
+//   up to 8 warps:  8 columns a lane at most, 8 rows a step up to 4 of them, else 4 (a team
+//                   of 8 warps: 4), R * CPL <= 32 values of A in a lane's registers;
+//   16 warps:       n <= 4096 4 rows a step, then x in shared memory and 2 rows (FP32 4) to
+//                   8192 entries, 1 (FP32 2) to 12288, where the forward, which keeps no row
+//                   for a reverse, still takes 2 (FP32 4).
+template <typename T, int W, typename Go>
+static void qr_small(int64_t n, const Go& go) {
   switch ((n + 32 * W - 1) / (32 * W)) {
 #define KG_CPL(c) \
-  case c: go(qf_rows_kernel<T, W, c, qr_rows(c, W), FUSED>, qr_rows(c, W), QR_WARPS / W); break;
+  case c: go(QrShape<W, c, c - 1, (c <= 4 && W < 8 ? 8 : 4), false>{}); break;
     KG_CPL(1) KG_CPL(2) KG_CPL(3) KG_CPL(4) KG_CPL(5) KG_CPL(6) KG_CPL(7) KG_CPL(8)
 #undef KG_CPL
   }
 }
 
+//
+// FP64 teams of several warps on at most two rows an SM take one row a step: four rows on
+// one team leave the other SMs idle while its FP64 unit works through them (100 x 2001
+// 11.7 us, 9.0 with a row a step).
 template <typename T, bool FUSED, typename Go>
-static void qr_with_kernel(int64_t n, int team, const Go& go) {
-  switch (qr_warps(n, team)) {
-    case 1: qr_with_cpl<T, FUSED, 1>(n, go); break;
-    case 2: qr_with_cpl<T, FUSED, 2>(n, go); break;
-    case 4: qr_with_cpl<T, FUSED, 4>(n, go); break;
-    case 8: qr_with_cpl<T, FUSED, 8>(n, go); break;
+static void qr_with_shape(int64_t m, int64_t n, int team, const Go& go) {
+  constexpr int R2 = sizeof(T) == 8 ? 2 : 4, R1 = FUSED ? R2 / 2 : R2;
+  int w = team / 32;
+  if (!team)
+    for (w = 1; (int64_t)256 * w < n && w < 16;) w *= 2;
+  if (sizeof(T) == 8 && w >= 2 && m <= 2 * (int64_t)num_sms() && n <= 8192) {
+    switch (w) {
+      case 2: return go(QrShape<2, 8, 0, 1, false>{});
+      case 4: return go(QrShape<4, 8, 0, 1, false>{});
+      case 8: return go(QrShape<8, 8, 0, 1, false>{});
+    }
+    return n <= 4096 ? go(QrShape<16, 8, 0, 1, false>{}) : go(QrShape<16, 16, 8, 1, true>{});
   }
+  switch (w) {
+    case 1: return qr_small<T, 1>(n, go);
+    case 2: return qr_small<T, 2>(n, go);
+    case 4: return qr_small<T, 4>(n, go);
+    case 8: return qr_small<T, 8>(n, go);
+  }
+  const int64_t c = (n + 511) / 512;
+  if (c <= 4) return go(QrShape<16, 4, 0, 4, false>{});  // a caller's team of 512 only
+  if (c == 5) return go(QrShape<16, 5, 4, 4, false>{});
+  if (c == 6) return go(QrShape<16, 6, 5, 4, false>{});
+  if (c == 7) return go(QrShape<16, 7, 6, 4, false>{});
+  if (c == 8) return go(QrShape<16, 8, 7, 4, false>{});
+  if (c <= 10) return go(QrShape<16, 10, 8, R2, true>{});
+  if (c <= 12) return go(QrShape<16, 12, 10, R2, true>{});
+  if (c <= 14) return go(QrShape<16, 14, 12, R2, true>{});
+  if (c <= 16) return go(QrShape<16, 16, 14, R2, true>{});
+  if (c <= 18) return go(QrShape<16, 18, 16, R1, true>{});
+  if (c <= 20) return go(QrShape<16, 20, 18, R1, true>{});
+  if (c <= 22) return go(QrShape<16, 22, 20, R1, true>{});
+  return go(QrShape<16, 24, 22, R1, true>{});
 }
 
-bool qf_rows_supported(int64_t n) { return n <= 2048; }
+template <typename T, typename S>
+constexpr size_t qr_smem() { return S::XS ? sizeof(T) * S::CPL * S::THREADS : 0; }
 
-// One wave of resident CTAs, or fewer when every team has a group of rows.
+// One wave of resident CTAs, or fewer when a quarter of an SM's warps (one a scheduler,
+// which its FP64 unit needs no more than) or a whole CTA has a group of rows; a matrix of up
+// to 4096 entries is one CTA's, which writes the gradient itself.
 template <typename T>
 static int qr_grid_t(int64_t m, int64_t n, int team) {
   int64_t grid = 1;
-  qr_with_kernel<T, true>(n, team, [&](auto kern, int rows, int teams) {
+  if (m * n <= 4096) return 1;
+  qr_with_shape<T, true>(m, n, team, [&](auto shape) {
+    using S = decltype(shape);
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, QR_THREADS, 0) != cudaSuccess || occ < 1) {
+    auto kern = qf_rows_kernel<T, S, true>;
+    if (set_smem_once(kern, qr_smem<T, S>()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, S::THREADS, qr_smem<T, S>()) != cudaSuccess ||
+        occ < 1) {
       cudaGetLastError();
       occ = 1;
     }
-    const int64_t step = (int64_t)rows * teams;
+    const int64_t step = (int64_t)S::R * std::max(1, 4 / S::W);
     grid = std::min<int64_t>((m + step - 1) / step, (int64_t)num_sms() * occ);
   });
   return (int)std::max<int64_t>(1, grid);
@@ -279,16 +336,24 @@ int qf_rows_grid(int dtype, int64_t m, int64_t n, int team) {
 
 template <typename T, bool FUSED>
 static cudaError_t launch_rows(int grid, int team, const QrArgs<T>& a, cudaStream_t s) {
+  cudaError_t e = cudaErrorInvalidValue;
   prof_begin(s, FUSED ? "qf_rows_kernel<fused>" : "qf_rows_kernel<eval>");
-  qr_with_kernel<T, FUSED>(a.n, team, [&](auto kern, int, int) { kern<<<grid, QR_THREADS, 0, s>>>(a); });
+  qr_with_shape<T, FUSED>(a.m, a.n, team, [&](auto shape) {
+    using S = decltype(shape);
+    auto kern = qf_rows_kernel<T, S, FUSED>;
+    if (S::XS && (e = set_smem_once(kern, qr_smem<T, S>())) != cudaSuccess) return;
+    kern<<<grid, S::THREADS, qr_smem<T, S>(), s>>>(a);
+    e = cudaGetLastError();
+  });
   prof_end(s);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
-// The last CTA sums the partials itself up to this many bytes of them: about 32 loads a
-// thread, less than a second launch takes.
-constexpr int64_t QR_LAST_BYTES = 64 << 10;
+// The last CTA sums the partials itself up to this many bytes of them and this many columns,
+// one pass of at least two threads a column: 200 x 60 FP64 7.0 us, with a second launch 8.6;
+// 30 x 501, two passes, 12.7 and 8.2.
+constexpr int64_t QR_LAST_BYTES = 64 << 10, QR_LAST_N = 128;
 
 template <typename T>
 kg_status qf_rows_eval(const QfRowsCall<T>& c, cudaStream_t s) {
@@ -320,7 +385,7 @@ kg_status qf_rows_grad(const QfRowsCall<T>& c, cudaStream_t s) {
   a.gx = c.gx;
   a.gA = c.gA;
   a.accumulate = c.accumulate;
-  a.last = c.counter && (int64_t)c.grid * c.n * (int64_t)sizeof(T) <= QR_LAST_BYTES;
+  a.last = c.counter && c.n <= QR_LAST_N && (int64_t)c.grid * c.n * (int64_t)sizeof(T) <= QR_LAST_BYTES;
   cudaError_t e = launch_rows<T, true>(c.grid, c.team, a, s);
   if (e != cudaSuccess) return cuda_fail(e, "qf fused kernel");
   if (c.grid == 1 || a.last) return KG_OK;

@@ -21,7 +21,9 @@ def api(cuda_ok):
 
 # one CTA, the last CTA's sum, a second launch; full and ragged row groups; every team width
 SHAPES = [(1, 1), (7, 31), (8, 33), (9, 64), (65, 97), (300, 128), (1000, 129), (40000, 100), (8, 256),
-          (513, 257), (20001, 255), (70, 512), (3001, 513), (5, 1024), (2049, 1025), (4, 2048), (1999, 2047)]
+          (513, 257), (20001, 255), (70, 512), (3001, 513), (5, 1024), (2049, 1025), (4, 2048), (1999, 2047),
+          (333, 1024), (700, 2048), (1300, 2049), (610, 3000), (5, 3585), (400, 4096), (399, 4097), (301, 5121),
+          (77, 6200), (200, 7169), (310, 8191), (153, 8193), (31, 9300), (305, 10241), (160, 11300), (3, 12288)]
 
 
 @pytest.mark.parametrize("m,n", SHAPES)
@@ -32,8 +34,9 @@ def test_value_and_both_gradients(api, m, n, dtype):
     if dtype == "f32":
         A, x = f32_round(A), f32_round(x)
     f_ref, g_ref, gA_ref = O.quadform_grad(A, x, fbar=-0.75, want_gA=True)
-    # team: FP32 rows of n >= 1024, n % 4 == 0 otherwise run the TMA-streamed kernel
-    p = api.QuadForm(torch.tensor(A, dtype=dt, device="cuda"), arith="native", team=0 if n < 1024 else 256)
+    # team: FP32 problems of n >= 1024, n % 4 == 0 otherwise offer no gradient w.r.t. A
+    team = 0 if n < 1024 or n % 4 else 256 if n <= 2048 else 512
+    p = api.QuadForm(torch.tensor(A, dtype=dt, device="cuda"), arith="native", team=team)
     xt = torch.tensor(x, dtype=dt, device="cuda")
     gA = torch.full((m, n), 0.25, dtype=dt, device="cuda")
     gx = torch.full((n,), 0.5, dtype=dt, device="cuda")
@@ -54,7 +57,8 @@ def test_value_and_both_gradients(api, m, n, dtype):
     p.close()
 
 
-@pytest.mark.parametrize("team,n", [(32, 50), (128, 50), (128, 1000), (256, 50), (256, 1300)])
+@pytest.mark.parametrize("team,n", [(32, 50), (128, 50), (128, 1000), (256, 50), (256, 1300), (512, 50),
+                                   (512, 2000), (512, 4500)])
 @pytest.mark.parametrize("strategy", ["fused", "transpose", "atomic"])
 def test_team_widths_and_strategies(api, team, n, strategy):
     A, x = W.quadform_inputs(n, m=203, seed=team + n)
@@ -115,3 +119,28 @@ def test_float_pair_rows_paths_agree_bitwise(api, m, n, monkeypatch):
         assert o[3] == fe
         if n <= 4096 or o is out[1]:  # (longer rows: the per-load split's gradient is another kernel)
             assert o[0] == f and np.array_equal(o[1], g) and np.array_equal(o[2], g2)
+
+
+@pytest.mark.parametrize("m,n", [(304, 1024), (1001, 1500), (9001, 2048)])
+def test_f32_short_rows_run_several_a_step(api, m, n):
+    # FP32, n % 4 == 0, 1024 <= n <= 2048: the streamed kernel's shapes by the several-rows
+    # kernel; what the streamed kernel refuses stays refused (misaligned x, a gradient w.r.t. A)
+    from paper_2507_13204_gb300 import _lib as L
+    A, x = W.quadform_inputs(n, m=m, seed=m + n)
+    A, x = f32_round(A), f32_round(x)
+    f_ref, g_ref = O.quadform_grad(A, x, fbar=0.5)
+    p = api.QuadForm(torch.tensor(A, dtype=torch.float32, device="cuda"))
+    xt = torch.tensor(x, dtype=torch.float32, device="cuda")
+    seed = torch.tensor(0.5, dtype=torch.float32, device="cuda")
+    f, g = p.grad(xt, seed=seed)
+    fe = p.eval(xt)
+    g2 = p.grad(xt, seed=seed)[1]
+    p.sync()
+    assert rel_scalar(f.item(), f_ref) <= TOL["f32"] and rel_scalar(fe.item(), f_ref) <= TOL["f32"]
+    assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f32"] and torch.equal(g, g2)
+    off = torch.empty(n + 1, dtype=torch.float32, device="cuda")[1:].copy_(xt)
+    for call in (lambda: p.grad(off), lambda: p.grad(xt, gx=off), lambda: p.eval(off),
+                 lambda: p.grad(xt, gdata=torch.empty(m, n, dtype=torch.float32, device="cuda"))):
+        with pytest.raises(L.KGError):
+            call()
+    p.close()
