@@ -9,10 +9,9 @@
 // grid claims items from a device queue head (one atomicAdd per item) until
 // the table is exhausted.
 //   dense tile:  rows [r0, r0 + R): y_i by a row team (4 .. 256 threads,
-//                about 8 columns a thread), ybar_i = 2 y_i, private xbar
-//                partial of the tile written to the instance's partial buffer;
-//                on float-pair copies (pair batches) the rows arrive by bulk
-//                copies into a shared-memory ring, otherwise by plain loads;
+//                about 8 columns a thread), four rows a step, ybar_i = 2 y_i,
+//                private xbar partial of the tile written to the instance's
+//                partial buffer; the next step's rows are prefetched into L2;
 //                pair arithmetic runs on packed column pairs (kg_pair2.cuh);
 //   tet tile:    elements [e0, e0 + T): f_e and the scatter of c_e into gu (zeroed
 //                by a small kernel earlier in the graph): one global reduction per
@@ -108,24 +107,18 @@ __device__ __forceinline__ void prefetch_range_l2(const void* p, size_t bytes) {
   }
 }
 
+// The bytes of rows [r, r + rows) of a dense instance (one step's) into L2.
+__device__ __forceinline__ void prefetch_rows_l2(const BInst& I, int64_t r, int64_t rows, size_t es) {
+  const int64_t pitch = I.prep ? I.pitch : I.n;
+  prefetch_range_l2(static_cast<const unsigned char*>(I.d0) + r * pitch * es, (size_t)(rows * pitch) * es);
+}
+
 // Barrier over the TEAM threads of one row team: the whole CTA for TEAM = BT,
 // otherwise hardware barrier 1 + team (TEAM = 64 or 128).
 template <int TEAM>
 __device__ __forceinline__ void team_barrier(int team) {
   if constexpr (TEAM == BT) __syncthreads();
   else named_barrier(1 + team, TEAM);
-}
-
-// The team's sum of its TW warps' row sums ra[q * 2 + upper] (q < TW), for a
-// team wider than a warp: lane l takes warp l mod TW's and a butterfly over TW
-// lanes (inside the lane's half-warp, so over one row) gives every lane the
-// same total, with log2(TW) pair additions a thread instead of TW - 1.
-template <int TW>
-__device__ __forceinline__ Acc team_warps_sum(const Acc* ra, int lane, bool upper) {
-  Acc k = ra[(lane & (TW - 1)) * 2 + (upper ? 1 : 0)];
-#pragma unroll
-  for (int o = TW / 2; o > 0; o >>= 1) k = acc_add(k, shfl_xor_acc2(k, o));
-  return k;
 }
 
 // Rows [w.start, w.start + w.count) of a dense instance in native arithmetic, B_NR rows per
@@ -156,6 +149,10 @@ __device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp,
   const int64_t r1 = w.start + w.count;
   const int steps = (w.count + R * NT - 1) / (R * NT);
   for (int c = 0; c < steps; ++c) {
+    if (tid == 0 && c + 1 < steps) {
+      const int64_t rn = w.start + (int64_t)(c + 1) * R * NT;
+      prefetch_rows_l2(I, rn, r1 - rn < R * NT ? r1 - rn : R * NT, sizeof(T));
+    }
     const int64_t r0 = w.start + ((int64_t)c * NT + team) * R;
     const int rows = r0 < r1 ? (int)(r1 - r0 < R ? r1 - r0 : R) : 0;
     const T* Ar = A + (rows > 0 ? r0 : w.start) * (int64_t)n + lt;
@@ -227,59 +224,9 @@ __device__ double dense_tile(const BInst& I, const BItem& w, unsigned char* wsp,
   return f;
 }
 
-// ---- dense tiles of pair batches: two rows per team and step, columns in packed pairs ----
+// ---- dense tiles of pair batches: B_NR rows per team and step, columns in packed pairs ----
 // Team thread lt holds the column pairs jp = lt + k TEAM, k < KM (odd n: the last
-// pair's second column is a zero).  Rows r and r + NT of a step are reduced
-// together: one transposed butterfly for both dot products (the first exchange
-// hands each half of the team one row), so the reduction and, for teams wider
-// than a warp, the barrier are paid once per two rows.  `sync` runs between the
-// warps' sums and their use; it is the barrier of teams wider than a warp, and
-// true from it (on all threads) ends the tile.
-template <int TEAM, int KM, typename Sync>
-__device__ __forceinline__ bool pair_two_rows(const Pair2 (&av)[2][KM], int kp, const Pair2 (&xp)[KM],
-                                              Acc2 (&xb)[KM], Acc& fp, const bool (&vr)[2], double* red,
-                                              int par, const Sync& sync) {
-  constexpr int W = TEAM < 32 ? TEAM : 32;  // lanes of the team inside one warp
-  constexpr int TW = TEAM > 32 ? TEAM / 32 : 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = threadIdx.x / TEAM;
-  const bool upper = (lane & (W / 2)) != 0;  // keeps the second row
-  Acc2 y2[2] = {acc2_prod(av[0][0], xp[0]), acc2_prod(av[1][0], xp[0])};
-#pragma unroll
-  for (int k = 1; k < KM; ++k) {
-    if (k < kp) {
-      acc2_fma(y2[0], av[0][k], xp[k]);
-      acc2_fma(y2[1], av[1][k], xp[k]);
-    }
-  }
-  const Acc y[2] = {acc2_sum(y2[0]), acc2_sum(y2[1])};
-  Acc keep = upper ? y[1] : y[0];
-  keep = acc_add(keep, shfl_xor_acc2(upper ? y[0] : y[1], W / 2));
-#pragma unroll
-  for (int o = W / 4; o > 0; o >>= 1) keep = acc_add(keep, shfl_xor_acc2(keep, o));
-  // two buffers: step c + 1 writes the other while step c's sums are read
-  Acc* ra = reinterpret_cast<Acc*>(red) + par * 2 * BW + team * 2 * TW;  // [TW][2]
-  if constexpr (TEAM > 32)
-    if ((lane & (W / 2 - 1)) == 0) ra[(warp % TW) * 2 + (upper ? 1 : 0)] = keep;
-  if (sync()) return true;
-  if constexpr (TEAM > 32) keep = team_warps_sum<TW>(ra, lane, upper);
-  const Acc other = shfl_xor_acc2(keep, W / 2);
-  const Acc yt[2] = {upper ? other : keep, upper ? keep : other};
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    if (vr[q]) {
-      const Pair yq = acc_pair(yt[q]);
-      if (TEAM <= 32 || warp % TW == 0) {  // f: the team's first warp
-        const Pair y2q = pair_mul(yq, yq);
-        fp = acc_add(fp, Acc{y2q.h, y2q.l});
-      }
-      const Pair2 yb = pair2_dup(Pair{2.0f * yq.h, 2.0f * yq.l});  // exact
-#pragma unroll
-      for (int k = 0; k < KM; ++k)
-        if (k < kp) acc2_fma(xb[k], av[q][k], yb);
-    }
-  }
-  return false;
-}
+// pair's second column is a zero).
 
 // x in float pairs for the thread's column pairs.
 template <int TEAM, int KM>
@@ -297,15 +244,15 @@ __device__ __forceinline__ void pair_load_x(const BInst& I, Pair2 (&xp)[KM], Acc
 }
 
 // The end of a pair tile: the teams' partials combined in team order, two column
-// pairs of every thread at a time through RING_WS entries (outside the ring, into
-// which the next item's copies may be landing), and the tile's f.
-constexpr int RING_WS = 1024;  // Acc entries of the combine buffer (8 KB)
+// pairs of every thread at a time through B_WS entries, and the tile's f (fp: the
+// thread's sum, zero where it counts no row).
+constexpr int B_WS = 1024;  // Acc entries of the combine buffer (8 KB)
 
 template <int TEAM, int KM>
 __device__ double pair_tile_end(const BInst& I, const BItem& w, const Acc2 (&xb)[KM], Acc fp,
                                 unsigned char* wsp, double* red) {
   constexpr int NT = BT / TEAM, H = 2;
-  static_assert(2 * BT * H <= RING_WS, "the combine buffer holds two column pairs of all threads");
+  static_assert(2 * BT * H <= B_WS, "the combine buffer holds two column pairs of all threads");
   const int tid = threadIdx.x, lt = tid % TEAM, team = tid / TEAM;
   const int np2 = I.pitch / 2;
   auto entry = [](Acc2 c) {
@@ -343,168 +290,127 @@ __device__ double pair_tile_end(const BInst& I, const BItem& w, const Acc2 (&xb)
     }
   }
   Acc* ra = reinterpret_cast<Acc*>(red);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) fp = acc_add(fp, shfl_xor_acc2(fp, o));
   __syncthreads();
-  if (lt == 0) ra[team] = fp;
+  if ((tid & 31) == 0) ra[tid >> 5] = fp;
   __syncthreads();
   Acc tot = ra[0];
-  for (int t2 = 1; t2 < NT; ++t2) tot = acc_add(tot, ra[t2]);
+  for (int q = 1; q < BW; ++q) tot = acc_add(tot, ra[q]);
   __syncthreads();
   return acc_to_double(tot);
 }
 
-// Rows of a pair-batch instance without a float-pair copy: FP64 data, split on
-// every load, in the ring path's order of operations (the same bits).
-template <int TEAM>
-__device__ double dense_tile_split(const BInst& I, const BItem& w, unsigned char* wsp, double* red, bool& bad) {
-  constexpr int NT = BT / TEAM, KM = B_CPT / 2;
-  const int lt = threadIdx.x % TEAM, team = threadIdx.x / TEAM;
-  const double* __restrict__ A = static_cast<const double*>(I.d0);
-  const int n = I.n, kp = (I.pitch / 2 + TEAM - 1) / TEAM;
-  Pair2 xp[KM];
-  Acc2 xb[KM];
-  pair_load_x<TEAM>(I, xp, xb, bad);
-  Acc fp = acc_zero();
-  const int64_t r1 = w.start + w.count;
-  const int steps = (w.count + 2 * NT - 1) / (2 * NT);
-  for (int c = 0; c < steps; ++c) {
-    const int64_t row0 = w.start + (int64_t)c * 2 * NT;
-    const int64_t rr[2] = {row0 + team, row0 + NT + team};
-    const bool vr[2] = {rr[0] < r1, rr[1] < r1};
-    Pair2 av[2][KM];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const double* Ar = A + (vr[q] ? rr[q] : w.start) * (int64_t)n;
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        const int j = 2 * (lt + k * TEAM);
-        const double v0 = vr[q] && j < n ? __ldcs(Ar + j) : 0.0;
-        const double v1 = vr[q] && j + 1 < n ? __ldcs(Ar + j + 1) : 0.0;
-        av[q][k] = pair2_of(split_f64(v0), split_f64(v1));
-      }
-    }
-    pair_two_rows<TEAM>(av, kp, xp, xb, fp, vr, red, c & 1, [&] {
-      if constexpr (TEAM > 32) team_barrier<TEAM>(team);
-      return false;
-    });
-    if ((c & 7) == 7) {
-#pragma unroll
-      for (int k = 0; k < KM; ++k) acc2_renorm(xb[k]);
-    }
-  }
-  __syncthreads();
-  return pair_tile_end<TEAM>(I, w, xb, fp, wsp, red);
-}
-
-// ---- ... on float-pair copies: rows staged by bulk copies ----
-// A tile's rows are contiguous, so its data arrives by 1-D bulk copies (TMA)
-// into a ring of RING_S shared-memory slots, one iteration group (the 2 NT rows
-// one step of the teams takes, at most 32 KB: 4 column pairs a team thread) a
-// slot, while the teams compute on the slot before: bytes in flight without
-// registers.  Rows of a copy are `pitch` entries, so they start on 16-byte
-// boundaries.  All threads count the chunks the CTA has consumed (g), which
-// gives each slot's barrier phase across tiles; thread 0, the only one that
-// issues, counts the chunks issued (iss).  When a tile has no chunk left to
-// issue, the slots it frees take the first chunks of the CTA's next item
-// (claimed when this one started) if that is a ring tile too, so the copies
-// run on across the tile boundary.
-constexpr int RING_S = 3;
-constexpr int RING_SLOT = 32768;
-
-struct Ring {
-  unsigned char* slots;  // RING_S * RING_SLOT bytes
-  uint64_t* full;        // RING_S barriers: a slot's copy has landed
-};
-
-// The CTA's next item as ring chunks (thread 0 only); nchunks 0: not a ring tile.
-struct RingNext {
-  const double* src;   // its first row
-  int64_t chunk;       // entries a chunk (2 NT pitch)
-  int64_t total;       // entries of the item (count pitch)
-  int nchunks;
-};
-
-__device__ __forceinline__ void ring_issue(const Ring& R, uint32_t g, const void* src, size_t bytes) {
-  const int slot = (int)(g % RING_S);
-  mbar_arrive_expect_tx(&R.full[slot], (uint32_t)bytes);
-  tma_load_1d(R.slots + slot * RING_SLOT, src, (uint32_t)bytes, &R.full[slot]);
-}
-
-// Rows of an instance with a copy, read from the ring.  Returns the tile's f;
-// sets `failed` (on all threads) when a copy did not land within the wait limit,
-// after waiting for the CTA's other copies in flight.
-// KP > 0: the column pairs per team thread, ceil(pitch / 2 / TEAM), fixed at
-// compile time (no test but the last pair's); 0: at run time.
-template <int TEAM, int KP>
-__device__ double dense_tile_ring(const BInst& I, const BItem& w, const Ring& R, uint32_t& g,
-                                  uint32_t& iss, const RingNext& nx, unsigned char* wsp, double* red,
-                                  bool& bad, bool& failed) {
-  const int tid = threadIdx.x;
-  const double* __restrict__ A = static_cast<const double*>(I.d0);  // float pairs, 8 bytes an entry
-  constexpr int NT = BT / TEAM, KM = KP ? KP : B_CPT / 2;
+// Rows [w.start, w.start + w.count) of an instance of a pair batch, as the native tiles:
+// B_NR rows per team and step, their loads together (up to 64 KB a CTA in flight), one
+// transposed butterfly and, for teams wider than a warp, one barrier for all of them; the
+// next step's rows are prefetched into L2.  PREP: from the float-pair copy, 16 bytes a column
+// pair; otherwise FP64 data, split on every load, in the same order (the same bits).
+// KP > 0: ceil(pitch / 2 / TEAM) column pairs a thread, no test but the last one's; 0: at run
+// time.  Returns the tile's f.
+// Bound by instruction issue and the loads' latency, 2 CTAs an SM.  Against two rows a step
+// through a shared-memory ring of bulk copies (a CTA barrier a step, a shared-memory pass):
+// 128 dense (n to 2048) + 16 tet instances 178 -> 156 us, 32 + 4 49.7 -> 43.0, 16 + 2
+// 45.3 -> 33.0; 4096 + 512 4.13 -> 3.51 ms (17.87 GB, 0.75 of the copy peak).
+template <int TEAM, int KP, bool PREP>
+__device__ double dense_tile_pair(const BInst& I, const BItem& w, unsigned char* wsp, double* red, bool& bad) {
+  constexpr int R = B_NR, WL = TEAM < 32 ? TEAM : 32, GL = WL / R;  // lanes of a row's total in a warp
+  constexpr int NT = BT / TEAM, KM = KP ? KP : B_CPT / 2, TW = TEAM > 32 ? TEAM / 32 : 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lt = tid % TEAM, team = tid / TEAM;
-  const int np = I.pitch, np2 = np / 2;
-  const int kp = KP ? KP : (np2 + TEAM - 1) / TEAM;
-  // pair k of this thread is in the row: compile-time true below the last one
+  const int n = I.n, np2 = I.pitch / 2;
   auto in_row = [&](int k) { return (KP && k < KP - 1) || lt + k * TEAM < np2; };
   Pair2 xp[KM];
   Acc2 xb[KM];
   pair_load_x<TEAM>(I, xp, xb, bad);
   Acc fp = acc_zero();
+  const int row = (lane % WL) / GL;  // whose total this lane holds
+  const bool counts = lane % GL == 0 && (TEAM <= 32 || warp % TW == 0);
   const int64_t r1 = w.start + w.count;
-  const int nchunks = (w.count + 2 * NT - 1) / (2 * NT);
-  auto chunk_src = [&](int c) { return A + (w.start + (int64_t)c * 2 * NT) * np; };
-  auto chunk_bytes = [&](int c) {
-    const int64_t left = r1 - (w.start + (int64_t)c * 2 * NT);
-    return (size_t)(left < 2 * NT ? left : 2 * NT) * np * 8;
-  };
-  const uint32_t g0 = g;  // this tile's chunk c is the CTA's chunk g0 + c
-  if (tid == 0)  // (the first ones may have been issued by the tile before)
-    for (; (int)(iss - g0) < nchunks && iss - g0 < (uint32_t)RING_S; ++iss)
-      ring_issue(R, iss, chunk_src((int)(iss - g0)), chunk_bytes((int)(iss - g0)));
-  for (int c = 0; c < nchunks; ++c) {
-    const int slot = (int)(g % RING_S);
-    const bool ok = mbar_wait_bounded(&R.full[slot], (g / RING_S) & 1u);
-    const float4* buf = reinterpret_cast<const float4*>(R.slots + slot * RING_SLOT);
-    const int64_t row0 = w.start + (int64_t)c * 2 * NT;
-    const bool vr[2] = {ok && row0 + team < r1, ok && row0 + NT + team < r1};
-    Pair2 av[2][KM];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const float4* Ar = buf + (q * NT + team) * np2;
-#pragma unroll
-      for (int k = 0; k < KM; ++k)
-        av[q][k] = vr[q] && in_row(k) ? pair2_load(Ar + lt + k * TEAM) : Pair2{f2_zero(), f2_zero()};
+  const int steps = (w.count + R * NT - 1) / (R * NT);
+  for (int c = 0; c < steps; ++c) {
+    if (tid == 0 && c + 1 < steps) {
+      const int64_t rn = w.start + (int64_t)(c + 1) * R * NT;
+      prefetch_rows_l2(I, rn, r1 - rn < R * NT ? r1 - rn : R * NT, 8);
     }
-    // one CTA barrier a chunk: the slot's entries are in registers by then, so the
-    // slot is refilled behind it; it also publishes the warps' sums
-    const bool lost = pair_two_rows<TEAM>(av, kp, xp, xb, fp, vr, red, c & 1, [&] {
-      if (__syncthreads_or(!ok)) return true;
-      if (tid == 0 && iss - g0 < (uint32_t)(nchunks + nx.nchunks)) {
-        const int k = (int)(iss - g0);
-        if (k < nchunks) {
-          ring_issue(R, iss, chunk_src(k), chunk_bytes(k));
-        } else {  // the next item's chunk k - nchunks
-          const int64_t e0 = (int64_t)(k - nchunks) * nx.chunk, left = nx.total - e0;
-          ring_issue(R, iss, nx.src + e0, (size_t)(left < nx.chunk ? left : nx.chunk) * 8);
+    const int64_t r0 = w.start + ((int64_t)c * NT + team) * R;
+    const int rows = r0 < r1 ? (int)(r1 - r0 < R ? r1 - r0 : R) : 0;
+    const int64_t first = rows > 0 ? r0 : w.start;
+    Pair2 av[R][KM];
+    if constexpr (PREP) {
+      const ulonglong2* Ar = static_cast<const ulonglong2*>(I.d0) + first * np2 + lt;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {
+          const ulonglong2 q = r < rows && in_row(k) ? __ldcs(Ar + k * TEAM) : make_ulonglong2(0ull, 0ull);
+          av[r][k] = Pair2{F2{q.x}, F2{q.y}};
         }
-        ++iss;
+        Ar += np2;
       }
-      return false;
-    });
-    if (lost) {
-      if (tid == 0)  // do not go on with a copy into this CTA's shared memory in flight
-        for (uint32_t h = g; h < iss; ++h) mbar_wait_bounded(&R.full[h % RING_S], (h / RING_S) & 1u);
-      failed = true;
-      __syncthreads();
-      return 0.0;
+    } else {
+      const double* Ar = static_cast<const double*>(I.d0) + first * n;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {
+          const int j = 2 * (lt + k * TEAM);
+          const double v0 = r < rows && j < n ? __ldcs(Ar + j) : 0.0;
+          const double v1 = r < rows && j + 1 < n ? __ldcs(Ar + j + 1) : 0.0;
+          av[r][k] = pair2_of(split_f64(v0), split_f64(v1));
+        }
+        Ar += n;
+      }
     }
-    ++g;
-    if ((c & 7) == 7) {
+    Acc d[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      Acc2 y = acc2_prod(av[r][0], xp[0]);
+#pragma unroll
+      for (int k = 1; k < KM; ++k) acc2_fma(y, av[r][k], xp[k]);
+      d[r] = acc2_sum(y);
+    }
+    int o = WL / 2;
+#pragma unroll
+    for (int q = R / 2; q > 0; q >>= 1, o >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < q; ++i)
+        d[i] = acc_add(up ? d[i + q] : d[i], shfl_xor_acc2(up ? d[i] : d[i + q], o));
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) d[0] = acc_add(d[0], shfl_xor_acc2(d[0], o));
+    Acc tot = d[0];
+    if constexpr (TEAM > 32) {
+      static_assert(TW <= GL, "the butterfly over the warps stays inside a row's lanes");
+      Acc* rt = reinterpret_cast<Acc*>(red) + ((c & 1) * BW + team * TW) * R;  // [TW][R]
+      if (lane % GL == 0) rt[(warp % TW) * R + row] = tot;
+      team_barrier<TEAM>(team);
+      tot = rt[(lane % TW) * R + row];
+#pragma unroll
+      for (int q = TW / 2; q > 0; q >>= 1) tot = acc_add(tot, shfl_xor_acc2(tot, q));
+    }
+    const Pair y = acc_pair(tot);  // rows past the tile's end: zero
+    if (TEAM <= 32 || warp % TW == 0) {
+      const Pair y2 = pair_mul(y, y);
+      fp = acc_add(fp, Acc{y2.h, y2.l});
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int src = (lane & ~(WL - 1)) + r * GL;
+      const Pair2 yb = pair2_dup(Pair{2.0f * __shfl_sync(0xffffffffu, y.h, src),
+                                      2.0f * __shfl_sync(0xffffffffu, y.l, src)});  // exact
+#pragma unroll
+      for (int k = 0; k < KM; ++k) acc2_fma(xb[k], av[r][k], yb);
+    }
+    if ((c & 3) == 3) {
+      acc_renorm(fp);
 #pragma unroll
       for (int k = 0; k < KM; ++k) acc2_renorm(xb[k]);
     }
   }
-  return pair_tile_end<TEAM>(I, w, xb, fp, wsp, red);
+  __syncthreads();
+  return pair_tile_end<TEAM>(I, w, xb, counts ? fp : acc_zero(), wsp, red);
 }
 
 // Elements [w.start, w.start + w.count) of a tet instance; returns the tile's f.
@@ -620,35 +526,23 @@ struct NativeTile {
   }
 };
 
-struct SplitTile {
+template <bool PREP>
+struct PairTile {
   const BInst& I;
   const BItem& w;
   unsigned char* wsp;
   double* red;
   bool& bad;
-  template <int TEAM>
-  __device__ __forceinline__ double run() const { return dense_tile_split<TEAM>(I, w, wsp, red, bad); }
-};
-
-struct RingTile {
-  const BInst& I;
-  const BItem& w;
-  const Ring& R;
-  uint32_t &g, &iss;
-  const RingNext& nx;
-  unsigned char* wsp;
-  double* red;
-  bool &bad, &failed;
   // the team is the smallest power of two (>= 4) with 4 column pairs a thread, so
   // above 4 threads a team thread has 3 or 4
   template <int TEAM>
   __device__ __forceinline__ double run() const {
-    if constexpr (TEAM > 4) {
+    if constexpr (TEAM > 4 && PREP) {
       const int kp = (I.pitch / 2 + TEAM - 1) / TEAM;
-      if (kp == 4) return dense_tile_ring<TEAM, 4>(I, w, R, g, iss, nx, wsp, red, bad, failed);
-      if (kp == 3) return dense_tile_ring<TEAM, 3>(I, w, R, g, iss, nx, wsp, red, bad, failed);
+      if (kp == 4) return dense_tile_pair<TEAM, 4, PREP>(I, w, wsp, red, bad);
+      if (kp == 3) return dense_tile_pair<TEAM, 3, PREP>(I, w, wsp, red, bad);
     }
-    return dense_tile_ring<TEAM, 0>(I, w, R, g, iss, nx, wsp, red, bad, failed);
+    return dense_tile_pair<TEAM, 0, PREP>(I, w, wsp, red, bad);
   }
 };
 
@@ -692,51 +586,54 @@ __device__ void sum_columns(const BInst& I, int j0, int cols) {
 
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
-  // PAIR: [log table][ring: RING_S slots][combine buffer][red][ring barriers].
-  // Otherwise [wsp][red].
+  // [PAIR: log table][combine buffer][red]
   extern __shared__ __align__(16) unsigned char smem[];
   float4* tab = reinterpret_cast<float4*>(smem);
-  unsigned char* slots = smem + (PAIR ? kLogTableSize * sizeof(float4) : 0);
-  unsigned char* rws = slots + (PAIR ? (size_t)RING_S * RING_SLOT : 0);  // combine buffer
-  double* red = reinterpret_cast<double*>(rws + (PAIR ? RING_WS * sizeof(Acc) : (size_t)BT * B_CPT * 8));
-  Ring R{slots, reinterpret_cast<uint64_t*>(red + 64)};
-  uint32_t g = 0, iss = 0;  // ring chunks consumed by this CTA; issued (thread 0)
+  unsigned char* wsp = smem + (PAIR ? kLogTableSize * sizeof(float4) : 0);
+  double* red = reinterpret_cast<double*>(wsp + (PAIR ? B_WS * sizeof(Acc) : (size_t)BT * B_CPT * 8));
   __shared__ int s_item, s_last;
+  // PAIR: the item and its instance, registers being short in the tiles.  The native kernels
+  // hold them in registers (32 dense + 4 tet FP32 instances: 29.0 us, 33.3 in shared memory)
+  __shared__ BItem s_w;
+  __shared__ BInst s_I;
   const int tid = threadIdx.x;
   if constexpr (PAIR) {
     for (int i = tid; i < kLogTableSize; i += BT) tab[i] = a.logtab[i];
-    if (tid == 0) {
-      for (int i = 0; i < RING_S; ++i) mbar_init(&R.full[i], 1);
-      fence_barrier_init();
-    }
   }
-  bool bad = false, failed = false;
-  // items are claimed one ahead: the next one's first copies can be issued
-  // during this one (pair batches)
+  bool bad = false;
+  // items are claimed one ahead: the next one's first rows go into L2 during this one
   if (tid == 0) s_item = (int)atomicAdd(&a.head[0], 1u);
   __syncthreads();
   int it = s_item;
   for (;;) {
     __syncthreads();  // every thread has read s_item
     if (it >= a.nitems) break;
-    RingNext nx{nullptr, 0, 0, 0};
     if (tid == 0) {
       const int nit = (int)atomicAdd(&a.head[0], 1u);
       s_item = nit;
-      if (PAIR && nit < a.nitems) {
+      if (nit < a.nitems) {
         const BItem wn = a.items[nit];
         const BInst& In = a.insts[wn.inst];
-        if (In.kind == BK_DENSE && In.prep && wn.tile >= 0) {
-          const int64_t rows = 2 * (BT / In.team);  // a step's
-          nx.src = static_cast<const double*>(In.d0) + wn.start * (int64_t)In.pitch;
-          nx.chunk = rows * In.pitch;
-          nx.total = (int64_t)wn.count * In.pitch;
-          nx.nchunks = (int)((wn.count + rows - 1) / rows);
+        if (In.kind == BK_DENSE && wn.tile >= 0) {
+          const int64_t rows = B_NR * (BT / In.team);
+          prefetch_rows_l2(In, wn.start, rows < wn.count ? rows : wn.count, sizeof(T));
         }
       }
     }
-    const BItem w = a.items[it];
-    const BInst I = a.insts[w.inst];
+    BItem wr;
+    BInst Ir;
+    if constexpr (PAIR) {
+      if (tid == 32) {
+        s_w = a.items[it];
+        s_I = a.insts[s_w.inst];
+      }
+      __syncthreads();
+    } else {
+      wr = a.items[it];
+      Ir = a.insts[wr.inst];
+    }
+    const BItem& w = PAIR ? s_w : wr;
+    const BInst& I = PAIR ? s_I : Ir;
     if (w.tile < 0) {
       // every tile item comes before the sum items and is held by a running CTA (this
       // one has none left), so the wait ends
@@ -765,32 +662,20 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
       it = s_item;
       continue;
     }
-    // the tile's contiguous data into L2 while the first loads are in flight (not
-    // for the ring's tiles: their copies stream it, and whole-tile prefetches of
-    // every CTA exceed L2 and are evicted before use)
-    if (tid == 0) {
-      if (I.kind == BK_DENSE) {
-        if (!(PAIR && I.prep))
-          prefetch_range_l2(static_cast<const T*>(I.d0) + w.start * (int64_t)I.n,
-                            (size_t)w.count * I.n * sizeof(T));
-      } else {
-        prefetch_range_l2(static_cast<const int4*>(I.d0) + w.start, (size_t)w.count * 16);
-        prefetch_range_l2(static_cast<const T*>(I.d1) + w.start * 12, (size_t)w.count * 12 * sizeof(T));
-      }
+    // a tet tile's contiguous data into L2 while the first loads are in flight (dense tiles
+    // prefetch a step ahead: whole tiles of every CTA exceed L2 and are evicted before use)
+    if (tid == 0 && I.kind == BK_TET) {
+      prefetch_range_l2(static_cast<const int4*>(I.d0) + w.start, (size_t)w.count * 16);
+      prefetch_range_l2(static_cast<const T*>(I.d1) + w.start * 12, (size_t)w.count * 12 * sizeof(T));
     }
     double ft;
     const bool prep = PAIR && I.prep;
     if (I.kind == BK_DENSE) {
-      if constexpr (PAIR) {
-        ft = prep ? with_team(I.team, RingTile{I, w, R, g, iss, nx, rws, red, bad, failed})
-                  : with_team(I.team, SplitTile{I, w, rws, red, bad});
-        if (failed) {  // a copy did not land: this CTA leaves the queue
-          if (tid == 0) set_error(a.err, ERRBIT_TIMEOUT);
-          break;
-        }
-      } else {
-        ft = with_team(I.team, NativeTile<T>{I, w, rws, red});
-      }
+      if constexpr (PAIR)
+        ft = prep ? with_team(I.team, PairTile<true>{I, w, wsp, red, bad})
+                  : with_team(I.team, PairTile<false>{I, w, wsp, red, bad});
+      else
+        ft = with_team(I.team, NativeTile<T>{I, w, wsp, red});
     } else {
       if (a.warpc)
         ft = prep ? tet_tile<T, PAIR, true, true>(I, w, tab, a.K, red, bad)
@@ -853,9 +738,7 @@ using namespace kg;
 namespace {
 
 size_t batched_smem(bool pair) {
-  if (pair)
-    return kLogTableSize * sizeof(float4) + (size_t)RING_S * RING_SLOT + RING_WS * sizeof(Acc) +
-           64 * sizeof(double) + RING_S * sizeof(uint64_t);
+  if (pair) return kLogTableSize * sizeof(float4) + B_WS * sizeof(Acc) + 64 * sizeof(double);
   return (size_t)BT * B_CPT * 8 + 64 * sizeof(double);
 }
 
@@ -988,7 +871,7 @@ Plan make_plan(const std::vector<kg_problem*>& probs, const std::vector<const vo
       P.tet_ids.push_back(idx);
     }
     if (cap > 0.0) {  // whole steps of the row teams or of the CTA's threads, 4 at least
-      const int64_t unit = I.kind == BK_DENSE ? (pair ? 2 : B_NR) * (BT / I.team) : BT;
+      const int64_t unit = I.kind == BK_DENSE ? B_NR * (BT / I.team) : BT;
       const int64_t most = (int64_t)(cap / item_cost(p, unit, es)) * unit;
       per = std::min(per, std::max(most, 4 * unit));
     }
@@ -1074,13 +957,6 @@ kg_status devplan_alloc(DevPlan& D, Plan& P, cudaStream_t s) {
                            cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return cuda_fail(e, "batch set-up");
   return KG_OK;
-}
-
-// The pair kernels' shared memory (the ring) is above the 48 KB default: raise
-// their limit before the first occupancy query or launch.
-cudaError_t batched_smem_attrs() {
-  return cudaFuncSetAttribute(batched_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)batched_smem(true));
 }
 
 int batched_grid(bool pair) {
@@ -1234,8 +1110,8 @@ kg_status autotune(kg_batch* b, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   std::map<std::string, int> cache = cache_read();
   bool dirty = false;
-  // "k4": dense tiles of pair batches in packed column pairs through a ring of bulk copies
-  const std::string prefix = b->gpu + "|k4|" + (b->dtype == KG_F64 ? "f64" : "f32") + "|" +
+  // "k5": dense tiles take four rows a step
+  const std::string prefix = b->gpu + "|k5|" + (b->dtype == KG_F64 ? "f64" : "f32") + "|" +
                              (b->pair ? "pair" : "native") + "|";
   const std::vector<int> dense_cands{4, 8, 16, 32, 64, 128, 256}, tet_cands{1024, 2048, 4096, 8192, 16384};
   std::map<std::pair<int, int>, std::vector<int>> sample;
@@ -1390,10 +1266,6 @@ kg_status kg_batch_create(kg_batch** out, kg_problem* const* probs, int count,
       b->prep[i] = q;
       budget -= bytes;
     }
-  }
-  if (rc == KG_OK) {
-    cudaError_t e = batched_smem_attrs();
-    if (e != cudaSuccess) rc = cuda_fail(e, "kg_batch_create: kernel attributes");
   }
   if (rc == KG_OK) {
     b->gpu = gpu_name();
