@@ -845,18 +845,23 @@ def make_workload(name: str, arith: str, size: int = 0, rows: int = 0, strategy:
 # fingerprint it was taken with; after any change to them the field is null until re-measured.
 _CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2507_13204_gb300", "csrc")
 _TRAFFIC = {
-    ('dense', 'f64'): (816462080, ['quadform_pair.cu', 'kg_pair.cuh', 'kg_device.cuh'],
-                       '78d8ecfe03606423'),
-    ('dense32', 'f32'): (405942784, ['quadform_f32.cu', 'kg_pair.cuh', 'kg_device.cuh'],
-                         '801a828817b83d19'),
-    ('tet', 'f64'): (711157760, ['tet_pair.cu', 'kg_tet_elem.cuh', 'kg_pair.cuh', 'kg_device.cuh'],
-                     '33085ea1051816f5'),
-    ('tet32', 'f32'): (469459712, ['tet_tile.cu', 'kg_tet_elem.cuh', 'kg_pair.cuh', 'kg_device.cuh'],
-                       '166f724fdbe0f6dd'),
-    ('tetcsr', 'f64'): (787957760, ['tet_tile.cu', 'kg_tet_elem.cuh', 'kg_pair.cuh', 'kg_device.cuh'],
-                        '166f724fdbe0f6dd'),
-    ('batched', 'f64'): (18503473152, ['batched.cu', 'kg_tet_elem.cuh', 'kg_pair.cuh', 'kg_device.cuh'],
-                         '2bc7e7b9c7b540ad'),
+    ('dense', 'f64'): (810304256, ['quadform_pair.cu', 'kg_pair2.cuh', 'kg_pair.cuh',
+                                   'kg_device.cuh'],
+                       '34dd7c3a696dbd8d'),
+    ('dense32', 'f32'): (406196992, ['quadform_f32.cu', 'kg_pair.cuh', 'kg_device.cuh'],
+                         '37122eb7736d090a'),
+    ('tet', 'f64'): (714715392, ['tet_pair.cu', 'kg_tet_elem.cuh', 'kg_pair2.cuh',
+                                 'kg_pair.cuh', 'kg_device.cuh'],
+                     '143fcd4f52adcd1d'),
+    ('tet32', 'f32'): (469544448, ['tet_tile.cu', 'kg_tet_elem.cuh', 'kg_pair2.cuh',
+                                   'kg_pair.cuh', 'kg_device.cuh'],
+                       'a33a8a9047986e28'),
+    ('tetcsr', 'f64'): (789700864, ['tet_tile.cu', 'kg_tet_elem.cuh', 'kg_pair2.cuh',
+                                    'kg_pair.cuh', 'kg_device.cuh'],
+                        'a33a8a9047986e28'),
+    ('batched', 'f64'): (19266515968, ['batched.cu', 'kg_tet_elem.cuh', 'kg_pair2.cuh',
+                                       'kg_pair.cuh', 'kg_device.cuh'],
+                         '93a88286d21cdcbf'),
 }
 
 
