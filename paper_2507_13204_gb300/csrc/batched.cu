@@ -823,8 +823,9 @@ constexpr int B_SUM_TILES = 16;
 // No tile is larger than a CTA's share of the batch / B_SHARE, so that a batch of few
 // large instances still fills the grid: the autotuner's tiles (up to 256 rows, right for
 // batches of thousands) gave 128 dense and 16 tet instances two items a CTA.  Measured on
-// that batch, 630 MB: shares of 2, 3, 4 and 6 take 183, 174, 172 and 185 us (tuned tiles
-// of 128 rows), 172, 171, 174 and 183 us (of 64).
+// that batch, 630 MB, shares of 2, 3, 4 and 6: float pairs 157, 156, 159 and 163 us, FP32
+// 80, 82, 85 and 93, native FP64 497, 458, 427 and 422; 32 + 4 and 16 + 2 instances do not
+// differ (their tiles are at the 4 steps make_plan leaves).
 constexpr int B_SHARE = 3;
 
 // prep[i]: the float-pair copy of problem i's A (dense) or G (tet) that the
@@ -1099,7 +1100,7 @@ kg_status time_plan(kg_batch* b, const std::vector<int>& ids, const Tuning& tu, 
 // fastest wins.  A smaller sample favours small tiles for want of parallelism
 // that the whole batch has (make_plan cuts them to a CTA's share anyway): there
 // the largest within 10% wins (on 128 dense and 16 tet instances the fastest
-// ones made tiles of 16 rows and 187 us, these 171).  Choices are cached by GPU name, kind, dtype, arithmetic and bucket.
+// ones made tiles of 16 rows and 187 us, these 171, both with tiles of two rows a step).  Choices are cached by GPU name, kind, dtype, arithmetic and bucket.
 kg_status autotune(kg_batch* b, cudaStream_t s) {
   std::map<std::pair<int, int>, std::vector<int>> groups;  // (kind, bucket) -> instance ids
   for (int i = 0; i < (int)b->probs.size(); ++i) {
