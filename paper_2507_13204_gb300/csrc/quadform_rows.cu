@@ -154,12 +154,14 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
 #pragma unroll
       for (int o = WG / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     }
-    if (row >= rows) tot = T(0);  // past the end: 0 times an infinite x is no row's value
+    // past the end there is no row: neither 0 times an infinite x nor, below, an infinite seed
+    // times 0 is one's value
+    if (row >= rows) tot = T(0);
     if (W == 1 || warp % W == 0) fsum.add(tot);  // one warp of the team: an FP64 instruction a row
     if constexpr (!FUSED) {
       if (a.y && row < rows && lane % G == 0 && (W == 1 || warp % W == 0)) a.y[r0 + row] = tot;
     } else {
-      const T ybl = fb2 * tot;
+      const T ybl = row < rows ? fb2 * tot : T(0);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const T yb = R == 1 ? ybl : __shfl_sync(0xffffffffu, ybl, r * G);

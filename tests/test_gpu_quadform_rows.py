@@ -144,3 +144,26 @@ def test_f32_short_rows_run_several_a_step(api, m, n):
         with pytest.raises(L.KGError):
             call()
     p.close()
+
+
+@pytest.mark.parametrize("fbar", [np.inf, -np.inf])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("m,n", [(9, 40), (611, 100), (3, 300), (611, 300), (613, 1001), (305, 2001), (611, 3001),
+                                 (613, 5501), (613, 6501), (305, 8197), (611, 9001)])
+def test_infinite_seed_and_ragged_row_group(api, m, n, dtype, fbar):
+    # positive A and x: 2 fbar y_i A_ij and 2 fbar y_i x_j are infinities of fbar's sign, and so
+    # are their sums.  The rows missing from the last group (of 8, 4 or 2) and the teams past
+    # the end must not add infinity times zero
+    dt = torch.float64 if dtype == "f64" else torch.float32
+    rng = np.random.default_rng(m + n)
+    A, x = f32_round(rng.uniform(0.5, 1, (m, n))), f32_round(rng.uniform(0.5, 1, n))
+    ybar = 2 * fbar * (A @ x)
+    assert (ybar @ A == fbar).all() and (np.outer(ybar, x) == fbar).all()
+    p = api.QuadForm(torch.tensor(A, dtype=dt, device="cuda"), arith="native")
+    gA = torch.zeros((m, n), dtype=dt, device="cuda")
+    f, g = p.grad(torch.tensor(x, dtype=dt, device="cuda"), gdata=gA,
+                  seed=torch.tensor(fbar, dtype=dt, device="cuda"))
+    p.sync()
+    assert rel_scalar(f.item(), O.quadform_value(A, x)) <= TOL[dtype]
+    assert bool((g == fbar).all()) and bool((gA == fbar).all())
+    p.close()
