@@ -19,8 +19,9 @@
 // A dense instance of few tiles is summed into gx and f by the CTA that finishes
 // its last tile (a per-instance arrival counter); one of more than B_SUM_TILES
 // tiles by sum items of 256 columns at the end of the table, which wait for that
-// counter.  The last CTA to leave resets the queue head, so the graph can be
-// replayed as is.
+// counter.  The last CTA to leave resets the queue head and the counters, so the graph
+// can be replayed as is: no tile is running any more then, also when a sum item's
+// bounded wait gave up before its instance's last tile.
 //
 // Tile sizes R and T are chosen per (kind, size bucket) by an autotuner that
 // times candidates on the instances of the batch at kg_batch_create and keeps
@@ -72,7 +73,7 @@ struct BInst {
   void* gx;
   void* partials;  // dense: [ntiles][n] of T, or (pair) [ntiles][pitch] of Acc
   double* fpart;   // [ntiles]
-  unsigned* done;  // [0] tiles done, [1] sum items done
+  unsigned* done;  // tiles done
   int nsum;        // dense: items that sum the partials (0: the last tile's CTA does)
 };
 
@@ -87,8 +88,9 @@ struct BItem {
 struct BArgs {
   const BInst* insts;
   const BItem* items;
-  int nitems;
-  unsigned* head;  // [0] queue head, [1] CTAs that left
+  int nitems, ninst;
+  unsigned* head;  // [0] queue head, [1] CTAs that left, [2] sum items give up at once
+  unsigned* done;  // [ninst] the instances' counters
   unsigned* err;
   const float4* logtab;
   LogConsts K;
@@ -638,14 +640,17 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
       // every tile item comes before the sum items and is held by a running CTA (this
       // one has none left), so the wait ends
       if (tid == 0) {
+        const bool give_up = a.head[2] != 0u;
         const uint64_t t0 = global_ns();
+        unsigned arrived = ld_acquire_u32(I.done);
         s_last = 1;
-        while (ld_acquire_u32(I.done) < (unsigned)I.ntiles) {
-          if (global_ns() - t0 > kWaitLimitNs) {
+        while (give_up || arrived < (unsigned)I.ntiles) {
+          if (give_up || global_ns() - t0 > kWaitLimitNs) {
             set_error(a.err, ERRBIT_TIMEOUT);
             s_last = 0;
             break;
           }
+          arrived = ld_acquire_u32(I.done);
         }
         __threadfence();
       }
@@ -653,11 +658,6 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
       if (s_last) {
         if (w.start == 0 && tid < 32) sum_f<T>(I);
         sum_columns<T, PAIR>(I, (int)w.start, w.count);
-      }
-      __syncthreads();
-      if (tid == 0 && atomicAdd(I.done + 1, 1u) == (unsigned)I.nsum - 1u) {  // all have waited
-        I.done[0] = 0u;
-        I.done[1] = 0u;
       }
       it = s_item;
       continue;
@@ -693,18 +693,19 @@ __global__ void __launch_bounds__(BT, 2) batched_kernel(BArgs a) {
       __threadfence();
       if (tid < 32) sum_f<T>(I);
       if (I.kind == BK_DENSE) sum_columns<T, PAIR>(I, 0, I.n);
-      if (tid == 0) *I.done = 0u;
     }
     it = s_item;  // written by thread 0 before the barriers above
   }
   if (bad) set_error(a.err, ERRBIT_RANGE);
-  if (tid == 0) {  // the last CTA to leave resets the queue for the next replay
+  // the last CTA to leave resets the queue and the counters for the next replay
+  if (tid == 0) {
     __threadfence();
-    if (atomicAdd(&a.head[1], 1u) == gridDim.x - 1) {
-      a.head[0] = 0u;
-      a.head[1] = 0u;
-      __threadfence();
-    }
+    s_last = atomicAdd(&a.head[1], 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    for (int i = tid; i < a.ninst; i += BT) a.done[i] = 0u;
+    if (tid < 3) a.head[tid] = 0u;
   }
 }
 
@@ -938,17 +939,17 @@ kg_status devplan_alloc(DevPlan& D, Plan& P, cudaStream_t s) {
   if ((rc = al((void**)&D.items, sizeof(BItem) * P.items.size(), "work table")) != KG_OK) return rc;
   if ((rc = al((void**)&D.tet_ids, sizeof(int) * std::max<size_t>(1, P.tet_ids.size()), "tet ids")) != KG_OK) return rc;
   if ((rc = al((void**)&D.head, 16, "queue head")) != KG_OK) return rc;
-  if ((rc = al((void**)&D.done, 2 * sizeof(unsigned) * P.insts.size(), "arrival counters")) != KG_OK) return rc;
+  if ((rc = al((void**)&D.done, sizeof(unsigned) * P.insts.size(), "arrival counters")) != KG_OK) return rc;
   if ((rc = al((void**)&D.parts, std::max<size_t>(256, P.part_bytes), "partials")) != KG_OK) return rc;
   if ((rc = al((void**)&D.fpart, sizeof(double) * std::max<size_t>(1, P.fparts), "f partials")) != KG_OK) return rc;
   for (int i = 0; i < D.ninst; ++i) {
     P.insts[i].partials = D.parts + P.part_off[i];
     P.insts[i].fpart = D.fpart + P.fpart_off[i];
-    P.insts[i].done = D.done + 2 * i;
+    P.insts[i].done = D.done + i;
   }
   cudaError_t e;
   if ((e = cudaMemsetAsync(D.head, 0, 16, s)) != cudaSuccess) return cuda_fail(e, "batch set-up");
-  if ((e = cudaMemsetAsync(D.done, 0, 2 * sizeof(unsigned) * P.insts.size(), s)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(D.done, 0, sizeof(unsigned) * P.insts.size(), s)) != cudaSuccess)
     return cuda_fail(e, "batch set-up");
   if ((e = cudaMemcpyAsync(D.items, P.items.data(), sizeof(BItem) * P.items.size(),
                            cudaMemcpyHostToDevice, s)) != cudaSuccess)
@@ -1006,7 +1007,9 @@ kg_status launch_plan(const DevPlan& D, int dtype, bool pair, bool warp, unsigne
   a.insts = D.insts;
   a.items = D.items;
   a.nitems = D.nitems;
+  a.ninst = D.ninst;
   a.head = D.head;
+  a.done = D.done;
   a.err = err;
   a.K = log_consts();
   if (pair) {
@@ -1283,6 +1286,13 @@ kg_status kg_batch_create(kg_batch** out, kg_problem* const* probs, int count,
     for (int i = 0; i < count; ++i) ids[i] = i;
     b->plan = make_plan(b->probs, b->prep, ids, b->tune, b->pair, b->es, b->grid);
     rc = devplan_alloc(b->dev, b->plan, s);
+  }
+  // for tests: the sum items of the first replay give up instead of waiting
+  const char* give_up = std::getenv("KG_TEST_BATCH_GIVE_UP");
+  if (rc == KG_OK && give_up && give_up[0] == '1') {
+    const unsigned one = 1u;
+    cudaError_t e = cudaMemcpyAsync(b->dev.head + 2, &one, sizeof(one), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) rc = cuda_fail(e, "kg_batch_create");
   }
   if (rc == KG_OK) {
     cudaError_t e = cudaStreamSynchronize(s);

@@ -323,3 +323,37 @@ def test_batch_of_many_tiles_an_instance(api, dtype, tmp_path, monkeypatch):
         assert rel_l2(g.cpu().numpy(), g_ref) <= TOL[dtype], A.shape
         assert torch.equal(g, g1)
     batch.close()
+
+
+def test_batch_after_sum_items_that_gave_up(api, monkeypatch):
+    from paper_2507_13204_gb300 import _lib as L
+    # the first replay's sum items give up without waiting: reported once, and the next replays
+    # find counters on which no tile of the first one is left
+    monkeypatch.setenv("KG_NO_AUTOTUNE", "1")
+    monkeypatch.setenv("KG_TEST_BATCH_GIVE_UP", "1")
+    shapes = [(20000, 257), (6000, 1023), (4000, 2047), (1, 5)]
+    probs, host, xs = [], [], []
+    for k, (m, n) in enumerate(shapes):
+        A, x = W.quadform_inputs(n, m=m, seed=70 + k)
+        host.append((A, x))
+        probs.append(api.QuadForm(torch.tensor(A, device="cuda")))
+        xs.append(torch.tensor(x, device="cuda"))
+    fs = [torch.empty((), dtype=torch.float64, device="cuda") for _ in shapes]
+    gs = [torch.empty_like(x) for x in xs]
+    for arith in ("pair", "native"):
+        batch = api.Batch(probs, arith=arith)
+        batch.grad(xs, fs, gs)
+        with pytest.raises(L.KGError, match="gave up"):
+            batch.sync()
+        for _ in range(3):
+            for t in fs + gs:
+                t.fill_(7.0)
+            batch.grad(xs, fs, gs)
+            batch.sync()
+            for (A, x), f, g in zip(host, fs, gs):
+                f_ref, g_ref = O.quadform_grad(A, x)
+                assert rel_scalar(f.item(), f_ref) <= TOL["f64"], (arith, A.shape)
+                assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f64"], (arith, A.shape)
+        batch.close()
+    for p in probs:
+        p.close()
