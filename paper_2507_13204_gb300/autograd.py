@@ -92,8 +92,8 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
     A step is the library's value and gradient (with policy "tape": the taping forward and the
     reverse pass from the tape) and one update kernel on the current stream, called directly:
     a step through torch.autograd took about 250 us of host time, eight times the device's
-    on a mesh of 1.5e6 elements.  Inputs the direct calls do not take (other layouts,
-    subclasses, grad mode off) go through KGTetEnergy.
+    on a mesh of 1.5e6 elements.  What the direct calls do not take (other layouts,
+    subclasses, grad mode off, an `eta` that is not a plain number) goes through KGTetEnergy.
 
     With `checkpoint` and `every` > 0, {u, step} is saved every `every` steps
     (atomically: written to a temporary file, then renamed); with `resume`, a
@@ -110,7 +110,7 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
     # the shared-memory-table gradient costs more than a taping forward and the tape's scatter
     tape = mode == "tape" and (policy == "tape" or (policy == "auto" and strategy == "shared"))
     direct = (type(u) is torch.Tensor and u.dim() == 1 and u.is_contiguous() and torch.is_grad_enabled()
-              and (policy != "tape" or tape))
+              and (policy != "tape" or tape) and isinstance(eta, (int, float)) and not isinstance(eta, bool))
     f = g = None
     for t in range(start, steps):
         if direct:

@@ -189,3 +189,26 @@ def test_descent_direct_steps_match_autograd_steps(mods, strategy, mode, policy)
         ag.gradient_descent(p, u0.view(-1, 1), ETA, 1, policy=policy)
     with torch.no_grad(), pytest.raises(RuntimeError):
         ag.gradient_descent(p, u0, ETA, 1, policy=policy)
+
+
+def _descent_by_autograd(ag, p, u, eta, steps):
+    for _ in range(steps):
+        ut = u.clone().requires_grad_(True)
+        (g,) = torch.autograd.grad(ag.KGTetEnergy.apply(ut, p), ut)
+        u = u - eta * g
+    return u.detach()
+
+
+@pytest.mark.parametrize("kind", ["per vertex", "0-d", "0-d requires grad", "0-d cuda", "numpy", "bool", "int"])
+def test_descent_takes_every_kind_of_step_length(mods, kind):
+    api, ag = mods
+    mesh = W.tet_mesh(4, jitter_seed=2, perm_seed=4)
+    p = _tet(api, mesh, strategy="csr", mode="recompute")
+    u0 = torch.tensor(np.random.default_rng(5).uniform(-1, 1, mesh.nv), device="cuda")
+    eta = {"per vertex": torch.linspace(0, ETA, mesh.nv, dtype=torch.float64, device="cuda"),
+           "0-d": torch.tensor(ETA), "0-d requires grad": torch.tensor(ETA, requires_grad=True),
+           "0-d cuda": torch.tensor(ETA, dtype=torch.float64, device="cuda"), "numpy": np.float64(ETA),
+           "bool": True, "int": 0}[kind]
+    got = ag.gradient_descent(p, u0, eta, 3)
+    assert not got.requires_grad
+    assert rel_l2(got.cpu().numpy(), _descent_by_autograd(ag, p, u0, eta, 3).cpu().numpy()) <= TOL["f64"]
