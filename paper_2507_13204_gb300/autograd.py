@@ -21,6 +21,7 @@ only: the reverse pass needs nothing but y, which the fused kernel rebuilds).
 from __future__ import annotations
 
 import os
+from contextlib import nullcontext
 
 import torch
 
@@ -84,6 +85,19 @@ def quad_form(x: torch.Tensor, problem: QuadForm) -> torch.Tensor:
     return KGQuadForm.apply(x, problem)
 
 
+def _autograd_watched() -> bool:
+    """Anomaly mode or saved-tensor hooks are on: they act on an autograd graph's nodes."""
+    return (torch.is_anomaly_enabled()
+            or torch._C._autograd._top_saved_tensors_default_hooks(False) is not None)
+
+
+def _range():
+    """The profiler range of a step that does not go through KGTetEnergy."""
+    if torch._C._autograd._profiler_enabled():
+        return torch.autograd.profiler.record_function("KGTetEnergy")
+    return nullcontext()
+
+
 def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: int,
                      policy: str = "auto", checkpoint: str | None = None, every: int = 0,
                      resume: bool = False, history: list | None = None) -> torch.Tensor:
@@ -93,7 +107,10 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
     reverse pass from the tape) and one update kernel on the current stream, called directly:
     a step through torch.autograd took about 250 us of host time, eight times the device's
     on a mesh of 1.5e6 elements.  What the direct calls do not take (other layouts,
-    subclasses, grad mode off, an `eta` that is not a plain number) goes through KGTetEnergy.
+    subclasses, grad mode off, an `eta` that is not a plain number) goes through KGTetEnergy,
+    and so does every step while anomaly mode or saved-tensor hooks are on.  A profiler sees
+    a range "KGTetEnergy" a step either way.  With policy "auto" the direct steps neither
+    read nor write a problem's tape (except for strategy "shared").
 
     With `checkpoint` and `every` > 0, {u, step} is saved every `every` steps
     (atomically: written to a temporary file, then renamed); with `resume`, a
@@ -110,7 +127,8 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
     # the shared-memory-table gradient costs more than a taping forward and the tape's scatter
     tape = mode == "tape" and (policy == "tape" or (policy == "auto" and strategy == "shared"))
     direct = (type(u) is torch.Tensor and u.dim() == 1 and u.is_contiguous() and torch.is_grad_enabled()
-              and (policy != "tape" or tape) and isinstance(eta, (int, float)) and not isinstance(eta, bool))
+              and (policy != "tape" or tape) and isinstance(eta, (int, float)) and not isinstance(eta, bool)
+              and not _autograd_watched())
     f = g = None
     for t in range(start, steps):
         if direct:
@@ -118,11 +136,12 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
                 f = torch.empty((), dtype=u.dtype, device=u.device)
             if g is None:
                 g = torch.empty_like(u)
-            if tape:
-                problem.eval_tape(u, f)
-                problem.grad_from_tape(gx=g)
-            else:
-                problem.grad(u, gx=g, f=f)
+            with _range():
+                if tape:
+                    problem.eval_tape(u, f)
+                    problem.grad_from_tape(gx=g)
+                else:
+                    problem.grad(u, gx=g, f=f)
             u.sub_(g, alpha=eta)
         else:
             ut = u.requires_grad_(True)

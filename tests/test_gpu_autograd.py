@@ -212,3 +212,24 @@ def test_descent_takes_every_kind_of_step_length(mods, kind):
     got = ag.gradient_descent(p, u0, eta, 3)
     assert not got.requires_grad
     assert rel_l2(got.cpu().numpy(), _descent_by_autograd(ag, p, u0, eta, 3).cpu().numpy()) <= TOL["f64"]
+
+
+def test_descent_is_seen_by_hooks_anomaly_mode_and_the_profiler(mods):
+    api, ag = mods
+    mesh = W.tet_mesh(4, jitter_seed=2, perm_seed=4)
+    p = _tet(api, mesh, strategy="csr", mode="recompute")
+    u0 = torch.tensor(np.random.default_rng(5).uniform(-1, 1, mesh.nv), device="cuda")
+    ref = ag.gradient_descent(p, u0, ETA, 3)
+    packed = []
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: packed.append(t.shape) or t.cpu(), lambda t: t.cuda()):
+        got = ag.gradient_descent(p, u0, ETA, 3)
+    assert packed == [u0.shape] * 3 and rel_l2(got.cpu().numpy(), ref.cpu().numpy()) <= TOL["f64"]
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU]) as prof:
+        ag.gradient_descent(p, u0, ETA, 3)
+    assert sum(e.count for e in prof.key_averages() if e.key == "KGTetEnergy") == 3
+    p32 = api.TetEnergy(torch.tensor(mesh.conn, device="cuda"),
+                        torch.tensor(mesh.G, dtype=torch.float32, device="cuda"), mesh.nv)
+    bad = u0.float()
+    bad[0] = np.inf  # a NaN gradient
+    with torch.autograd.detect_anomaly(), pytest.raises(RuntimeError):
+        ag.gradient_descent(p32, bad, ETA, 1)
