@@ -1257,11 +1257,11 @@ kg_status kg_batch_create(kg_batch** out, kg_problem* const* probs, int count,
     });
     for (int i : order) {
       kg_problem* p = b->probs[i];
-      const size_t bytes = 8 * (size_t)p->m * (size_t)p->n;
+      // rows of odd n are padded by a zero to whole column pairs
+      const size_t bytes = 8 * (size_t)p->m * (size_t)(p->n + (p->n & 1));
       if (bytes > budget) continue;
       void* q = nullptr;
-      // rows of odd n are padded by a zero to whole column pairs
-      if (dev_alloc(&q, 8 * (size_t)p->m * (size_t)(p->n + (p->n & 1))) != cudaSuccess) {
+      if (dev_alloc(&q, bytes) != cudaSuccess) {
         rc = fail(KG_ERR_OOM, "kg_batch_create: float-pair copy of A");
         break;
       }

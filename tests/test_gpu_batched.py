@@ -357,3 +357,28 @@ def test_batch_after_sum_items_that_gave_up(api, monkeypatch):
         batch.close()
     for p in probs:
         p.close()
+
+
+def test_copies_of_odd_rows_stay_within_the_budget(api, monkeypatch):
+    # rows of odd length are copied with a zero behind them; that belongs to the budget
+    monkeypatch.setenv("KG_NO_AUTOTUNE", "1")
+    m, n = 1 << 23, 1  # 64 MiB of doubles, 128 MiB as padded rows
+    A = torch.rand((m, n), dtype=torch.float64, device="cuda") + 0.5
+    p = api.QuadForm(A)
+    x = torch.ones(n, dtype=torch.float64, device="cuda")
+    ref = (A * A).sum().item()
+    taken = []
+    for budget in (8 * m * n, 8 * m * (n + 1)):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        batch = api.Batch([p], budget_bytes=budget)
+        taken.append(before - torch.cuda.mem_get_info()[0])
+        assert batch.config[0] == "pair"
+        f, g = torch.empty((), dtype=torch.float64, device="cuda"), torch.empty_like(x)
+        batch.grad([x], [f], [g])
+        batch.sync()
+        assert rel_scalar(f.item(), ref) <= TOL["f64"] and rel_scalar(g.item(), 2 * ref) <= TOL["f64"]
+        batch.close()
+    # the copy and a few MiB of work table and partials, or only those
+    assert taken[0] < 32 << 20 and 128 << 20 <= taken[1] < 160 << 20
+    p.close()
