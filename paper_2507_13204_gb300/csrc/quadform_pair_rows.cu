@@ -241,6 +241,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) qf_pair_rows_kernel(PrArgs a) 
       const Pair y2 = pair_mul(y, y);
       facc = acc_add(facc, Acc{y2.h, y2.l});
     }
+    ++done;
     if constexpr (FUSED) {
       const Pair ybl = pair_mul(fb2, y);
 #pragma unroll
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) qf_pair_rows_kernel(PrArgs a) 
 #pragma unroll
         for (int k = 0; k < KP; ++k) acc2_fma(xb[k], av[r][k], yb);
       }
-      if ((++done & 3) == 0) {
+      if ((done & 3) == 0) {
 #pragma unroll
         for (int k = 0; k < KP; ++k) acc2_renorm(xb[k]);
       }

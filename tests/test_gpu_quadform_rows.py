@@ -167,3 +167,24 @@ def test_infinite_seed_and_ragged_row_group(api, m, n, dtype, fbar):
     assert rel_scalar(f.item(), O.quadform_value(A, x)) <= TOL[dtype]
     assert bool((g == fbar).all()) and bool((gA == fbar).all())
     p.close()
+
+
+@pytest.mark.parametrize("m,n", [(401280, 1024)])
+def test_pair_value_of_a_tall_matrix_of_equal_rows(api, m, n):
+    # y_i^2 the same for every row: a thread that adds 330 of them (two CTAs an SM, four rows a
+    # step) keeps their bits only with its accumulator renormalised; in float arithmetic, 1.0e-11
+    # without and 2.7e-13 with it
+    a = 1.972628813822955
+    A = torch.zeros((m, n), dtype=torch.float64, device="cuda")
+    A[:, 0] = a
+    x = torch.zeros(n, dtype=torch.float64, device="cuda")
+    x[0] = 1.0
+    p = api.QuadForm(A, tape_budget_bytes=8 << 30)
+    assert p.config[2] == "pair"
+    f, g = p.grad(x)
+    fe = p.eval(x)
+    p.sync()
+    assert rel_scalar(fe.item(), m * a * a) <= TOL["f64"]
+    assert rel_scalar(f.item(), m * a * a) <= TOL["f64"]
+    assert rel_scalar(g[0].item(), 2 * m * a * a) <= TOL["f64"]
+    p.close()
