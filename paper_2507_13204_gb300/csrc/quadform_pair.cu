@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(QP_THREADS, 1) qf_pair_kernel(QpArgs a) {
     if (t == 0) {  // f in pair arithmetic: no FP64 instruction in the row loop
       const Pair y2 = pair_mul(y, y);
       facc = acc_add(facc, Acc{y2.h, y2.l});
+      if ((it & 7) == 7) acc_renorm(facc);
     }
     if (FUSED) {
       const Pair2 yb = pair2_dup(pair_mul(fb2, y));
@@ -462,6 +463,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) qf_pair_ws_kernel(QpArgs a) {
       if (t == 0) {
         const Pair y2 = pair_mul(y, y);
         facc = acc_add(facc, Acc{y2.h, y2.l});
+        if ((r & 7) == 7) acc_renorm(facc);
       }
       const Pair2 yb = pair2_dup(pair_mul(fb2, y));
 #pragma unroll

@@ -169,10 +169,10 @@ def test_infinite_seed_and_ragged_row_group(api, m, n, dtype, fbar):
     p.close()
 
 
-@pytest.mark.parametrize("m,n", [(401280, 1024)])
+@pytest.mark.parametrize("m,n", [(401280, 1024), (50160, 6000), (50160, 10242)])
 def test_pair_value_of_a_tall_matrix_of_equal_rows(api, m, n):
-    # y_i^2 the same for every row: a thread that adds 330 of them (two CTAs an SM, four rows a
-    # step) keeps their bits only with its accumulator renormalised; in float arithmetic, 1.0e-11
+    # y_i^2 the same for every row: a thread that adds 330 of them (two CTAs an SM and four rows a
+    # step, or a CTA an SM and a row a step) keeps their bits only with its accumulator renormalised; in float arithmetic, 1.0e-11
     # without and 2.7e-13 with it
     a = 1.972628813822955
     A = torch.zeros((m, n), dtype=torch.float64, device="cuda")
