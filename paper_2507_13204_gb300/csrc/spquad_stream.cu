@@ -177,7 +177,11 @@ __global__ void __launch_bounds__(SS_THREADS, ss_ctas(MODE)) spq_stream_kernel(S
         v[k] = e < cnt ? __ldcs(a.val + p0 + e) : val{};
       }
 #pragma unroll
-      for (int k = 0; k < SS_K; ++k) xv[k] = ss_x<AR>(__ldg(a.x + c[k]), bad);
+      for (int k = 0; k < SS_K; ++k) {
+        bool out = false;  // of range: an entry's x counts, the padding's does not
+        xv[k] = ss_x<AR>(__ldg(a.x + c[k]), out);
+        bad |= out && tid + k * SS_THREADS < cnt;
+      }
 #pragma unroll
       for (int k = 0; k < SS_K; ++k) {
         const int e = tid + k * SS_THREADS;

@@ -239,3 +239,29 @@ def test_row_blocks(api, name, kind, strategy):
         g4, g5 = p.grad(xt, seed=seed)[1].clone(), p.grad(xt, seed=seed)[1]
         assert torch.equal(g4, g5) and rel_l2(g4.cpu().numpy(), g_ref) <= tol
     p.close()
+
+
+@pytest.mark.parametrize("strategy", ["atomic", "transpose"])
+@pytest.mark.parametrize("name", ["no entries", "tw1", "tw4", "tw16"])
+def test_an_x_that_no_entry_reads_has_no_range(api, name, strategy):
+    from paper_2507_13204_gb300 import _lib as L
+    # column 0 has no entries; the blocks' lanes without an entry must not look at x[0] either
+    A = _csr_of_degrees([0] * 40 if name == "no entries" else BLOCKS[name], 211, seed=len(name))
+    A.col[A.col == 0] = 1
+    x = np.random.default_rng(6).uniform(0.5, 1, A.n)
+    f_ref, g_ref, gv_ref = O.spquadform_grad(A.rowptr, A.col, A.val, x, want_gval=True)
+    p = _problem(api, A, strategy=strategy, arith="pair")
+    for x0 in (1e-30, np.inf):
+        x[0] = x0
+        gv = torch.zeros(A.nnz, dtype=torch.float64, device="cuda")
+        f, g = p.grad(torch.tensor(x, device="cuda"), gdata=gv if A.nnz else None)
+        fe = p.eval(torch.tensor(x, device="cuda"))
+        p.sync()
+        assert rel_scalar(f.item(), f_ref) <= TOL["f64"] and rel_scalar(fe.item(), f_ref) <= TOL["f64"]
+        assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f64"] and rel_l2(gv.cpu().numpy(), gv_ref) <= TOL["f64"]
+    if name != "no entries":  # one that an entry reads is refused
+        x[0], x[1] = 1.0, 1e-30
+        p.grad(torch.tensor(x, device="cuda"))
+        with pytest.raises(L.KGError):
+            p.sync()
+    p.close()
