@@ -103,9 +103,12 @@ typedef enum { KG_F64 = 0, KG_F32 = 1 } kg_dtype;
  *             (FP32, and FP64 in PAIR arithmetic with the prepared A for
  *             2048 < n <= 10240) and those that take several shorter rows a step
  *             in PAIR arithmetic sum them in their own tail after a bounded
- *             grid barrier, as one cooperative launch; the others (and these
- *             when the grid cannot be resident at once) in the last CTA or in
- *             a second small kernel, with the same bits.
+ *             grid barrier, as one cooperative launch, or, when the grid cannot
+ *             be resident at once, in a second small kernel with the same bits.
+ *             The NATIVE kernels sum them in the last CTA (n <= 128, few CTAs)
+ *             or in a second small kernel, each in an order of its own:
+ *             kg_quadform_grad_noalloc, which always takes the second kernel,
+ *             and kg_grad can differ in the last bits.
  *   SHARED    (tet) the forward schedule with the scatter-adds of each tile of
  *             elements first combined per vertex in a shared-memory table, then
  *             one global atomic per distinct vertex (Sec. 5: shared memory for

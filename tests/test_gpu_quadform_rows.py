@@ -188,3 +188,42 @@ def test_pair_value_of_a_tall_matrix_of_equal_rows(api, m, n):
     assert rel_scalar(f.item(), m * a * a) <= TOL["f64"]
     assert rel_scalar(g[0].item(), 2 * m * a * a) <= TOL["f64"]
     p.close()
+
+
+# more rows than two an SM (the FP64 one-row kernels take fewer), not a whole number of groups,
+# in the widths whose other shapes above are short: 13 to 14 and 21 to 28 columns a lane
+@pytest.mark.parametrize("m,n", [(611, 3073), (613, 3584), (611, 5500), (613, 6500), (609, 7167)])
+def test_wide_rows_in_ragged_groups(api, m, n):
+    for dtype in ("f64", "f32"):
+        dt = torch.float64 if dtype == "f64" else torch.float32
+        rnd = f32_round if dtype == "f32" else (lambda a: a)
+        A, x = (rnd(a) for a in W.quadform_inputs(n, m=m, seed=m + n))
+        f_ref, g_ref, gA_ref = O.quadform_grad(A, x, fbar=-0.75, want_gA=True)
+        # FP32 problems of n % 4 == 0 otherwise offer no gradient w.r.t. A
+        p = api.QuadForm(torch.tensor(A, dtype=dt, device="cuda"), arith="native", team=512)
+        xt = torch.tensor(x, dtype=dt, device="cuda")
+        gA = torch.empty((m, n), dtype=dt, device="cuda")
+        f, g = p.grad(xt, gdata=gA, seed=torch.tensor(-0.75, dtype=dt, device="cuda"))
+        fe = p.eval(xt)
+        p.sync()
+        assert rel_scalar(f.item(), f_ref) <= TOL[dtype]
+        assert rel_scalar(fe.item(), O.quadform_value(A, x)) <= TOL[dtype]
+        assert rel_l2(g.cpu().numpy(), g_ref) <= TOL[dtype]
+        assert rel_l2(gA.cpu().numpy(), gA_ref) <= TOL[dtype]
+        p.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("m,n", [(611, 300), (613, 1001), (613, 2001), (611, 3001), (613, 5501)])
+def test_infinite_x_and_ragged_row_group_of_several_warps(api, m, n, dtype):
+    dt = torch.float64 if dtype == "f64" else torch.float32
+    x = torch.ones(n, dtype=dt, device="cuda")
+    x[n - 1] = np.inf
+    p = api.QuadForm(torch.ones((m, n), dtype=dt, device="cuda"), arith="native")
+    f, g = p.grad(x)
+    fe = p.eval(x)
+    p.sync()
+    assert bool((g == np.inf).all())
+    if dtype == "f64":  # (FP32: the compensated sum of squares has no infinity)
+        assert f.item() == np.inf and fe.item() == np.inf
+    p.close()
