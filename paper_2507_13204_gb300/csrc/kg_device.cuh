@@ -55,6 +55,36 @@ __device__ __forceinline__ void finish_sum(double partial, double* fpart, unsign
   }
 }
 
+// The same by the first warp alone (partial in thread 0): for grids of up to a few
+// hundred CTAs, whose partials are a handful of loads a lane.  A sum over the CTA is ten
+// FP64 adds in every warp, 0.7 us of the FP64 unit in CTAs of 8 warps.
+template <typename T>
+__device__ __forceinline__ void finish_sum_warp(double partial, double* fpart, unsigned* counter, T* out) {
+  if (threadIdx.x >= 32) return;
+  unsigned arrived = 0u;
+  if (threadIdx.x == 0) {
+    fpart[blockIdx.x] = partial;
+    __threadfence();
+    arrived = atomicAdd(counter, 1u);
+  }
+  arrived = __shfl_sync(0xffffffffu, arrived, 0);
+  if (arrived != gridDim.x - 1) return;
+  __threadfence();
+  double s = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i + 32 * u < (int)gridDim.x ? __ldcg(&fpart[i + 32 * u]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  s = warp_sum(s);
+  if (threadIdx.x == 0) {
+    if (out) *out = (T)s;
+    *counter = 0u;
+  }
+}
+
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");

@@ -14,11 +14,14 @@
 //   - only teams wider than a warp (n > 256) exchange through shared memory, once per
 //     R rows.
 // CPL is fixed at compile time, ceil(n / (32 W)) up to n = 4096 and even above, so that
-// at most the last two column slots are tested or idle.  Groups of R rows go round-robin over all teams of the grid; xbar is
-// accumulated in registers, combined over the CTA's teams in team order and, for grids
-// of one CTA, written as the gradient; larger grids write a row of partials per CTA,
-// summed in a fixed order by the CTA that finishes last (few partials) or by
-// qf_reduce_kernel: bitwise reproducible.
+// at most the last two column slots are tested or idle.  Groups of R rows go round-robin over
+// all teams of the grid, each team by itself: with a barrier of the whole CTA the teams without
+// a group kept the FP64 unit busy with zeros (300 x 1024 value 8.3 -> 5.5 us, 610 x 1000 value
+// and gradient 18.8 -> 12.7, 3000 x 1000 29.4 -> 23.4, together with f summed by the warps that
+// hold it instead of the whole CTA).  xbar is accumulated in registers, combined over the CTA's
+// teams in team order and, for grids of one CTA, written as the gradient; larger grids write a
+// row of partials per CTA, summed in a fixed order by the CTA that finishes last (few partials)
+// or by qf_reduce_kernel: bitwise reproducible.
 //
 // Measured (value and gradient, one call, against one row a team and step with a butterfly
 // per row): FP64 150001 x 255 857 -> 160 us (its DFMAs take 122), 20000 x 2051 963 -> 250
@@ -117,16 +120,15 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
   FSum<T> fsum;  // of row lane / G of every group (counted once per row below)
 
   // group g of R rows goes to team g / gridDim.x of CTA g % gridDim.x, round by round
-  const int64_t groups = (a.m + R - 1) / R;
-  const int64_t nteams = (int64_t)gridDim.x * NT;
+  const unsigned groups = (unsigned)((a.m + R - 1) / R);  // m < 2^31
+  const int64_t first = blockIdx.x + (int64_t)team * gridDim.x, all = (int64_t)gridDim.x * NT;
+  const unsigned step = all < groups ? (unsigned)all : groups;
   int par = 0;
-  // the trip count is that of the CTA's first team: teams of W > 1 meet at a CTA barrier
-  for (int64_t g0 = blockIdx.x; g0 < groups; g0 += nteams, par ^= 1) {
-    const int64_t grp = g0 + (int64_t)team * gridDim.x;
-    const int64_t r0 = grp * R;
-    if (W == 1 && grp >= groups) break;
-    const int rows = grp < groups ? (int)(a.m - r0 < R ? a.m - r0 : R) : 0;
-    const T* Ar = a.A + (rows > 0 ? r0 : 0) * (int64_t)n + lt;
+  // each team by itself: one without a group in the last round leaves the FP64 unit to the others
+  for (unsigned grp = first < groups ? (unsigned)first : groups; grp < groups; grp += step, par ^= 1) {
+    const int64_t r0 = (int64_t)grp * R;
+    const int rows = (int)(a.m - r0 < R ? a.m - r0 : R);
+    const T* Ar = a.A + r0 * (int64_t)n + lt;
     T av[R][CPL];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -147,7 +149,8 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
     if constexpr (W > 1) {
       T* rd = red + par * WARPS * R + team * W * R;
       if (lane % G == 0) rd[(warp % W) * R + row] = tot;
-      __syncthreads();
+      if constexpr (NT == 1) __syncthreads();
+      else named_barrier(1 + team, TEAM);
       tot = rd[(lane % WG) * R + row];
 #pragma unroll
       for (int i = G; i < W; i += G) tot += rd[(i + lane % G) * R + row];
@@ -180,11 +183,23 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
     }
   }
 
-  // the CTA's f: one lane per row of a group, one warp per team
-  const double fcta =
-      block_sum(lane % G == 0 && (W == 1 || warp % W == 0) ? fsum.get() : 0.0, fred);
+  // the CTA's f, in thread 0: one lane per row of a group, one warp per team (a sum over the
+  // whole CTA would occupy the FP64 unit for 1.3 us in CTAs of 16 warps)
+  double fcta = 0.0;
+  if (W == 1 || warp % W == 0) {
+    double fs = fsum.get();
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
+    if (lane == 0) fred[team] = fs;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    fcta = fred[0];
+#pragma unroll
+    for (int t = 1; t < NT; ++t) fcta += fred[t];
+  }
   if constexpr (!FUSED) {
-    finish_sum<T>(fcta, a.fpart, a.counter, a.f, 0, fred);
+    finish_sum_warp<T>(fcta, a.fpart, a.counter, a.f);
     return;
   } else {
     const bool one = gridDim.x == 1;
@@ -238,12 +253,20 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
       for (int q = 1; q < pgs; ++q) s += xbs[q * cw + j];
       a.gx[j] = a.accumulate ? a.gx[j] + s : s;
     }
-    double fs = 0.0;
-    for (int i = threadIdx.x; i < parts; i += THREADS) fs += __ldcg(a.fpart + i);
-    fs = block_sum(fs, fred);
-    if (threadIdx.x == 0) {
-      if (a.f) *a.f = (T)fs;
-      *a.counter = 0u;
+    if (warp == 0) {
+      double fs = 0.0;
+      for (int i = lane; i < parts; i += 8 * 32) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = i + 32 * u < parts ? __ldcg(a.fpart + i + 32 * u) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) fs += v[u];
+      }
+      fs = warp_sum(fs);
+      if (lane == 0) {
+        if (a.f) *a.f = (T)fs;
+        *a.counter = 0u;
+      }
     }
   }
 }
