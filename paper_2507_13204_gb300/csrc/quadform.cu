@@ -90,8 +90,10 @@ __global__ void __launch_bounds__(256) qf_transpose_kernel(const T* __restrict__
 // a butterfly, then the 16 warps' sums are added in warp order.  Block 0 also sums the
 // per-CTA f partials into *f.  Narrow blocks spread the loads of a short row of partials
 // over the chip: 304 partials of 255 doubles took 7.0 us in 8 blocks of 32 columns.  Up to
-// 64 partials take 32 columns a block (CX): 64 bytes would leave half the threads idle in
-// four times the blocks (30 partials of 9001 doubles: 3 us more).
+// 64 partials, and rows of which 32 columns a block fill the chip, take these (CX): 64 bytes
+// would leave threads idle in four times the blocks, each with the same FP64 adds to finish
+// (30 partials of 9001 doubles: 3 us more; value and gradient of 150 x 12288 23.2 -> 19.4 us,
+// of 500 x 12288 46.5 -> 42.9).
 template <typename T, int CX>
 __global__ void __launch_bounds__(512) qf_reduce_kernel(const T* __restrict__ partials, int nparts,
                                                         int n, const double* __restrict__ fpart,
@@ -300,8 +302,8 @@ static QfRowsCall<T> rows_call(kg_problem* p, const void* x, void* f) {
 template <typename T>
 kg_status qf_reduce_partials(const T* partials, int nparts, int n, const double* fpart, int nf, T* gx,
                              T* f, int accumulate, cudaStream_t s) {
-  const bool few = nparts <= 64;
-  const int cx = few ? 32 : 64 / (int)sizeof(T);
+  const bool wide = nparts <= 64 || n >= 32 * num_sms();
+  const int cx = wide ? 32 : 64 / (int)sizeof(T);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((n + cx - 1) / cx);
   cfg.blockDim = dim3(512);
@@ -311,7 +313,7 @@ kg_status qf_reduce_partials(const T* partials, int nparts, int n, const double*
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  auto kern = few ? qf_reduce_kernel<T, 32> : qf_reduce_kernel<T, 64 / (int)sizeof(T)>;
+  auto kern = wide ? qf_reduce_kernel<T, 32> : qf_reduce_kernel<T, 64 / (int)sizeof(T)>;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, partials, nparts, n, fpart, nf, gx, f, accumulate);
   count_launch();
   return e == cudaSuccess ? KG_OK : cuda_fail(e, "qf reduce kernel");
