@@ -279,6 +279,10 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
 //   16 warps:       n <= 4096 4 rows a step, then x in shared memory and 2 rows (FP32 4) to
 //                   8192 entries, 1 (FP32 2) to 12288, where the forward, which keeps no row
 //                   for a reverse, still takes 2 (FP32 4).
+//   FP64 teams of several warps on at most two rows an SM take one row a step: several rows on
+//   one team leave the other SMs idle while its FP64 unit works through them, and the rows
+//   missing from a step cost the unit as much as rows (100 x 2001 value and gradient 11.7 us,
+//   9.0 with a row a step; the value of 80 x 12288 12.1 and 8.9).
 template <typename T, int W, typename Go>
 static void qr_small(int64_t n, const Go& go) {
   switch ((n + 32 * W - 1) / (32 * W)) {
@@ -289,17 +293,14 @@ static void qr_small(int64_t n, const Go& go) {
   }
 }
 
-//
-// FP64 teams of several warps on at most two rows an SM take one row a step: four rows on
-// one team leave the other SMs idle while its FP64 unit works through them (100 x 2001
-// 11.7 us, 9.0 with a row a step).
 template <typename T, bool FUSED, typename Go>
 static void qr_with_shape(int64_t m, int64_t n, int team, const Go& go) {
-  constexpr int R2 = sizeof(T) == 8 ? 2 : 4, R1 = FUSED ? R2 / 2 : R2;
+  constexpr int R2 = sizeof(T) == 8 ? 2 : 4, R1 = FUSED ? R2 / 2 : R2, R0 = sizeof(T) == 8 ? 1 : R1;
   int w = team / 32;
   if (!team)
     for (w = 1; (int64_t)256 * w < n && w < 16;) w *= 2;
-  if (sizeof(T) == 8 && w >= 2 && m <= 2 * (int64_t)num_sms() && n <= 8192) {
+  const bool few = sizeof(T) == 8 && w >= 2 && m <= 2 * (int64_t)num_sms();
+  if (few && n <= 8192) {
     switch (w) {
       case 2: return go(QrShape<2, 8, 0, 1, false>{});
       case 4: return go(QrShape<4, 8, 0, 1, false>{});
@@ -323,6 +324,12 @@ static void qr_with_shape(int64_t m, int64_t n, int team, const Go& go) {
   if (c <= 12) return go(QrShape<16, 12, 10, R2, true>{});
   if (c <= 14) return go(QrShape<16, 14, 12, R2, true>{});
   if (c <= 16) return go(QrShape<16, 16, 14, R2, true>{});
+  if (few) {
+    if (c <= 18) return go(QrShape<16, 18, 16, R0, true>{});
+    if (c <= 20) return go(QrShape<16, 20, 18, R0, true>{});
+    if (c <= 22) return go(QrShape<16, 22, 20, R0, true>{});
+    return go(QrShape<16, 24, 22, R0, true>{});
+  }
   if (c <= 18) return go(QrShape<16, 18, 16, R1, true>{});
   if (c <= 20) return go(QrShape<16, 20, 18, R1, true>{});
   if (c <= 22) return go(QrShape<16, 22, 20, R1, true>{});
