@@ -46,7 +46,8 @@ struct QfConfig {
   int cpt = 1;      // columns per team thread (compile-time variant)
   int grid = 1;     // CTAs
   int rows_per_cta = 1;
-  int rgrid = 0;     // CTAs of the native forward and fused kernels (quadform_rows.cu)
+  int rgrid = 0;     // CTAs of the native fused kernels (quadform_rows.cu)
+  int egrid = 0;     // ... and of the native forward
   int streamed = 0;  // 1: FP32 TMA-streamed kernel (quadform_f32.cu)
   int coop = 0;      // 1: the streamed gradient (pair, FP32) reduces its partials in one cooperative launch
 };
@@ -131,7 +132,7 @@ struct QfRowsCall {
   T* gA;
   int accumulate;
 };
-int qf_rows_grid(int dtype, int64_t m, int64_t n, int team);
+int qf_rows_grid(int dtype, int64_t m, int64_t n, int team, bool eval);
 template <typename T>
 kg_status qf_rows_eval(const QfRowsCall<T>& c, cudaStream_t s);
 template <typename T>

@@ -227,7 +227,8 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
     c.team = c.block = 512;
     // short rows: several at a step instead (40000 x 1024 96.8 -> 32 us, 40000 x 2048 97.6 -> 56);
     // with fewer rows than CTAs of the streamed kernel, one a CTA is as good
-    if (p->n <= 2048 && p->m >= 2 * (int64_t)num_sms()) c.rgrid = qf_rows_grid(KG_F32, p->m, p->n, 0);
+    if (p->n <= 2048 && p->m >= 2 * (int64_t)num_sms())
+      c.rgrid = c.egrid = qf_rows_grid(KG_F32, p->m, p->n, 0, false);  // more than one CTA
     const int most = std::max(c.grid, c.rgrid);
     kg_status rc = ws_common(p, most, s);
     if (rc == KG_OK) rc = ws_alloc(p, &p->partials, 4 * (size_t)most * p->n, "xbar partials (FP32)");
@@ -253,8 +254,9 @@ kg_status qf_setup(kg_problem* p, cudaStream_t s) {
   if (p->opt.tile > 0) rows = p->opt.tile;
   c.rows_per_cta = (int)rows;
   c.grid = (int)((p->m + rows - 1) / rows);
-  c.rgrid = p->opt.tile > 0 ? c.grid : qf_rows_grid(p->dtype, p->m, p->n, p->opt.team);
-  int fp = std::max({c.grid, c.rgrid, transpose_chunks(p)});
+  c.rgrid = p->opt.tile > 0 ? c.grid : qf_rows_grid(p->dtype, p->m, p->n, p->opt.team, false);
+  c.egrid = p->opt.tile > 0 ? c.grid : qf_rows_grid(p->dtype, p->m, p->n, p->opt.team, true);
+  int fp = std::max({c.grid, c.rgrid, c.egrid, transpose_chunks(p)});
   kg_status rc = ws_common(p, fp, s);
   if (rc != KG_OK) return rc;
   if (p->strategy == KG_STRATEGY_FUSED || p->strategy == KG_STRATEGY_TRANSPOSE) {
@@ -327,6 +329,7 @@ template <typename T>
 static kg_status qf_eval_t(kg_problem* p, const void* x, void* f, T* y, cudaStream_t s) {
   QfRowsCall<T> r = rows_call<T>(p, x, f);
   r.y = y;
+  r.grid = p->qf.egrid;
   return qf_rows_eval(r, s);
 }
 
@@ -407,7 +410,7 @@ kg_status qf_native_fused_on_scratch(const double* A, int64_t m, int64_t n, cons
   r.x = x;
   r.m = m;
   r.n = n;
-  r.grid = (int)std::min<int64_t>(qf_rows_grid(KG_F64, m, n, 0), max_grid);
+  r.grid = (int)std::min<int64_t>(qf_rows_grid(KG_F64, m, n, 0, false), max_grid);
   r.partials = scratch;
   r.fpart = scratch + (size_t)r.grid * n;
   r.f = f;

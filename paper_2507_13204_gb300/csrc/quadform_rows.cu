@@ -340,14 +340,21 @@ template <typename T, typename S>
 constexpr size_t qr_smem() { return S::XS ? sizeof(T) * S::CPL * S::THREADS : 0; }
 
 // One wave of resident CTAs, or fewer when a quarter of an SM's warps (one a scheduler,
-// which its FP64 unit needs no more than) or a whole CTA has a group of rows; a matrix of up
-// to 4096 entries is one CTA's, which writes the gradient itself.
+// which its FP64 unit needs no more than) or a whole CTA has a group of rows.
+//   - The gradient of up to 4096 entries is one CTA's, which writes it itself, when its teams
+//     need at most 2 rounds (FP64) or 5: 64 x 64 5.6 us and 7.1 with several CTAs, 128 x 8 6.6
+//     and 6.4, 256 x 8 10.6 and 6.5; FP32 300 x 8 5.0 and 5.5, 512 x 8 6.9 and 5.3.
+//   - The forward has no partials to sum: several CTAs are as fast at 8 rows and faster above
+//     (FP32 300 x 8 5.0 and 3.9).  In FP64 it spreads its groups over the SMs, one FP64 unit
+//     each: 150 x 16 7.6 -> 4.6, 4 x 700 5.9 -> 4.3.
 template <typename T>
-static int qr_grid_t(int64_t m, int64_t n, int team) {
+static int qr_grid_t(int64_t m, int64_t n, int team, bool eval) {
   int64_t grid = 1;
-  if (m * n <= 4096) return 1;
+  const bool spread = eval && sizeof(T) == 8;
   qr_with_shape<T, true>(m, n, team, [&](auto shape) {
     using S = decltype(shape);
+    constexpr int one = S::R * S::NT * (sizeof(T) == 8 ? 2 : 5);  // rows of one CTA
+    if (!eval && m * n <= 4096 && m <= one) return;
     int occ = 0;
     auto kern = qf_rows_kernel<T, S, true>;
     if (set_smem_once(kern, qr_smem<T, S>()) != cudaSuccess ||
@@ -358,12 +365,13 @@ static int qr_grid_t(int64_t m, int64_t n, int team) {
     }
     const int64_t step = (int64_t)S::R * std::max(1, 4 / S::W);
     grid = std::min<int64_t>((m + step - 1) / step, (int64_t)num_sms() * occ);
+    if (spread) grid = std::max(grid, std::min<int64_t>((m + S::R - 1) / S::R, num_sms()));
   });
   return (int)std::max<int64_t>(1, grid);
 }
 
-int qf_rows_grid(int dtype, int64_t m, int64_t n, int team) {
-  return dtype == KG_F64 ? qr_grid_t<double>(m, n, team) : qr_grid_t<float>(m, n, team);
+int qf_rows_grid(int dtype, int64_t m, int64_t n, int team, bool eval) {
+  return dtype == KG_F64 ? qr_grid_t<double>(m, n, team, eval) : qr_grid_t<float>(m, n, team, eval);
 }
 
 template <typename T, bool FUSED>

@@ -227,3 +227,26 @@ def test_infinite_x_and_ragged_row_group_of_several_warps(api, m, n, dtype):
     if dtype == "f64":  # (FP32: the compensated sum of squares has no infinity)
         assert f.item() == np.inf and fe.item() == np.inf
     p.close()
+
+
+# few columns: one CTA's rounds end at 128 rows (FP64) and 320 (FP32) of up to 4096 entries in
+# all; the forward has a grid of its own
+@pytest.mark.parametrize("m,n", [(64, 1), (128, 8), (129, 8), (320, 8), (321, 12), (1000, 3), (4096, 1), (4097, 1),
+                                 (150, 16), (8, 512), (4, 700)])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_few_columns(api, m, n, dtype):
+    dt = torch.float64 if dtype == "f64" else torch.float32
+    A, x = W.quadform_inputs(n, m=m, seed=7 * m + n)
+    if dtype == "f32":
+        A, x = f32_round(A), f32_round(x)
+    f_ref, g_ref = O.quadform_grad(A, x)
+    p = api.QuadForm(torch.tensor(A, dtype=dt, device="cuda"), arith="native")
+    xt = torch.tensor(x, dtype=dt, device="cuda")
+    f, g = p.grad(xt)
+    fe = p.eval(xt)
+    f2, g2 = p.grad(xt)
+    p.sync()
+    assert rel_scalar(f.item(), f_ref) <= TOL[dtype] and rel_scalar(fe.item(), f_ref) <= TOL[dtype]
+    assert rel_l2(g.cpu().numpy(), g_ref) <= TOL[dtype]
+    assert torch.equal(f, f2) and torch.equal(g, g2)
+    p.close()
