@@ -279,10 +279,12 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
 //   16 warps:       n <= 4096 4 rows a step, then x in shared memory and 2 rows (FP32 4) to
 //                   8192 entries, 1 (FP32 2) to 12288, where the forward, which keeps no row
 //                   for a reverse, still takes 2 (FP32 4).
-//   FP64 teams of several warps on at most two rows an SM take one row a step: several rows on
-//   one team leave the other SMs idle while its FP64 unit works through them, and the rows
-//   missing from a step cost the unit as much as rows (100 x 2001 value and gradient 11.7 us,
-//   9.0 with a row a step; the value of 80 x 12288 12.1 and 8.9).
+//   FP64 rows of more than 128 entries, at most two an SM, are taken one a step by teams of two
+//   warps or more: several rows on one team leave the other SMs idle while its FP64 unit works
+//   through them, and the rows missing from a step cost the unit as much as rows (value and
+//   gradient of 100 x 2001 11.7 us, 9.0 with a row a step; of 150 x 256 9.6 and 7.1; the value
+//   of 80 x 12288 12.1 and 8.9).  Rows of up to 256 entries on one CTA stay with its eight
+//   one-warp teams (31 x 129 5.9 us, 6.7 one a step).
 template <typename T, int W, typename Go>
 static void qr_small(int64_t n, const Go& go) {
   switch ((n + 32 * W - 1) / (32 * W)) {
@@ -299,9 +301,10 @@ static void qr_with_shape(int64_t m, int64_t n, int team, const Go& go) {
   int w = team / 32;
   if (!team)
     for (w = 1; (int64_t)256 * w < n && w < 16;) w *= 2;
-  const bool few = sizeof(T) == 8 && w >= 2 && m <= 2 * (int64_t)num_sms();
+  const bool few = sizeof(T) == 8 && m <= 2 * (int64_t)num_sms() && (w >= 2 || (!team && n > 128 && m * n > 4096));
   if (few && n <= 8192) {
     switch (w) {
+      case 1: return go(QrShape<2, 4, 0, 1, false>{});
       case 2: return go(QrShape<2, 8, 0, 1, false>{});
       case 4: return go(QrShape<4, 8, 0, 1, false>{});
       case 8: return go(QrShape<8, 8, 0, 1, false>{});

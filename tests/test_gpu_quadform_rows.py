@@ -250,3 +250,21 @@ def test_few_columns(api, m, n, dtype):
     assert rel_l2(g.cpu().numpy(), g_ref) <= TOL[dtype]
     assert torch.equal(f, f2) and torch.equal(g, g2)
     p.close()
+
+
+@pytest.mark.parametrize("m,n", [(1, 129), (16, 129), (16, 256), (17, 240), (64, 250), (150, 193), (304, 256),
+                                 (305, 255)])
+def test_few_rows_of_one_and_two_warps(api, m, n):
+    # FP64 rows of 129 to 256 entries, up to two an SM: a team of two warps, one row a step
+    A, x = W.quadform_inputs(n, m=m, seed=5 * m + n)
+    f_ref, g_ref, gA_ref = O.quadform_grad(A, x, fbar=0.5, want_gA=True)
+    p = api.QuadForm(torch.tensor(A, device="cuda"), arith="native")
+    xt = torch.tensor(x, device="cuda")
+    gA = torch.empty((m, n), dtype=torch.float64, device="cuda")
+    f, g = p.grad(xt, gdata=gA, seed=torch.tensor(0.5, dtype=torch.float64, device="cuda"))
+    fe = p.eval(xt)
+    p.sync()
+    assert rel_scalar(f.item(), f_ref) <= TOL["f64"] and rel_scalar(fe.item(), f_ref) <= TOL["f64"]
+    assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["f64"]
+    assert rel_l2(gA.cpu().numpy(), gA_ref) <= TOL["f64"]
+    p.close()
