@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) qf_pair_rows_kernel(PrArgs a) 
   constexpr int W = NTH / 32, G = 32 / R;  // G lanes hold a row's total
   __shared__ Acc sums[2][W][R];
   __shared__ Acc red[FUSED ? W : 1][16][2];
-  __shared__ double fred[32];
+  __shared__ double fred[FUSED ? 32 : 1];
   __shared__ int go;
   extern __shared__ __align__(16) float4 xs[];  // XS: [KP][NTH]
   const int np2 = a.n >> 1, t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -259,10 +259,14 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) qf_pair_rows_kernel(PrArgs a) 
     if ((done & 7) == 7) acc_renorm(facc);
   }
 
-  // the CTA's f: warp 0's rows, one lane each
-  const double fcta = block_sum(warp == 0 && lane % G == 0 ? acc_to_double(facc) : 0.0, fred);
+  // the CTA's f: warp 0's rows, one lane each, in pairs (an FP64 sum over the CTA is 0.7 us)
+  if (warp == 0) {
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) facc = acc_add(facc, pr_shfl(facc, o));
+  }
+  const double fcta = acc_to_double(facc);  // in thread 0
   if constexpr (!FUSED) {
-    finish_sum<double>(fcta, a.fpart, a.counter, a.f, 0, fred);
+    finish_sum_warp<double>(fcta, a.fpart, a.counter, a.f);
   } else {
     float4* out = a.partials + (int64_t)blockIdx.x * np2;
 #pragma unroll
