@@ -110,12 +110,6 @@ __device__ __forceinline__ void acc2_renorm(Acc2& c) {
   c.l = e;
 }
 
-__device__ __forceinline__ Acc2 acc2_add(Acc2 a, Acc2 b) {
-  F2 s, r;
-  two_sum2(a.s, b.s, s, r);
-  return Acc2{s, f2_add(f2_add(a.l, b.l), r)};
-}
-
 // The two accumulators by themselves, and their sum.
 __device__ __forceinline__ Acc acc2_x(Acc2 a) { return Acc{f2_get(a.s).x, f2_get(a.l).x}; }
 __device__ __forceinline__ Acc acc2_y(Acc2 a) { return Acc{f2_get(a.s).y, f2_get(a.l).y}; }

@@ -343,24 +343,26 @@ static int pr_resident(K kern, int64_t n) {
   return occ;
 }
 
-// Rows of 2050 to 4096 entries run here when there are 4 rows an SM: 700 x 2500 takes 13.1 us
-// here and by the warp-specialized kernel (its start-up and this one's fewer CTAs even
-// out), 4000 x 2500 23.4 against 32.2, 20000 x 4096 115 against 134.  Longer rows: the
-// gradient is the warp-specialized kernel's (10000 x 5000 91 against 87 there, 10000 x 8000
-// 129 against 107), the forward this one's (74.7 against 87, 101 against 105).
+// Rows of 2050 to 4096 entries run here when there are 4 rows an SM, the gradient of more than
+// 3600 entries when there are 8: 610 x 2560 takes 10.6 us here and 13.2 by the warp-specialized
+// kernel, 850 x 3584 13.8 and 14.5, 700 x 3700 15.7 and 13.5, 1216 x 4096 16.0 and 16.6, 2432 x
+// 4096 22.8 and 25.4, 20000 x 4096 115 and 134.  Longer rows: the gradient is the warp-
+// specialized kernel's (10000 x 5000 91 against 87 there, 10000 x 8000 129 against 107), the
+// forward this one's (74.7 against 87, 101 against 105).
 bool qf_pair_rows_supported(int64_t m, int64_t n, bool eval) {
-  return n > 512 && (n <= 2048 || (n <= (eval ? PR_NEVAL : PR_NGRAD) && m >= 4 * (int64_t)num_sms()));
+  if (n <= 2048) return true;
+  return n <= (eval ? PR_NEVAL : PR_NGRAD) && m >= (eval || n <= 3600 ? 4 : 8) * (int64_t)num_sms();
 }
 
-// One wave of resident CTAs at most, and no more than an even share of the steps needs
-// (500 steps on 304 CTAs take two rounds: 250 CTAs do, with fewer partials).
+// One wave of resident CTAs, or one a step.  Fewer, so that all CTAs take as many steps (305
+// steps on 153 CTAs instead of 304), left SMs with half their warps: 610 x 4096 16.7 -> 13.8 us,
+// 610 x 2560 11.9 -> 10.6, 1400 x 1500 11.8 -> 10.8; more partials cost at most 0.3 us.
 int qf_pair_rows_grid(const kg_problem* p) {
   int occ = 0;
   pr_with_kernel<true, true, true>(p->n, [&](auto k) { occ = pr_resident(k, p->n); });
   const int rows = pr_shape(p->n).rows;
   const int64_t steps = (p->m + rows - 1) / rows;
-  const int64_t most = (int64_t)num_sms() * std::max(occ, 1), rounds = (steps + most - 1) / most;
-  return (int)((steps + rounds - 1) / rounds);
+  return (int)std::min(steps, (int64_t)num_sms() * std::max(occ, 1));
 }
 
 // Whether the gradient runs as one cooperative launch.  A grid of at most 64 CTAs leaves
