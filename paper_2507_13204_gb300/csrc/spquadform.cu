@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_row_kernel(SqArgs<T> a) {
       v[u] = p < p1 ? __ldg(a.val + p) : T(0);
     }
 #pragma unroll
-    for (int u = 0; u < SQ_U; ++u) xv[u] = __ldg(a.x + c[u]);  // column 0 for padding (n >= 1)
+    for (int u = 0; u < SQ_U; ++u)  // no value for padding: 0 times an infinite x[0] is no entry's
+      xv[u] = p0 + tl + u * TW < p1 ? __ldg(a.x + c[u]) : T(0);
     T yp = T(0);
 #pragma unroll
     for (int u = 0; u < SQ_U; ++u) yp = fma(v[u], xv[u], yp);
@@ -107,7 +108,8 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_row_kernel(SqArgs<T> a) {
         vv[u] = p < p1 ? __ldg(a.val + p) : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < SQ_U; ++u) yp = fma(vv[u], __ldg(a.x + cc[u]), yp);
+      for (int u = 0; u < SQ_U; ++u)
+        yp = fma(vv[u], pb + tl + u * TW < p1 ? __ldg(a.x + cc[u]) : T(0), yp);
     }
     const T y = team_sum(yp, TW);
     if (act && tl == 0) fl.add(y);
@@ -168,7 +170,8 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_col_kernel(const int* __restri
         v[u] = q < q1 ? __ldg(valT + q) : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < SQ_U; ++u) s = fma(v[u], __ldg(y + r[u]), s);  // row 0 for padding
+      for (int u = 0; u < SQ_U; ++u)  // nor for row 0
+        s = fma(v[u], qb + tl + u * TW < q1 ? __ldg(y + r[u]) : T(0), s);
     }
     s = team_sum(s, TW);
     if (act && tl == 0) {

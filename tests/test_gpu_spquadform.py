@@ -266,3 +266,32 @@ def test_an_x_that_no_entry_reads_has_no_range(api, name, strategy, team):
         with pytest.raises(L.KGError):
             p.sync()
     p.close()
+
+
+@pytest.mark.parametrize("strategy", ["atomic", "transpose"])
+@pytest.mark.parametrize("team", [0, 8])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("name", ["tw2", "tw4", "tw16", "row teams"])
+def test_an_infinite_x_stays_in_its_rows(api, name, dtype, team, strategy):
+    # column 0 is in row 0 only, and x[0] is infinite: y_0 is, and the gradient of row 0's
+    # columns; lanes without an entry, which load x[0] or y_0, must not spread it
+    A = _csr_of_degrees(BLOCKS[name], 3000, seed=3)
+    rng = np.random.default_rng(9)
+    A.val, x = f32_round(rng.uniform(0.5, 1, A.nnz)), f32_round(rng.uniform(0.5, 1, A.n))
+    A.col[A.col == 0] = 1
+    A.col[0] = 0
+    x[0] = np.inf
+    dt = torch.float32 if dtype == "f32" else torch.float64
+    rows = np.repeat(np.arange(A.m), np.diff(A.rowptr))
+    y = np.zeros(A.m)
+    np.add.at(y, rows, A.val * x[A.col])
+    ref = np.zeros(A.n)
+    np.add.at(ref, A.col, 2 * A.val * y[rows])
+    hit = np.isinf(ref)
+    assert hit[0] and hit.sum() < A.n // 2 and not np.isnan(ref).any()
+    p = _problem(api, A, dt, strategy=strategy, arith="native", team=team)
+    g = p.grad(torch.tensor(x, dtype=dt, device="cuda"))[1].cpu().numpy()
+    p.sync()
+    assert np.array_equal(np.isinf(g), hit)
+    assert rel_l2(g[~hit], ref[~hit]) <= TOL[dtype]
+    p.close()
