@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_row_pair_kernel(SqPairArgs a) 
       }
 #pragma unroll
       for (int u = 0; u < SQ_U; ++u) {
-        const double xd = __ldg(a.x + c[u]);  // column 0 for padding (n >= 1): its range does not count
-        bad |= !pair_in_range(xd) && pb + tl + u * TW < p1;
+        const double xd = __ldg(a.x + c[u]);  // column 0 for padding (n >= 1)
+        bad |= !pair_in_range(xd);
         const Pair xp = split_f64(xd);
         acc_fma(ya, v[u].x, v[u].y, xp.h, xp.l);
       }
