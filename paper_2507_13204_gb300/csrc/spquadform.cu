@@ -66,6 +66,22 @@ __device__ __forceinline__ T team_sum(T v, int tw) {
   return v;
 }
 
+// Lanes without an entry gather x[0] (column pass: y of row 0) with a zero value.  0 times an
+// infinite x[0] is no entry's product, so a sum that is not finite is taken again from the
+// entries alone (masks in the main loops cost up to 10 %, long FP64 rows).  The test is on the
+// bits: an FP64 comparison would occupy the FP64 unit.
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+__device__ __forceinline__ bool not_finite(float v) { return (__float_as_int(v) & 0x7f800000) == 0x7f800000; }
+
+// The lane's share of sum_p val[p] x[idx[p]] over [p0, p1), one entry at a time.
+template <typename T, int TW>
+__device__ __forceinline__ T entries_sum(const T* val, const int* idx, const T* x, int p0, int p1) {
+  T s = T(0);
+#pragma unroll 1
+  for (int p = p0 + (threadIdx.x & (TW - 1)); p < p1; p += TW) s = fma(val[p], x[idx[p]], s);
+  return s;
+}
+
 // Entries a lane handles per step: all their loads are issued before any use,
 // so that a lane keeps SQ_U index loads, then SQ_U gathers, in flight.
 constexpr int SQ_U = 4;
@@ -93,8 +109,7 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_row_kernel(SqArgs<T> a) {
       v[u] = p < p1 ? __ldg(a.val + p) : T(0);
     }
 #pragma unroll
-    for (int u = 0; u < SQ_U; ++u)  // no value for padding: 0 times an infinite x[0] is no entry's
-      xv[u] = p0 + tl + u * TW < p1 ? __ldg(a.x + c[u]) : T(0);
+    for (int u = 0; u < SQ_U; ++u) xv[u] = __ldg(a.x + c[u]);  // column 0 for padding (n >= 1)
     T yp = T(0);
 #pragma unroll
     for (int u = 0; u < SQ_U; ++u) yp = fma(v[u], xv[u], yp);
@@ -108,10 +123,10 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_row_kernel(SqArgs<T> a) {
         vv[u] = p < p1 ? __ldg(a.val + p) : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < SQ_U; ++u)
-        yp = fma(vv[u], pb + tl + u * TW < p1 ? __ldg(a.x + cc[u]) : T(0), yp);
+      for (int u = 0; u < SQ_U; ++u) yp = fma(vv[u], __ldg(a.x + cc[u]), yp);
     }
-    const T y = team_sum(yp, TW);
+    T y = team_sum(yp, TW);
+    if (__any_sync(0xffffffffu, not_finite(y))) y = team_sum(entries_sum<T, TW>(a.val, a.col, a.x, p0, p1), TW);
     if (act && tl == 0) fl.add(y);
     if constexpr (MODE == SQ_ROWPASS) {
       if (act && tl == 0) a.y[i] = y;
@@ -170,10 +185,10 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_col_kernel(const int* __restri
         v[u] = q < q1 ? __ldg(valT + q) : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < SQ_U; ++u)  // nor for row 0
-        s = fma(v[u], qb + tl + u * TW < q1 ? __ldg(y + r[u]) : T(0), s);
+      for (int u = 0; u < SQ_U; ++u) s = fma(v[u], __ldg(y + r[u]), s);  // row 0 for padding
     }
     s = team_sum(s, TW);
+    if (__any_sync(0xffffffffu, not_finite(s))) s = team_sum(entries_sum<T, TW>(valT, rowT, y, q0, q1), TW);
     if (act && tl == 0) {
       const T g = fb2 * s;
       gx[j] = accumulate ? gx[j] + g : g;
@@ -241,7 +256,7 @@ __global__ void __launch_bounds__(SQ_THREADS) spq_row_pair_kernel(SqPairArgs a) 
       }
 #pragma unroll
       for (int u = 0; u < SQ_U; ++u) {
-        const double xd = __ldg(a.x + c[u]);  // column 0 for padding (n >= 1)
+        const double xd = __ldg(a.x + c[u]);  // column 0 for padding (n >= 1): its range counts, too
         bad |= !pair_in_range(xd);
         const Pair xp = split_f64(xd);
         acc_fma(ya, v[u].x, v[u].y, xp.h, xp.l);
