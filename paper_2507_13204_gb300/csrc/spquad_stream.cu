@@ -262,11 +262,29 @@ int spq_stream_team(double avg) {
 // entries on 5000 columns 193 -> 209), and so does every gradient w.r.t. the values, whose
 // long rows a team walks entry by entry.  FP64 rows of up to 76 entries run here (gradients
 // 185 -> 175 us, 113 -> 101, 143 -> 134, forwards 122 -> 119, 79 -> 65; 100..200 entries
-// 37.0 -> 39.1, CSC).
+// 37.0 -> 39.1, CSC).  Of more than 20 blocks an SM the row teams keep
+//   - thin blocks, of fewer than 700 entries because TW has just doubled (100000 rows; 350000
+//     rows): the forward in pairs (39 entries a row 27.6 us there, 37.1 here; 21 a row 64 and
+//     90), its row pass from TW = 8 (39 a row 51.7 and 57.3), the native atomic gradient from
+//     TW = 8 (42 a row 54 and 59, 21 a row 107 and 124);
+//   - the forward in pairs of TW = 16, which has no reverse to keep the entries for (60 entries
+//     a row 40.4 and 45.0);
+//   - the native atomic gradient with values of TW = 32 (120 a row 138 and 182).
+// Fewer blocks hide less latency there (20000 rows of 39 15.0 us and 12.9, the forward).
 bool spq_stream_takes(const kg_problem* p, int mode, bool gval) {
-  if (!p->sq_stream) return false;
-  if (gval) return true;
-  return p->dtype == KG_F32 ? mode == SS_ATOMIC && p->sq_stream <= 8 : p->sq_stream <= 16;
+  const int tw = p->sq_stream;
+  if (!tw) return false;
+  if (p->dtype == KG_F32) return gval || (mode == SS_ATOMIC && tw <= 8);
+  const int rb = SS_THREADS / tw;
+  const bool many = (p->m + rb - 1) / rb > 20 * (int64_t)num_sms();
+  const bool thin = many && tw > 1 && (double)p->nnz / (double)p->m * rb < 700.0;
+  if (p->arith == KG_ARITH_PAIR) {
+    if (gval) return true;
+    if (mode == SS_EVAL) return tw <= (many ? 8 : 16) && !thin;
+    return tw <= 16 && !(mode == SS_ROWPASS && tw >= 8 && thin);
+  }
+  if (mode == SS_ATOMIC) return tw <= (gval && !many ? 32 : 16) && !(tw >= 8 && thin);
+  return gval || tw <= 16;
 }
 
 template <int AR, int MODE, typename Go>

@@ -294,3 +294,26 @@ def test_an_infinite_x_stays_in_its_rows(api, name, dtype, team, strategy):
     assert np.array_equal(np.isinf(g), hit)
     assert rel_l2(g[~hit], ref[~hit]) <= TOL[dtype]
     p.close()
+
+
+@pytest.mark.parametrize("deg", [6, 10, 21, 39, 60, 100])
+@pytest.mark.parametrize("kind", ["pair", "native"])
+def test_many_blocks_of_fp64_rows(api, deg, kind):
+    # more than 20 row blocks an SM: some passes of these row lengths go to the row teams
+    A = _csr_of_degrees([deg] * 200000, 5000, seed=deg)
+    x = np.random.default_rng(8).uniform(-1, 1, A.n)
+    f_ref, g_ref, gv_ref = O.spquadform_grad(A.rowptr, A.col, A.val, x, want_gval=True)
+    xt = torch.tensor(x, device="cuda")
+    for strategy in ("atomic", "transpose"):
+        p = _problem(api, A, strategy=strategy, arith=kind)
+        gv = torch.empty(A.nnz, dtype=torch.float64, device="cuda")
+        f, g = p.grad(xt, gdata=gv)
+        f2, g2 = p.grad(xt)
+        fe = p.eval(xt)
+        p.sync()
+        for v in (f, f2, fe):
+            assert rel_scalar(v.item(), f_ref) <= TOL["f64"]
+        for v in (g, g2):
+            assert rel_l2(v.cpu().numpy(), g_ref) <= TOL["f64"]
+        assert rel_l2(gv.cpu().numpy(), gv_ref) <= TOL["f64"]
+        p.close()
