@@ -385,6 +385,53 @@ __device__ __forceinline__ void elem_native_hvp(const int4 c, const T* __restric
 
 // The Hessian-vector arithmetic of one element in float pairs, from its G_e
 // and the gathered U (point) and V (direction): hc[k] = (G_e^T (wd g + w gd))_k.
+// Twice: one value at a time, in 64 registers, for the kernels whose scatter waits on
+// memory and that gain more from a fourth CTA an SM (tile sums 128 us at 80^3, 133 packed;
+// one atomic a contribution 127 and 129.5), and two at a time, in 80, for the warp combine
+// (125.7; 129.5 one at a time).
+__device__ __forceinline__ void elem_pair_hvp_scalar(const Pair (&G)[12], const Pair (&U)[4],
+                                                   const Pair (&V)[4], Pair fb2, Pair (&hc)[4]) {
+  Pair g[3], gd[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    Acc a = acc_prod(G[4 * r].h, G[4 * r].l, U[0].h, U[0].l);
+    Acc b = acc_prod(G[4 * r].h, G[4 * r].l, V[0].h, V[0].l);
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+      acc_fma(a, G[4 * r + k].h, G[4 * r + k].l, U[k].h, U[k].l);
+      acc_fma(b, G[4 * r + k].h, G[4 * r + k].l, V[k].h, V[k].l);
+    }
+    g[r] = acc_pair(a);
+    gd[r] = acc_pair(b);
+  }
+  Acc sa = acc_prod(g[0].h, g[0].l, g[0].h, g[0].l);
+  Acc sda = acc_prod(g[0].h, g[0].l, gd[0].h, gd[0].l);
+#pragma unroll
+  for (int r = 1; r < 3; ++r) {
+    acc_fma(sa, g[r].h, g[r].l, g[r].h, g[r].l);
+    acc_fma(sda, g[r].h, g[r].l, gd[r].h, gd[r].l);
+  }
+  const Pair s = acc_pair(sa);
+  Pair sd = acc_pair(sda);
+  sd.h *= 2.0f;  // exact
+  sd.l *= 2.0f;
+  const Pair rt = pair_recip(pair_add(Pair{1.0f, 0.0f}, s));
+  const Pair w = pair_mul(fb2, rt);
+  Pair wd = pair_mul(pair_mul(w, sd), rt);
+  wd.h = -wd.h;
+  wd.l = -wd.l;
+  Pair h[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) h[r] = pair_add(pair_mul(wd, g[r]), pair_mul(w, gd[r]));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    Acc a = acc_prod(G[k].h, G[k].l, h[0].h, h[0].l);
+#pragma unroll
+    for (int r = 1; r < 3; ++r) acc_fma(a, G[4 * r + k].h, G[4 * r + k].l, h[r].h, h[r].l);
+    hc[k] = acc_pair(a);
+  }
+}
+
 __device__ __forceinline__ void elem_pair_hvp_core(const Pair2 (&G)[6], const Pair2 (&U)[2],
                                                    const Pair2 (&V)[2], Pair fb2, Pair (&hc)[4]) {
   Pair g[3], gd[3];
@@ -426,18 +473,39 @@ __device__ __forceinline__ void elem_pair_hvp_core(const Pair2 (&G)[6], const Pa
   }
 }
 
-// The same in float-pair arithmetic (FP64 data); fb2 = 2 fbar as a pair.
-template <typename Sink, bool PREP = false, bool USPLIT = false>
+// The same in float-pair arithmetic (FP64 data); fb2 = 2 fbar as a pair.  PACKED: two values
+// at a time.
+template <bool PACKED, typename Sink, bool PREP = false, bool USPLIT = false>
 __device__ __forceinline__ void elem_pair_hvp(const int4 c, const double* __restrict__ Gs,
                                               const double* __restrict__ u,
                                               const double* __restrict__ v, Pair fb2,
                                               const Sink& gu, bool& bad) {
-  Pair2 G[6], U[2], V[2];
-  elem_pair_load_G<PREP>(Gs, G);
-  elem_pair_load_u<USPLIT>(c, u, U, bad);
-  elem_pair_load_u<USPLIT>(c, v, V, bad);
   Pair hc[4];
-  elem_pair_hvp_core(G, U, V, fb2, hc);
+  if constexpr (PACKED) {
+    Pair2 G[6], U[2], V[2];
+    elem_pair_load_G<PREP>(Gs, G);
+    elem_pair_load_u<USPLIT>(c, u, U, bad);
+    elem_pair_load_u<USPLIT>(c, v, V, bad);
+    elem_pair_hvp_core(G, U, V, fb2, hc);
+  } else {  // the prepared data only
+    static_assert(PREP && USPLIT, "the tile and the direct kernels run on prepared data");
+    Pair G[12], U[4], V[4];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const float4 q = reinterpret_cast<const float4*>(Gs)[i];
+      G[2 * i] = Pair{q.x, q.z};
+      G[2 * i + 1] = Pair{q.y, q.w};
+    }
+    const int idx[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 qu = __ldg(reinterpret_cast<const float2*>(u) + idx[k]);
+      const float2 qv = __ldg(reinterpret_cast<const float2*>(v) + idx[k]);
+      U[k] = Pair{qu.x, qu.y};
+      V[k] = Pair{qv.x, qv.y};
+    }
+    elem_pair_hvp_scalar(G, U, V, fb2, hc);
+  }
   sink_pair(gu, 0, c.x, hc[0]);
   sink_pair(gu, 1, c.y, hc[1]);
   sink_pair(gu, 2, c.z, hc[2]);

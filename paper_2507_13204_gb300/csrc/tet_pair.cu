@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(TS_THREADS) tet_staged_kernel(TsArgs<T> a) {
         auto run = [&](const auto& sink) {
           if constexpr (MODE == TS_HVP) {
             if constexpr (PAIR)
-              elem_pair_hvp<std::decay_t<decltype(sink)>, PREP, true>(
+              elem_pair_hvp<true, std::decay_t<decltype(sink)>, PREP, true>(
                   c, reinterpret_cast<const double*>(Gs), reinterpret_cast<const double*>(a.u),
                   reinterpret_cast<const double*>(a.v), fb2, sink, bad);
             else
@@ -311,7 +311,7 @@ __global__ void pair_split_vec_kernel(const double* __restrict__ u, const double
 // trip count, so the warp combine can run).  GRAD and HVP read u (and v) as
 // float pairs split once per call.
 template <int MODE, bool WARPC>
-__global__ void __launch_bounds__(TS_THREADS, MODE == TS_HVP ? 3 : 4) tet_direct_pair_kernel(TsArgs<double> a) {
+__global__ void __launch_bounds__(TS_THREADS, MODE == TS_HVP && WARPC ? 3 : 4) tet_direct_pair_kernel(TsArgs<double> a) {
   __shared__ float4 tab[kLogTableSize];
   __shared__ double red[2 * TS_WARPS];
   constexpr bool REV = MODE == TS_GRAD || MODE == TS_HVP;
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(TS_THREADS, MODE == TS_HVP ? 3 : 4) tet_direct
     if (act) {
       auto run = [&](const auto& sink) {
         if constexpr (MODE == TS_HVP)
-          elem_pair_hvp<std::decay_t<decltype(sink)>, true, true>(
+          elem_pair_hvp<WARPC, std::decay_t<decltype(sink)>, true, true>(
               c, Gp + e * 12, u, reinterpret_cast<const double*>(a.v), fb2, sink, bad);
         else
           elem_pair<MODE, std::decay_t<decltype(sink)>, true, USPLIT>(

@@ -164,7 +164,7 @@ struct TileArgs {
 // in ascending order and issues one global reduction -- or, STORE (the
 // reproducible CSR strategy), writes the sum to the tile's partials instead.
 template <int MODE, bool STORE>
-__global__ void __launch_bounds__(TL_THREADS, MODE == TS_HVP ? 3 : 4) tet_tile_pair_kernel(TileArgs a) {
+__global__ void __launch_bounds__(TL_THREADS, 4) tet_tile_pair_kernel(TileArgs a) {
   __shared__ float4 tab[kLogTableSize];
   __shared__ __align__(16) float2 c_s[TL_THREADS / 32][TL_C];  // float4 stores
   __shared__ double red[2 * (TL_THREADS / 32)];
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(TL_THREADS, MODE == TS_HVP ? 3 : 4) tet_tile_p
         elem_pair<TS_GRAD, CollectSink<double>, true, true>(c, a.G + e * 12, a.u, fb2, tab, a.K, lsum,
                                                              CollectSink<double>{wv, wp}, nullptr, bad);
       else
-        elem_pair_hvp<CollectSink<double>, true, true>(c, a.G + e * 12, a.u, a.v, fb2,
+        elem_pair_hvp<false, CollectSink<double>, true, true>(c, a.G + e * 12, a.u, a.v, fb2,
                                                        CollectSink<double>{wv, wp}, bad);
       float4* cs = reinterpret_cast<float4*>(cw + 4 * lane);
       cs[0] = make_float4(wp[0].h, wp[0].l, wp[1].h, wp[1].l);
