@@ -1102,8 +1102,11 @@ kg_status time_plan(kg_batch* b, const std::vector<int>& ids, const Tuning& tu, 
 // persistent grid (or on all of them); the largest tile within 3% of the
 // fastest wins.  A smaller sample favours small tiles for want of parallelism
 // that the whole batch has (make_plan cuts them to a CTA's share anyway): there
-// the largest within 10% wins (on 128 dense and 16 tet instances the fastest
-// ones made tiles of 16 rows and 187 us, these 171, both with tiles of two rows a step).  Choices are cached by GPU name, kind, dtype, arithmetic and bucket.
+// the largest within 10% wins, in float pairs and FP32 (128 dense and 16 tet
+// instances: pairs 157 to 159 us over six tunings, 156 to 166 within 3%; FP32
+// 81 and 82).  Native FP64 is bound by its FP64 unit, whose work larger tiles
+// spread less evenly: 3% there as well (419 us, 459 within 10%).  Choices are
+// cached by GPU name, kind, dtype, arithmetic and bucket.
 kg_status autotune(kg_batch* b, cudaStream_t s) {
   std::map<std::pair<int, int>, std::vector<int>> groups;  // (kind, bucket) -> instance ids
   for (int i = 0; i < (int)b->probs.size(); ++i) {
@@ -1114,8 +1117,8 @@ kg_status autotune(kg_batch* b, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   std::map<std::string, int> cache = cache_read();
   bool dirty = false;
-  // "k5": dense tiles take four rows a step
-  const std::string prefix = b->gpu + "|k5|" + (b->dtype == KG_F64 ? "f64" : "f32") + "|" +
+  // "k6": dense tiles take four rows a step, native FP64 the largest within 3%
+  const std::string prefix = b->gpu + "|k6|" + (b->dtype == KG_F64 ? "f64" : "f32") + "|" +
                              (b->pair ? "pair" : "native") + "|";
   const std::vector<int> dense_cands{4, 8, 16, 32, 64, 128, 256}, tet_cands{1024, 2048, 4096, 8192, 16384};
   std::map<std::pair<int, int>, std::vector<int>> sample;
@@ -1162,7 +1165,8 @@ kg_status autotune(kg_batch* b, cudaStream_t s) {
     if (rc != KG_OK) break;
     int64_t items = 0;
     for (int i : ids) items += (b->probs[i]->m + cands.back() - 1) / cands.back();
-    const float slack = items >= 4 * (int64_t)b->grid ? 1.03f : 1.10f;
+    const bool fp64 = b->dtype == KG_F64 && !b->pair;
+    const float slack = fp64 || items >= 4 * (int64_t)b->grid ? 1.03f : 1.10f;
     const float least = *std::min_element(ms.begin(), ms.end());
     int best = cands[0];
     for (size_t i = 0; i < cands.size(); ++i)
