@@ -576,9 +576,14 @@ static SqPairArgs sq_pair_args(kg_problem* p, const void* x, void* f, const void
   return a;
 }
 
+// Which of the two kernels a row pass runs.
+static const char* row_name(const kg_problem* p, int mode, bool gval, const char* teams, const char* blocks) {
+  return spq_stream_takes(p, mode, gval) ? blocks : teams;
+}
+
 static kg_status spq_pair_eval(kg_problem* p, const void* x, void* f, cudaStream_t s) {
   SqPairArgs a = sq_pair_args(p, x, f, nullptr);
-  prof_begin(s, "spq_row_pair_kernel<eval>");
+  prof_begin(s, row_name(p, SQ_EVAL, false, "spq_row_pair_kernel<eval>", "spq_stream_kernel<eval>"));
   cudaError_t e = launch_row_pair<SQ_EVAL>(p, a, s);
   prof_end(s);
   count_launch();
@@ -598,7 +603,7 @@ static kg_status spq_pair_grad(kg_problem* p, const void* x, void* f, void* gx, 
       count_launch();
     }
     a.gx = static_cast<double*>(gx);
-    prof_begin(s, "spq_row_pair_kernel<atomic>");
+    prof_begin(s, row_name(p, SQ_ATOMIC, gval != nullptr, "spq_row_pair_kernel<atomic>", "spq_stream_kernel<atomic>"));
     e = launch_row_pair<SQ_ATOMIC>(p, a, s);
     prof_end(s);
     count_launch();
@@ -632,7 +637,7 @@ static SqArgs<T> sq_args(kg_problem* p, const void* x, void* f, const void* seed
 template <typename T>
 static kg_status spq_eval_t(kg_problem* p, const void* x, void* f, cudaStream_t s) {
   SqArgs<T> a = sq_args<T>(p, x, f, nullptr);
-  prof_begin(s, "spq_row_kernel<eval>");
+  prof_begin(s, row_name(p, SQ_EVAL, false, "spq_row_kernel<eval>", "spq_stream_kernel<eval>"));
   cudaError_t e = launch_row<T, SQ_EVAL>(p, a, s);
   prof_end(s);
   count_launch();
@@ -653,7 +658,7 @@ static kg_status spq_grad_t(kg_problem* p, const void* x, void* f, void* gx, voi
       count_launch();
     }
     a.gx = static_cast<T*>(gx);
-    prof_begin(s, "spq_row_kernel<atomic>");
+    prof_begin(s, row_name(p, SQ_ATOMIC, gval != nullptr, "spq_row_kernel<atomic>", "spq_stream_kernel<atomic>"));
     e = launch_row<T, SQ_ATOMIC>(p, a, s);
     prof_end(s);
     count_launch();
