@@ -824,9 +824,9 @@ constexpr int B_SUM_TILES = 16;
 // No tile is larger than a CTA's share of the batch / B_SHARE, so that a batch of few
 // large instances still fills the grid: the autotuner's tiles (up to 256 rows, right for
 // batches of thousands) gave 128 dense and 16 tet instances two items a CTA.  Measured on
-// that batch, 630 MB, shares of 2, 3, 4 and 6: float pairs 157, 156, 159 and 163 us, FP32
-// 80, 82, 85 and 93, native FP64 497, 458, 427 and 422; 32 + 4 and 16 + 2 instances do not
-// differ (their tiles are at the 4 steps make_plan leaves).
+// that batch, 630 MB, shares of 2, 3, 4 and 6 (medians of six tunings): float pairs 160, 156,
+// 159 and 164 us, FP32 79, 81, 83 and 92, native FP64 462, 419, 426 and 421; 32 + 4 instances
+// 66, 68, 69 and 69, 16 + 2 do not differ (their tiles are at the 4 steps make_plan leaves).
 constexpr int B_SHARE = 3;
 
 // prep[i]: the float-pair copy of problem i's A (dense) or G (tet) that the

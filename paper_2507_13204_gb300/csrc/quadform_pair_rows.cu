@@ -12,8 +12,8 @@
 // memory.  xbar accumulates in registers.  Steps go round-robin over the grid.
 //
 // Measured (value and gradient, device time, against a row at a time): 2000 x 1500 21.4 ->
-// 12.8 us, 40000 x 1024 236 -> 67, 40000 x 2048 294 -> 119 (5.5 TB/s), 20000 x 2500
-// 141 -> 80; the forward 206 -> 50, 238 -> 99 (6.6 TB/s), 135 -> 64.  The rest of the
+// 11.1 us, 40000 x 1024 236 -> 68, 40000 x 2048 294 -> 121 (5.4 TB/s), 20000 x 2500
+// 141 -> 81; the forward 206 -> 51, 238 -> 100 (6.5 TB/s), 135 -> 66.  The rest of the
 // gradient is issue: 24 packed and scalar FP32 operations an entry.
 //
 // The CTAs' partials are summed in a fixed order: behind a bounded grid barrier in the

@@ -24,9 +24,9 @@
 // or by qf_reduce_kernel: bitwise reproducible.
 //
 // Measured (value and gradient, one call, against one row a team and step with a butterfly
-// per row): FP64 150001 x 255 857 -> 160 us (its DFMAs take 122), 20000 x 2051 963 -> 250
-// (131), 10000 x 5001 484 -> 243 (160), 10000 x 9999 478 -> 475 (320); FP32 400000 x 100
-// 121 -> 36.6 us (its bytes take 23.6), 40000 x 1024 96.8 -> 31 (24), 20000 x 4095
+// per row): FP64 150001 x 255 857 -> 158 us (its DFMAs take 122), 20000 x 2051 963 -> 248
+// (131), 10000 x 5001 484 -> 242 (160), 10000 x 9999 478 -> 478 (320); FP32 400000 x 100
+// 121 -> 35.9 us (its bytes take 23.6), 40000 x 1024 96.8 -> 31 (24), 20000 x 4095
 // 157 -> 72 (48).
 #include <cuda_runtime.h>
 
