@@ -69,6 +69,7 @@ __device__ __forceinline__ void finish_sum_warp(double partial, double* fpart, u
   }
   arrived = __shfl_sync(0xffffffffu, arrived, 0);
   if (arrived != gridDim.x - 1) return;
+  __syncwarp();  // orders the lanes behind thread 0's arrival
   __threadfence();
   double s = 0.0;
   for (int i = threadIdx.x; i < (int)gridDim.x; i += 8 * 32) {
