@@ -21,7 +21,6 @@ only: the reverse pass needs nothing but y, which the fused kernel rebuilds).
 from __future__ import annotations
 
 import os
-from contextlib import nullcontext
 
 import torch
 
@@ -91,11 +90,12 @@ def _autograd_watched() -> bool:
             or torch._C._autograd._top_saved_tensors_default_hooks(False) is not None)
 
 
-def _range():
-    """The profiler range of a step that does not go through KGTetEnergy."""
-    if torch._C._autograd._profiler_enabled():
-        return torch.autograd.profiler.record_function("KGTetEnergy")
-    return nullcontext()
+def _value_and_grad(problem: TetEnergy, u, f, g, tape: bool):
+    if tape:
+        problem.eval_tape(u, f)
+        problem.grad_from_tape(gx=g)
+    else:
+        problem.grad(u, gx=g, f=f)
 
 
 def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: int,
@@ -129,6 +129,7 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
     direct = (type(u) is torch.Tensor and u.dim() == 1 and u.is_contiguous() and torch.is_grad_enabled()
               and (policy != "tape" or tape) and isinstance(eta, (int, float)) and not isinstance(eta, bool)
               and not _autograd_watched())
+    profiled = torch._C._autograd._profiler_enabled()
     f = g = None
     for t in range(start, steps):
         if direct:
@@ -136,12 +137,11 @@ def gradient_descent(problem: TetEnergy, u0: torch.Tensor, eta: float, steps: in
                 f = torch.empty((), dtype=u.dtype, device=u.device)
             if g is None:
                 g = torch.empty_like(u)
-            with _range():
-                if tape:
-                    problem.eval_tape(u, f)
-                    problem.grad_from_tape(gx=g)
-                else:
-                    problem.grad(u, gx=g, f=f)
+            if profiled:
+                with torch.autograd.profiler.record_function("KGTetEnergy"):
+                    _value_and_grad(problem, u, f, g, tape)
+            else:
+                _value_and_grad(problem, u, f, g, tape)
             u.sub_(g, alpha=eta)
         else:
             ut = u.requires_grad_(True)
