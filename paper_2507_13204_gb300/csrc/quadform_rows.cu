@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(S::THREADS, S::THREADS == 512 ? 1 : sizeof(T) 
   const int64_t first = blockIdx.x + (int64_t)team * gridDim.x, all = (int64_t)gridDim.x * NT;
   const unsigned step = all < groups ? (unsigned)all : groups;
   int par = 0;
-  // each team by itself: one without a group in the last round leaves the FP64 unit to the others
+  // each team by itself: one that runs out of groups leaves the FP64 unit to the others
   for (unsigned grp = first < groups ? (unsigned)first : groups; grp < groups; grp += step, par ^= 1) {
     const int64_t r0 = (int64_t)grp * R;
     const int rows = (int)(a.m - r0 < R ? a.m - r0 : R);
